@@ -24,7 +24,7 @@ namespace {
 
 struct BatchArgs {
     const int4 *cta_team;     // per CTA: team, rank in team, team size, class
-    unsigned *team_bar;       // 2 per team: arrivals, generation
+    unsigned long long *team_bar;   // kBarWords per team
     int *team_q;              // per team: the queue slot it is working on
     int *cls_next;            // per class: next queue slot
     const int *cls_begin;     // per class: queue range in `order`
@@ -38,9 +38,10 @@ struct BatchArgs {
 template <int ALGO, int MODE>
 __global__ void __launch_bounds__(kBlock, min_blocks<MODE>()) batch_kernel(BatchArgs b) {
     const int4 ct = b.cta_team[blockIdx.x];
-    const Team t{ct.y, ct.z, b.team_bar + 2 * ct.x};
+    const Team t{ct.y, ct.z, b.team_bar + (int64_t)kBarWords * ct.x};
     const int cls = ct.w;
     uint32_t ring_used;
+    team_begin();
     fixpoint_prologue<ALGO, MODE>(ring_used);
     for (;;) {
         if (t.rank == 0 && threadIdx.x == 0) b.team_q[ct.x] = b.cls_begin[cls] + atomicAdd(&b.cls_next[cls], 1);
@@ -289,7 +290,7 @@ fg_status batch_launch(const fg_query *qs, int32_t nq, const fg_batch_options *o
         int teams = 0;
         for (int t : kp.class_teams) teams += t;
         const int nc = (int)kp.class_size.size();
-        zero_bytes += Workspace::need(2 * teams, 4) + Workspace::need(teams, 4) + Workspace::need(nc, 4);
+        zero_bytes += Workspace::need((int64_t)kBarWords * teams, 8) + Workspace::need(teams, 4) + Workspace::need(nc, 4);
         table_bytes += Workspace::need(kp.ctas, sizeof(int4)) + 2 * Workspace::need(nc, 4);
     }
     job.staged.assign(nq, false);
@@ -366,7 +367,7 @@ fg_status batch_launch(const fg_query *qs, int32_t nq, const fg_batch_options *o
         int teams = 0;
         for (int t : kp.class_teams) teams += t;
         BatchArgs a;
-        a.team_bar = zw.take<unsigned>(2 * teams);
+        a.team_bar = zw.take<unsigned long long>((int64_t)kBarWords * teams);
         a.team_q = zw.take<int>(teams);
         a.cls_next = zw.take<int>(nc);
         int4 *d_ct = tw.take<int4>(kp.ctas);

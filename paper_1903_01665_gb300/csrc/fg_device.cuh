@@ -314,7 +314,7 @@ struct BucketOp : AsyncOp<kSSSP> {
                 if ((int)lane_id() == leader) base = atomicAdd(far_size, __popc(am));
                 base = __shfl_sync(am, base, leader) + __popc(am & lanemask_lt());
                 if (base < far_cap) far[base] = v;
-                else atomicOr(&ctrl->status, kStWorklist);
+                else raise_error(ctrl, kStWorklist);
             }
         }
         return false;
@@ -421,7 +421,7 @@ __device__ __forceinline__ void warp_flush(WarpBuf *b, int cnt, int32_t *list, i
     for (int i = (int)lane_id(); i < cnt; i += 32) {
         int pos = base + i;
         if (pos < cap) list[pos] = b->item[i];
-        else atomicOr(&c->status, kStWorklist);
+        else raise_error(c, kStWorklist);
     }
     __syncwarp();
 }
@@ -477,7 +477,7 @@ struct ClassPush {
             if (base + nck <= cap_high) {
                 for (int k = 0; k < nck; k++) high[base + k] = make_int2(v, (int32_t)(b + (uint32_t)k * kChunk));
             } else {
-                atomicOr(&c->status, kStWorklist);
+                raise_error(c, kStWorklist);
             }
         }
     }
@@ -532,7 +532,7 @@ struct LbPush {
                     list[pos] = buf->item[i];
                     off[pos] = run;
                 } else {
-                    atomicOr(&c->status, kStWorklist);
+                    raise_error(c, kStWorklist);
                 }
             }
             run += deg[k];
@@ -1450,7 +1450,7 @@ __device__ __forceinline__ bool warp_stream(WarpRing<W> &R, uint64_t pol, uint32
             const uint32_t gj = base + (uint32_t)j;
             ring_wait(&R.full[gj % kWStages], (gj / kWStages) & 1u, timeout_ns);
         }
-        atomicOr(&c->status, kStTimeout);
+        raise_error(c, kStTimeout);
     }
     __syncwarp();
     used = base + (uint32_t)(ok ? count : issued);
@@ -1791,8 +1791,8 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
     int n_barriers = 0;
     bool done = false;
     // every grid barrier of the query; CTA 0 optionally timestamps each
-    auto sync_ = [&]() -> bool {
-        bool r = team_sync(t, c, p.timeout_ns);
+    auto sync_ = [&](int add = 0) -> bool {
+        bool r = team_sync(t, c, p.timeout_ns, add);
         if (tid == 0) {
             if (p.trace && n_barriers < p.trace_cap) p.trace[n_barriers] = global_ns();
             n_barriers++;
@@ -1800,6 +1800,7 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
         return r;
     };
 
+    if (threadIdx.x == 0) bar_state().err = 0;   // of this query
     // the source in internal ids (a renumbered graph takes original ones)
     const int32_t source = (ALGO != kCC && p.new_of) ? __ldg(p.new_of + p.source) : p.source;
     // ---- init: values, stamps, initial worklist (a2)
@@ -1850,8 +1851,8 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
     bool ok = sync_();
 
     if (SYNC && ok) {
-        int pass_ctr = 0;
-        int64_t ch_before = 0;   // changes of the round before the previous one (the same in every thread)
+        int64_t ch_prev = 0;     // changes of the previous round, from its barrier (the same in every thread)
+        int64_t ch_before = 0;   // changes of the round before it
         constexpr bool kW = (ALGO == kSSSP);   // the edge rings carry weights for SSSP only
         // edge-sync: a round is sparse if the previous one accepted fewer
         // candidates than n / 2^FG_SPARSE_SHIFT (round 1: only the source is
@@ -1863,19 +1864,17 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
         constexpr int kPullShift = ALGO == kBFS ? FG_PULL_SHIFT_BFS : (ALGO == kCC ? FG_PULL_SHIFT_CC : FG_PULL_SHIFT_SSSP);
         auto pull_round = [&](int r) -> bool {
             if (r == 1) return ALGO == kCC;
-            const int64_t ch = __ldcg(&c->changed[(r - 1) % 3]);
-            return kPullShift >= 0 ? (ch << kPullShift) > (int64_t)n : (ch >> -kPullShift) > (int64_t)n;
+            return kPullShift >= 0 ? (ch_prev << kPullShift) > (int64_t)n : (ch_prev >> -kPullShift) > (int64_t)n;
         };
         auto sparse_round = [&](int r) -> bool {
             if (r == 1) return ALGO != kCC;
-            return ((int64_t)__ldcg(&c->changed[(r - 1) % 3]) << FG_SPARSE_SHIFT) < (int64_t)n;
+            return (ch_prev << FG_SPARSE_SHIFT) < (int64_t)n;
         };
         for (int r = 1;; r++) {
             if (r > p.max_rounds) {
                 if (tid == 0) atomicOr(&c->status, kStRoundCap);
                 break;
             }
-            if (tid == 0) c->changed[(r + 1) % 3] = 0;
             rounds = r;
             const bool pull = (MODE == kPull) && pull_round(r);
             if (pull && tid == 0) c->pull_rounds++;
@@ -1899,7 +1898,6 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
                 int32_t *next = (r & 1) ? p.B : p.A;
                 const int32_t *scur = (r & 1) ? p.S1 : p.S0;
                 int32_t *snext = (r & 1) ? p.S0 : p.S1;
-                const int64_t ch_prev = r == 1 ? 0 : (int64_t)__ldcg(&c->changed[(r - 1) % 3]);
                 // a growing frontier reaches many vertices for the first time:
                 // most candidates then pass the first filter (R-MAT 22 SSSP round
                 // 3: 15.7 M of 20.8 M), and the running minimum saves their MINs
@@ -1926,11 +1924,10 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
                     if (!stream_all_edges<kW>(t, ring_used, g, op, a, c, p.timeout_ns)) break;
                 }
             }
-            int ch = block_sum(a.changed);
+            if (!sync_(a.changed)) break;
             a.changed = 0;
-            if (threadIdx.x == 0 && ch) atomicAdd(&c->changed[r % 3], ch);
-            if (!sync_()) break;
-            if (__ldcg(&c->changed[r % 3]) == 0) {
+            ch_prev = team_total();
+            if (ch_prev == 0) {
                 done = true;
                 if (tid == 0) c->result_in_b = (ALGO != kBFS) && (r & 1);
                 if (ALGO == kSSSP) {
@@ -1958,9 +1955,6 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
                 int32_t *snext = (r & 1) ? p.S0 : p.S1;
                 bool jok = true;
                 for (int pass = 0; pass < 16; pass++) {
-                    int slot = pass_ctr % 3;
-                    if (tid == 0) c->jchanged[(pass_ctr + 1) % 3] = 0;
-                    pass_ctr++;
                     int jc = 0;   // chains not yet at their root
                     for (int64_t v = tid; v < n; v += nth) {
                         const int32_t l0 = ldcg(next + v);
@@ -1982,11 +1976,9 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
                             stcg(snext + v, r + 1);
                         }
                     }
-                    jc = block_sum(jc);
-                    if (threadIdx.x == 0 && jc) atomicAdd(&c->jchanged[slot], jc);
-                    if (!sync_()) { jok = false; break; }
+                    if (!sync_(jc)) { jok = false; break; }
                     if (tid == 0) c->jump_passes++;
-                    if (__ldcg(&c->jchanged[slot]) == 0) break;
+                    if (team_total() == 0) break;
                 }
                 if (!jok) break;
             }
@@ -2088,7 +2080,7 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
                             if ((int)lane_id() == leader) base = atomicAdd(&c->far_size[(epoch + 1) % 3], __popc(am));
                             base = __shfl_sync(am, base, leader) + __popc(am & lanemask_lt());
                             if (base < p.far_cap) far_out[base] = v;
-                            else atomicOr(&c->status, kStWorklist);
+                            else raise_error(c, kStWorklist);
                         }
                     }
                     __syncwarp();

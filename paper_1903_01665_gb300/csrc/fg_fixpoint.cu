@@ -12,8 +12,9 @@ namespace {
 
 template <int ALGO, int MODE>
 __global__ void __launch_bounds__(kBlock, min_blocks<MODE>()) fixpoint_kernel(Params p) {
-    const Team t{(int)blockIdx.x, (int)gridDim.x, &p.ctrl->bar_count};
+    const Team t{(int)blockIdx.x, (int)gridDim.x, p.ctrl->bar};
     uint32_t ring_used;
+    team_begin();
     fixpoint_prologue<ALGO, MODE>(ring_used);
     query_body<ALGO, MODE>(p, t, ring_used);
 }

@@ -378,8 +378,9 @@ __device__ __forceinline__ void multi_body(const Params &p, const Team &t) {
     Acc a;
     int rounds = 0, n_barriers = 0;
     bool done = false;
-    auto sync_ = [&]() -> bool {
-        const bool ok = team_sync(t, c, p.timeout_ns);
+    if (threadIdx.x == 0) bar_state().err = 0;   // of this query
+    auto sync_ = [&](int add = 0) -> bool {
+        const bool ok = team_sync(t, c, p.timeout_ns, add);
         n_barriers++;
         return ok;
     };
@@ -417,18 +418,13 @@ __device__ __forceinline__ void multi_body(const Params &p, const Team &t) {
             if (tid == 0) atomicOr(&c->status, kStRoundCap);
             break;
         }
-        if (tid == 0) c->changed[(r + 1) % 3] = 0;
         rounds = r;
         ms_round<ALGO>(t, g, D, stamp, r, nf, a);
-        const int ch = block_sum(a.changed);
+        if (a.overflow) atomicOr(&c->status, kStOverflow);
+        a.overflow = 0;
+        if (!sync_(a.changed)) break;
         a.changed = 0;
-        const int of = block_sum(a.overflow);
-        if (threadIdx.x == 0) {
-            if (ch) atomicAdd(&c->changed[r % 3], ch);
-            if (of) atomicOr(&c->status, kStOverflow);
-        }
-        if (!sync_()) break;
-        if (__ldcg(&c->changed[r % 3]) != 0) continue;
+        if (team_total() != 0) continue;
         const int32_t T = ms_T;
         if (T >= kInf) {   // no width: nothing is ever far
             done = true;
@@ -752,8 +748,9 @@ __device__ __forceinline__ void multi_bfs_body(const Params &p, const Team &t) {
     Acc a;
     int rounds = 0, n_barriers = 0;
     bool done = false;
-    auto sync_ = [&]() -> bool {
-        const bool ok = team_sync(t, c, p.timeout_ns);
+    if (threadIdx.x == 0) bar_state().err = 0;   // of this query
+    auto sync_ = [&](int add = 0) -> bool {
+        const bool ok = team_sync(t, c, p.timeout_ns, add);
         n_barriers++;
         return ok;
     };
@@ -782,18 +779,15 @@ __device__ __forceinline__ void multi_bfs_body(const Params &p, const Team &t) {
             if (tid == 0) atomicOr(&c->status, kStRoundCap);
             break;
         }
-        if (tid == 0) c->changed[(r + 1) % 3] = 0;
         rounds = r;
         const uint8_t *cur = F + (r % 3) * np;
         uint8_t *nxt = F + ((r + 1) % 3) * np;
         int4 *clr = reinterpret_cast<int4 *>(F + ((r + 2) % 3) * np);   // the previous round's frontier
         for (int64_t i = tid; i < np / 16; i += nth) clr[i] = make_int4(0, 0, 0, 0);
         msb_round(t, g, p, vis, cur, nxt, r, a);
-        const int ch = block_sum(a.changed);
+        if (!sync_(a.changed)) break;
         a.changed = 0;
-        if (threadIdx.x == 0 && ch) atomicAdd(&c->changed[r % 3], ch);
-        if (!sync_()) break;
-        if (__ldcg(&c->changed[r % 3]) == 0) {
+        if (team_total() == 0) {
             done = true;
             break;
         }

@@ -25,7 +25,7 @@ namespace fg {
 namespace {
 
 constexpr int32_t kNaMaxN = FG_NOALLOC_MAX_VERTICES;
-constexpr size_t kNaCtrlBytes = 256;
+constexpr size_t kNaCtrlBytes = 1024;
 constexpr size_t kNaArrayBytes = (size_t)kNaMaxN * sizeof(int32_t);
 // control block, then buffer B, then stamp arrays S0 and S1 (fixed offsets)
 constexpr size_t kNaScratchBytes = kNaCtrlBytes + 3 * kNaArrayBytes;
@@ -70,6 +70,8 @@ __global__ void __launch_bounds__(kBlock) noalloc_sssp_kernel(NaParams p) {
     int32_t *B = reinterpret_cast<int32_t *>(p.scratch + kNaCtrlBytes);
     int32_t *S0 = reinterpret_cast<int32_t *>(p.scratch + kNaCtrlBytes + kNaArrayBytes);
     int32_t *S1 = reinterpret_cast<int32_t *>(p.scratch + kNaCtrlBytes + 2 * kNaArrayBytes);
+    const Team team{(int)blockIdx.x, (int)gridDim.x, c->bar};
+    team_begin();
     const int64_t tid = blockIdx.x * (int64_t)kBlock + threadIdx.x;
     const int64_t nth = (int64_t)gridDim.x * kBlock;
     const int32_t n = p.n;
@@ -91,7 +93,7 @@ __global__ void __launch_bounds__(kBlock) noalloc_sssp_kernel(NaParams p) {
         if (t < 0 || t >= n || (p.w && p.w[e] < 0)) bad = 1;
     }
     if (bad) atomicOr(&c->status, kNaBadInput);
-    if (!grid_sync(c, p.timeout_ns)) return;
+    if (!team_sync(team, c, p.timeout_ns)) return;
     if (__ldcg(&c->status) & kNaBadInput) return;
 
     const unsigned lane = lane_id();
@@ -106,7 +108,6 @@ __global__ void __launch_bounds__(kBlock) noalloc_sssp_kernel(NaParams p) {
             break;
         }
         rounds = r;
-        if (tid == 0) c->changed[(r + 1) % 3] = 0;
         const int32_t *cur = (r & 1) ? p.A : B;
         int32_t *next = (r & 1) ? B : p.A;
         const int32_t *scur = (r & 1) ? S1 : S0;
@@ -153,10 +154,8 @@ __global__ void __launch_bounds__(kBlock) noalloc_sssp_kernel(NaParams p) {
                 if (k < total) na_relax(p, cur, next, snext, r, ob + (k - oe), ov, changed, overflow);
             }
         }
-        changed = warp_sum(changed);
-        if (lane == 0 && changed) atomicAdd(&c->changed[r % 3], changed);
-        if (!grid_sync(c, p.timeout_ns)) return;
-        if (__ldcg(&c->changed[r % 3]) == 0) {
+        if (!team_sync(team, c, p.timeout_ns, changed)) return;
+        if (team_total() == 0) {
             res = next;
             break;
         }
@@ -167,7 +166,7 @@ __global__ void __launch_bounds__(kBlock) noalloc_sssp_kernel(NaParams p) {
     if (res == B)
         for (int64_t v = tid; v < n; v += nth) p.A[v] = ldcg(B + v);
     // overflow rule: a finite vertex with an edge to a vertex left at INF
-    if (!grid_sync(c, p.timeout_ns)) return;
+    if (!team_sync(team, c, p.timeout_ns)) return;
     if (!(__ldcg(&c->status) & kStOverflow)) return;
     for (int64_t u = tid; u < n; u += nth) {
         if (ldcg(p.A + u) == kInf) continue;
