@@ -641,8 +641,20 @@ __device__ __forceinline__ void relax_rows_of_warp(const int32_t *__restrict__ c
     }
 }
 
+// Vertex ids a warp tests per step of a dense scan: 128, four a lane, on
+// graphs that give every warp of the team as many; on smaller ones 8 to 32,
+// at most one a lane.  A step's edges are relaxed one batch after the other,
+// each a chain of three or four dependent loads, so on a small graph 128 ids
+// a step leave most warps idle while a few chain many batches (16,384
+// vertices of degree 8, 912 CTAs: 128 of 7,296 warps work, rounds of 60 K
+// edges take 33 us; with 8 ids a step 8 us).
+__device__ __forceinline__ int scan_step(int64_t n, int64_t nw) {
+    return n >= nw * 128 ? 128 : n > nw * 16 ? 32 : n > nw * 8 ? 16 : 8;
+}
+
 // Synchronous low-degree path: the warp scans 128 consecutive vertex ids per
-// step with 128-bit loads of the activity word (round stamp, or BFS level),
+// step (fewer on small graphs, scan_step) with 128-bit loads of the activity
+// word (round stamp, or BFS level),
 // compacts the active vertices with 1..31 out-edges into shared memory, and
 // relaxes their edges 32 rows at a time.  Mid and high vertices are expanded
 // from their bucket lists; vertices without out-edges have nothing to expand.
@@ -657,11 +669,15 @@ __device__ __forceinline__ void expand_low_dense(const Team &t, const uint32_t *
     const int wid = threadIdx.x >> 5;
     const int64_t gw = (t.rank * (int64_t)kBlock + threadIdx.x) >> 5;
     const int64_t nw = (int64_t)t.size * kWarps;
-    for (int64_t w0 = gw * 128; w0 < n; w0 += nw * 128) {
-        const int64_t v0 = w0 + 4 * lane;
-        if (lane == 0) a.scanned += min((int64_t)128, (int64_t)n - w0);
+    const int step = scan_step(n, nw);
+    for (int64_t w0 = gw * step; w0 < n; w0 += nw * step) {
+        const int64_t v0 = step == 128 ? w0 + 4 * lane : w0 + lane;
+        if (lane == 0) a.scanned += min((int64_t)step, (int64_t)n - w0);
         int32_t st[4];
-        if (v0 + 3 < n) {
+        if (step != 128) {
+            st[0] = (int)lane < step && v0 < n ? ldcg(actw + v0) : act_val - 1;
+            st[1] = st[2] = st[3] = act_val - 1;
+        } else if (v0 + 3 < n) {
             int4 t = __ldcg(reinterpret_cast<const int4 *>(actw + v0));
             st[0] = t.x; st[1] = t.y; st[2] = t.z; st[3] = t.w;
         } else {
@@ -824,12 +840,14 @@ __device__ __forceinline__ void expand_vertices(const Team &t, const uint32_t *_
         }
     }
     // low-degree vertices: a thread each, edges redistributed over the warp
-    for (int base = gw * 32; base < n_low; base += nw * 32) {
+    // (8 or 16 vertices a warp when the list is short, as in scan_step)
+    const int step = n_low > nw * 16 ? 32 : n_low > nw * 8 ? 16 : 8;
+    for (int base = gw * step; base < n_low; base += nw * step) {
         int i = base + (int)lane;
         int32_t vv = 0, u = 0;
         uint32_t rb = 0, d = 0;
         bool rq = false;
-        if (i < n_low) {
+        if ((int)lane < step && i < n_low) {
             u = ldcg(low + i);
             if (op.active(u, vv, rq)) {
                 op.own(u, vv);

@@ -247,13 +247,17 @@ __device__ __forceinline__ void ms_round(const Team &t, const View &g, int32_t *
             }
         }
     }
-    // ---- low-degree vertices (1..31 out-edges): dense scan of 128 ids per warp step
+    // ---- low-degree vertices (1..31 out-edges): dense scan of 128 ids per warp step (fewer on small graphs)
     const int32_t n = g.n;
-    for (int64_t w0 = (int64_t)gw * 128; w0 < n; w0 += (int64_t)nw * 128) {
-        const int64_t v0 = w0 + 4 * lane;
-        if (lane == 0) a.scanned += min((int64_t)128, (int64_t)n - w0);
+    const int step = scan_step(n, nw);
+    for (int64_t w0 = (int64_t)gw * step; w0 < n; w0 += (int64_t)nw * step) {
+        const int64_t v0 = step == 128 ? w0 + 4 * lane : w0 + lane;
+        if (lane == 0) a.scanned += min((int64_t)step, (int64_t)n - w0);
         int32_t st[4];
-        if (v0 + 3 < n) {
+        if (step != 128) {
+            st[0] = (int)lane < step && v0 < n ? ldcg(stamp + v0) : 0;
+            st[1] = st[2] = st[3] = 0;
+        } else if (v0 + 3 < n) {
             const int4 s4 = __ldcg(reinterpret_cast<const int4 *>(stamp + v0));
             st[0] = s4.x; st[1] = s4.y; st[2] = s4.z; st[3] = s4.w;
         } else {
@@ -657,12 +661,16 @@ __device__ __forceinline__ void msb_round(const Team &t, const View &g, const Pa
             }
         }
     }
-    // ---- low-degree vertices (1..31 out-edges): dense scan of the frontier bytes, 128 per warp step
+    // ---- low-degree vertices (1..31 out-edges): dense scan of the frontier bytes, 128 per warp step (fewer on
+    // small graphs)
     const int32_t n = g.n;
-    for (int64_t w0 = (int64_t)gw * 128; w0 < n; w0 += (int64_t)nw * 128) {
-        const int64_t v0 = w0 + 4 * lane;
-        if (lane == 0) a.scanned += min((int64_t)128, (int64_t)n - w0);
-        const uint32_t w4 = v0 < n ? ldcg_u32(cur + v0) : 0u;   // the buffers are padded to 16 bytes
+    const int step = scan_step(n, nw);
+    for (int64_t w0 = (int64_t)gw * step; w0 < n; w0 += (int64_t)nw * step) {
+        const int64_t v0 = step == 128 ? w0 + 4 * lane : w0 + lane;
+        if (lane == 0) a.scanned += min((int64_t)step, (int64_t)n - w0);
+        uint32_t w4 = 0;
+        if (step != 128) w4 = (int)lane < step && v0 < n ? (uint32_t)__ldcg(cur + v0) : 0u;
+        else if (v0 < n) w4 = ldcg_u32(cur + v0);   // the buffers are padded to 16 bytes
         bool act[4];
         uint32_t rb[4], d[4], fm[4];
 #pragma unroll
