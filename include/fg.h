@@ -16,7 +16,10 @@
  *                   in-place atomic MIN, run until the worklist is empty; an
  *                   SSSP generation whose worklist holds a quarter of the
  *                   vertices with out-edges or more tests every vertex
- *                   instead (queued, or lowered during the generation);
+ *                   instead (queued, or lowered during the generation); CC on
+ *                   a renumbered graph hooks every vertex under a small
+ *                   neighbour, links what is left outside the largest tree
+ *                   and compresses (three generations, whatever the graph);
  *   FG_EDGE_ASYNC   the same worklist expanded to its out-edges and relaxed
  *                   edge-parallel, in place; a generation whose worklist holds
  *                   a quarter of the edges or more (BFS: half) streams the
@@ -222,8 +225,8 @@ fg_status fg_cc(const fg_graph *g, int32_t *label_out, fg_mode mode);
  *   BFS   deep: FG_BUCKET from 2^21 vertices, else FG_VERTEX_SYNC;
  *         shallow: FG_PULL if skewed, else FG_VERTEX_SYNC;
  *   CC    deep: FG_PULL below 2^23 vertices, else FG_VERTEX_SYNC;
- *         shallow: FG_EDGE_SYNC if not skewed or below 2^14 vertices,
- *         FG_BUCKET below 2^19, else FG_VERTEX_ASYNC;
+ *         shallow: FG_EDGE_SYNC if not skewed, else FG_BUCKET below 2^19
+ *         vertices, FG_VERTEX_ASYNC from there on;
  * with 2 CTAs per SM for graphs of at most 3 million edges (BFS: 9 million),
  * whose rounds are short enough that a grid barrier over fewer CTAs pays,
  * else the occupancy limit.  FG_AUTO runs the plan (its CTAs per SM unless

@@ -1784,6 +1784,170 @@ constexpr int min_blocks() {
                                : FG_ASYNC_MIN_BLOCKS;
 }
 
+// ================================================================ components by hooking and linking
+// FG_VERTEX_ASYNC (and FG_BUCKET) CC on a renumbered graph: a forest of
+// parent labels instead of label propagation, after the sampled-neighbours
+// method of Sutton, Ben-Nun and Barak (Afforest, IPDPS 2018).  Propagation
+// passes over all symmetrised edges twice, each edge a random probe: 0.68 +
+// 0.61 ms on R-MAT 22 (134 M edges).  Here
+//   1. every vertex hooks under the smallest of its first few neighbours, if
+//      that is smaller than itself (a plain store: the labels start out so),
+//      and the chains are compressed to their roots;
+//   2. the first kCcHubs vertices, the hubs of a renumbered graph, link their
+//      first neighbours: two trees are joined by a compare-and-swap that
+//      hooks the larger root under the smaller label; compression again;
+//   3. the vertices outside the tree that holds the highest-degree vertex
+//      link all their edges; an edge inside that tree needs no look, and one
+//      that leaves it is seen from its other end (every edge is stored both
+//      ways);
+//   4. after a last compression every label is its tree's root, the smallest
+//      id of the component.
+// Parents only ever have smaller ids, so the forest stays one under any
+// order of the stores.  Renumbering puts the hubs first: almost every vertex
+// of a skewed graph has one among its first neighbours, few are left for step
+// 3, and the chains are a handful of steps.  A graph in its own order (a
+// grid) has chains as long as its side, and keeps the propagation.  The
+// walks read through L1: the big tree's root is one word that every vertex
+// asks for, and at one L2 slice those reads alone took 60 ms.  Measured on
+// R-MAT 22: 1.28 -> 0.18 ms, R-MAT 16 0.11 -> 0.03 ms; it is bound by the row
+// heads' sectors (85 us) and the barriers of five short passes.
+constexpr int kCcSampleLow = 4, kCcSampleMid = 32, kCcSampleHigh = 256;   // neighbours hooked by, per degree class
+constexpr int kCcHubs = 4096, kCcHubSample = 64;
+
+// joins the trees that hold labels x and y
+__device__ __forceinline__ void cc_link(int32_t *P, int32_t x, int32_t y, Acc &a) {
+    for (int k = 0; x != y; k++) {
+        const int32_t hi = max(x, y), lo = min(x, y);
+        int32_t up = ldcg(P + hi);
+        if (up == lo) return;
+        if (up == hi) {   // a root: hook it, unless another edge just did
+            up = atomicCAS(P + hi, hi, lo);
+            if (up == hi) {
+                a.updates++;
+                return;
+            }
+        } else if (k >= 16) {   // a long walk: halve the path (a label may move to any vertex above it)
+            const int32_t above = ldcg(P + up);
+            if (above < up) stcg(P + hi, up = above);
+        }
+        x = up;
+        y = lo;
+    }
+}
+
+struct CcLinkOp {
+    static constexpr bool kNextProbe = false;
+    int32_t *P;
+    int32_t giant;     // label of the tree that needs no look
+
+    __device__ __forceinline__ bool active(int32_t u, int32_t &val, bool &) const {
+        val = ldcg(P + u);
+        return val != giant;
+    }
+    __device__ __forceinline__ void own(int32_t, int32_t) const {}
+    __device__ __forceinline__ int32_t refresh(int32_t, int32_t val) const { return val; }
+    __device__ __forceinline__ bool cand(int32_t val, uint32_t, int32_t &c, Acc &) const {
+        c = val;
+        return true;
+    }
+    __device__ __forceinline__ int32_t probe(int32_t v) const { return ldca(P + v); }
+    __device__ __forceinline__ bool commit(int32_t, int32_t c, int32_t pv, Acc &a) const {
+        cc_link(P, c, pv, a);
+        return false;
+    }
+};
+
+// Every label to its root; no link runs at the same time.  A pass walks up to
+// 64 steps and repeats until every walk ended, so that a long chain (a path
+// inside a skewed graph) is shortened 64-fold a pass.
+template <class SYNC>
+__device__ __forceinline__ bool cc_compress(int32_t *P, int32_t n, int64_t tid, int64_t nth, const SYNC &sync_) {
+    for (;;) {
+        int open = 0;
+        for (int64_t v = tid; v < n; v += nth) {
+            const int32_t l0 = ldcg(P + v);
+            if (l0 == (int32_t)v) continue;
+            int32_t l = l0;
+            bool end = false;
+#pragma unroll 1
+            for (int k = 0; k < 64; k++) {
+                const int32_t ll = ldca(P + l);   // an old copy is a label further down the same chain
+                if (ll == l) {
+                    end = true;
+                    break;
+                }
+                l = ll;
+            }
+            open += !end;
+            if (l < l0) stcg(P + v, l);
+        }
+        if (!sync_(open)) return false;
+        if (team_total() == 0) return true;
+    }
+}
+
+// The smallest of v's first K * 32 neighbours and v itself, by a warp, stored as v's label.
+template <int K>
+__device__ __forceinline__ void cc_hook_by_warp(const View &g, int32_t *P, int32_t v, Acc &a) {
+    const uint32_t b = __ldg(g.row_off + v) + lane_id(), e = __ldg(g.row_off + v + 1);
+    int32_t l = v;
+#pragma unroll
+    for (int k = 0; k < K; k++)
+        if (b + 32 * k < e) {
+            l = min(l, __ldg(g.col + b + 32 * k));
+            a.edges++;
+        }
+    l = __reduce_min_sync(0xffffffffu, l);
+    if (lane_id() == 0) stcg(P + v, l);
+}
+
+// Steps 1-4 on the symmetrised view g; p.A holds the labels.  SYNC is the
+// query's barrier.  Returns false if a barrier failed.
+template <class SYNC>
+__device__ __forceinline__ bool cc_hook_link(const Params &p, const Team &t, const View &g, Acc &a,
+                                             const SYNC &sync_) {
+    int32_t *P = p.A;
+    const int64_t tid = t.rank * (int64_t)kBlock + threadIdx.x;
+    const int64_t nth = (int64_t)t.size * kBlock;
+    const int gw = (int)(tid >> 5), nw = (int)(nth >> 5);
+    for (int i = gw; i < g.n_high_chunks; i += nw) {
+        const int2 hc = __ldg(g.high + i);
+        if ((uint32_t)hc.y == __ldg(g.row_off + hc.x)) cc_hook_by_warp<kCcSampleHigh / 32>(g, P, hc.x, a);
+    }
+    for (int i = gw; i < g.n_mid; i += nw) cc_hook_by_warp<kCcSampleMid / 32>(g, P, __ldg(g.mid + i), a);
+    for (int64_t v = tid; v < g.n; v += nth) {
+        const uint32_t b = __ldg(g.row_off + v), e = __ldg(g.row_off + v + 1);
+        if (e - b >= (uint32_t)kLowMax) continue;
+        int32_t l = (int32_t)v;
+#pragma unroll
+        for (int k = 0; k < kCcSampleLow; k++)
+            if (b + k < e) l = min(l, __ldg(g.col + b + k));
+        stcg(P + v, l);
+        a.edges += min((uint32_t)kCcSampleLow, e - b);
+    }
+    if (!sync_()) return false;
+    if (!cc_compress(P, g.n, tid, nth, sync_)) return false;
+    for (int v = gw; v < min(g.n, kCcHubs); v += nw) {
+        const uint32_t b = __ldg(g.row_off + v), e = min(__ldg(g.row_off + v + 1), b + kCcHubSample);
+        const int32_t l = ldca(P + v);
+        for (uint32_t k = b + lane_id(); k < e; k += 32) {
+            cc_link(P, l, ldca(P + __ldg(g.col + k)), a);
+            a.edges++;
+        }
+    }
+    if (!sync_()) return false;
+    if (!cc_compress(P, g.n, tid, nth, sync_)) return false;
+    const int32_t pick = g.n_high_chunks > 0 ? __ldg(&g.high[0].x)
+                         : g.n_mid > 0       ? __ldg(g.mid)
+                         : g.n_low > 0       ? __ldg(g.low)
+                                             : 0;
+    const CcLinkOp op{P, ldcg(P + pick)};
+    expand_vertices(t, g.row_off, g.col, g.low, g.n_low, g.mid, g.n_mid, g.high, g.n_high_chunks, op, NoPush{}, a);
+    if (!sync_()) return false;
+    return cc_compress(P, g.n, tid, nth, sync_);
+}
+constexpr int kCcHookRounds = 3;   // generations it counts as: hooks, links, the last compression
+
 // The whole query -- init, rounds, convergence -- run by one team of CTAs
 // (the full grid for a single query, a slice of it in a batch).
 // Once per kernel launch, before the first fixpoint_body: the edge-sync
@@ -1821,8 +1985,12 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
     if (threadIdx.x == 0) bar_state().err = 0;   // of this query
     // the source in internal ids (a renumbered graph takes original ones)
     const int32_t source = (ALGO != kCC && p.new_of) ? __ldg(p.new_of + p.source) : p.source;
+    // components by hooking and linking: labels and everything else set there
+    const bool cc_hook = ALGO == kCC && (MODE == kVertexAsync || MODE == kBucket) && p.new_of;
     // ---- init: values, stamps, initial worklist (a2)
-    for (int64_t v = tid; v < n; v += nth) {
+    if (cc_hook && p.cc_min)
+        for (int64_t v = tid; v < n; v += nth) p.cc_min[v] = kInf;
+    for (int64_t v = cc_hook ? n : tid; v < n; v += nth) {
         int32_t x = (ALGO == kCC) ? (int32_t)v : (v == source ? 0 : kInf);
         p.A[v] = x;
         if (SYNC && ALGO != kBFS) {
@@ -1866,9 +2034,18 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
     }
     // failure-detection test: CTA 0 never arrives, the others' waits run out
     if (p.inject_missing_arrival && t.rank == 0) return;
-    bool ok = sync_();
+    bool ok = cc_hook || sync_();
 
-    if (SYNC && ok) {
+    if (cc_hook) {
+        if constexpr (ALGO == kCC && (MODE == kVertexAsync || MODE == kBucket)) {
+            if (p.max_rounds < kCcHookRounds) {
+                if (tid == 0) atomicOr(&c->status, kStRoundCap);
+            } else {
+                rounds = kCcHookRounds;
+                done = cc_hook_link(p, t, g, a, sync_);
+            }
+        }
+    } else if (SYNC && ok) {
         int64_t ch_prev = 0;     // changes of the previous round, from its barrier (the same in every thread)
         int64_t ch_before = 0;   // changes of the round before it
         constexpr bool kW = (ALGO == kSSSP);   // the edge rings carry weights for SSSP only
