@@ -34,11 +34,57 @@ namespace fg {
 namespace {
 
 
+// A thread's counters since the last barrier, 32 bits each: a round's count
+// of one warp stays below 2^32 (at most 2^32 symmetrised edges over the eight
+// warps of the smallest team).  stat_flush adds them at every barrier to the
+// CTA's 64-bit totals in shared memory, so that the kernels' hot loops carry
+// no 64-bit accumulator: twelve registers of the 40 that six CTAs per SM
+// leave, which were spilled in every vertex kernel.
 struct Acc {
-    unsigned long long edges = 0, verts = 0, updates = 0, pushes = 0, scanned = 0, pulled = 0;
+    uint32_t edges = 0, verts = 0, updates = 0, pushes = 0, scanned = 0, pulled = 0;
     int changed = 0;
     int overflow = 0;
 };
+constexpr int kStats = 6;
+struct StatTotals {
+    unsigned long long v[kStats][kWarps];
+};
+__device__ __forceinline__ StatTotals &stat_totals() {
+    __shared__ StatTotals s;
+    return s;
+}
+// Every warp clears its own totals (before the first flush of a query).
+__device__ __forceinline__ void stat_begin() {
+    if (lane_id() < kStats) stat_totals().v[lane_id()][threadIdx.x >> 5] = 0;
+    __syncwarp();
+}
+// Every lane of the warp calls it; a's counters (changed and overflow
+// excepted) go to the warp's totals.
+__device__ __forceinline__ void stat_flush(Acc &a) {
+    const uint32_t x[kStats] = {a.edges, a.verts, a.updates, a.pushes, a.scanned, a.pulled};
+    uint32_t mine = 0;
+#pragma unroll
+    for (int i = 0; i < kStats; i++) {
+        const uint32_t s = __reduce_add_sync(0xffffffffu, x[i]);
+        if ((int)lane_id() == i) mine = s;
+    }
+    if (lane_id() < kStats) stat_totals().v[lane_id()][threadIdx.x >> 5] += mine;
+    a.edges = a.verts = a.updates = a.pushes = a.scanned = a.pulled = 0;
+}
+// The CTA's totals to the query's control block, by every thread, after a barrier.
+__device__ __forceinline__ void stat_report(Acc &a, Ctrl *c) {
+    stat_flush(a);
+    if (__syncthreads_or(a.overflow) && threadIdx.x == 0) atomicOr(&c->status, kStOverflow);
+    if (threadIdx.x < kStats) {
+        unsigned long long s = 0;
+        for (int w = 0; w < kWarps; w++) s += stat_totals().v[threadIdx.x][w];
+        unsigned long long *const to[kStats] = {&c->st_edges,  &c->st_vertices, &c->st_updates,
+                                                &c->st_pushes, &c->st_scanned,  &c->st_pulled};
+#pragma unroll
+        for (int i = 0; i < kStats; i++)
+            if ((int)threadIdx.x == i && s) atomicAdd(to[i], s);
+    }
+}
 
 __device__ __forceinline__ int32_t warp_min(int32_t x) {
 #pragma unroll
@@ -1213,7 +1259,7 @@ __device__ __forceinline__ void flag_edge_tiles(const Team &t, const View &g, co
 #pragma unroll
             for (int j = 0; j < 4; j++) act[j] = vb + j < n && ldcg(actw + vb + j) == act_val;
         }
-        if (lane == 0) a.scanned += (uint64_t)min((int64_t)128, (int64_t)n - v0);
+        if (lane == 0) a.scanned += (uint32_t)min((int64_t)128, (int64_t)n - v0);
         uint32_t big_t0 = 0, big_t1 = 0;
         bool big = false;
 #pragma unroll
@@ -1491,7 +1537,7 @@ __device__ __forceinline__ bool stream_all_edges(const Team &t, uint32_t &used, 
     const int64_t ntiles = (g.m + kWTile - 1) / kWTile;
     const int64_t gw = (int64_t)t.rank * kWarps + (threadIdx.x >> 5), nw = (int64_t)t.size * kWarps;
     const int count = ntiles > gw ? (int)((ntiles - 1 - gw) / nw + 1) : 0;
-    if (t.rank == 0 && threadIdx.x == 0) a.scanned += (uint64_t)g.m;
+    if (t.rank == 0 && threadIdx.x == 0) a.scanned += (uint32_t)g.m;
     const bool ok = warp_stream(R.warp[threadIdx.x >> 5], R.pol, used, count,
                                 [&](int k) { return gw + (int64_t)k * nw; }, g, op, a, c, timeout_ns);
     return __syncthreads_and(ok);
@@ -1525,7 +1571,7 @@ __device__ __forceinline__ bool stream_flagged_edges(const Team &t, uint32_t &us
         if (lane == 0)
             for (int i = 0; i < na; i++) {
                 const int64_t e0 = (int64_t)s_wl[wid][i] * kWTile;
-                a.scanned += (uint64_t)min((int64_t)kWTile, g.m - e0);
+                a.scanned += (uint32_t)min((int64_t)kWTile, g.m - e0);
             }
         ok = warp_stream(R.warp[wid], R.pol, used, na, [&](int i) { return (int64_t)s_wl[wid][i]; }, g, op, a, c,
                          timeout_ns);
@@ -1660,7 +1706,7 @@ __device__ __forceinline__ void stream_edges_async(const Team &t, const View &g,
                                                    Acc &a) {
     const int64_t ntiles = (g.m + kWTile - 1) / kWTile;
     const int64_t gw = (int64_t)t.rank * kWarps + (threadIdx.x >> 5), nw = (int64_t)t.size * kWarps;
-    if (t.rank == 0 && threadIdx.x == 0) a.scanned += (uint64_t)g.m;
+    if (t.rank == 0 && threadIdx.x == 0) a.scanned += (uint32_t)g.m;
     for (int64_t tile = gw; tile < ntiles; tile += nw) {   // warp-uniform
         RawQuad r;
         raw_load<W>(g, tile * kWTile, r);
@@ -1973,7 +2019,9 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
     int n_barriers = 0;
     bool done = false;
     // every grid barrier of the query; CTA 0 optionally timestamps each
+    stat_begin();
     auto sync_ = [&](int add = 0) -> bool {
+        stat_flush(a);
         bool r = team_sync(t, c, p.timeout_ns, add);
         if (tid == 0) {
             if (p.trace && n_barriers < p.trace_cap) p.trace[n_barriers] = global_ns();
@@ -2347,25 +2395,14 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
                     }
                 }
                 push.flush();
-                if (tid == 0 && !dense) a.verts += (unsigned long long)n_in[0];
+                if (tid == 0 && !dense) a.verts += (uint32_t)n_in[0];
             }
             if (!sync_()) break;
         }
     }
 
     // ---- statistics
-    unsigned long long ev = block_sum(a.verts), ee = block_sum(a.edges), eu = block_sum(a.updates),
-                       ep = block_sum(a.pushes), es = block_sum(a.scanned), el = block_sum(a.pulled);
-    int of = block_sum(a.overflow);
-    if (threadIdx.x == 0) {
-        if (ev) atomicAdd(&c->st_vertices, ev);
-        if (ee) atomicAdd(&c->st_edges, ee);
-        if (eu) atomicAdd(&c->st_updates, eu);
-        if (ep) atomicAdd(&c->st_pushes, ep);
-        if (es) atomicAdd(&c->st_scanned, es);
-        if (el) atomicAdd(&c->st_pulled, el);
-        if (of) atomicOr(&c->status, kStOverflow);
-    }
+    stat_report(a, c);
     if (tid == 0) {
         c->rounds = rounds;
         c->barriers = n_barriers;

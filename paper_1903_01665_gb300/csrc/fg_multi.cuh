@@ -383,7 +383,9 @@ __device__ __forceinline__ void multi_body(const Params &p, const Team &t) {
     int rounds = 0, n_barriers = 0;
     bool done = false;
     if (threadIdx.x == 0) bar_state().err = 0;   // of this query
+    stat_begin();
     auto sync_ = [&](int add = 0) -> bool {
+        stat_flush(a);
         const bool ok = team_sync(t, c, p.timeout_ns, add);
         n_barriers++;
         return ok;
@@ -478,14 +480,7 @@ __device__ __forceinline__ void multi_body(const Params &p, const Team &t) {
         if (!sync_()) break;
     }
     // ---- statistics
-    const unsigned long long ev = block_sum(a.verts), ee = block_sum(a.edges), eu = block_sum(a.updates),
-                             es = block_sum(a.scanned);
-    if (threadIdx.x == 0) {
-        if (ev) atomicAdd(&c->st_vertices, ev);
-        if (ee) atomicAdd(&c->st_edges, ee);
-        if (eu) atomicAdd(&c->st_updates, eu);
-        if (es) atomicAdd(&c->st_scanned, es);
-    }
+    stat_report(a, c);
     if (tid == 0) {
         c->rounds = rounds;
         c->barriers = n_barriers;
@@ -757,7 +752,9 @@ __device__ __forceinline__ void multi_bfs_body(const Params &p, const Team &t) {
     int rounds = 0, n_barriers = 0;
     bool done = false;
     if (threadIdx.x == 0) bar_state().err = 0;   // of this query
+    stat_begin();
     auto sync_ = [&](int add = 0) -> bool {
+        stat_flush(a);
         const bool ok = team_sync(t, c, p.timeout_ns, add);
         n_barriers++;
         return ok;
@@ -800,14 +797,7 @@ __device__ __forceinline__ void multi_bfs_body(const Params &p, const Team &t) {
             break;
         }
     }
-    const unsigned long long ev = block_sum(a.verts), ee = block_sum(a.edges), eu = block_sum(a.updates),
-                             es = block_sum(a.scanned);
-    if (threadIdx.x == 0) {
-        if (ev) atomicAdd(&c->st_vertices, ev);
-        if (ee) atomicAdd(&c->st_edges, ee);
-        if (eu) atomicAdd(&c->st_updates, eu);
-        if (es) atomicAdd(&c->st_scanned, es);
-    }
+    stat_report(a, c);
     if (tid == 0) {
         c->rounds = rounds;
         c->barriers = n_barriers;
