@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "fg_internal.cuh"
+#include "fg_partition.cuh"
 
 namespace fg {
 
@@ -241,13 +242,36 @@ __global__ void k_fill_ones(int64_t m, int32_t *w) {
         w[e] = 1;
 }
 
-// src[e] = owner row of edge e, one warp per vertex.
-__global__ void k_src_from_rows(int32_t n, const uint32_t *__restrict__ ro, int32_t *src) {
-    int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t v = warp; v < n; v += nwarps) {
-        uint32_t b = ro[v], e = ro[v + 1];
-        for (uint32_t k = b + lane_id(); k < e; k += 32) src[k] = (int32_t)v;
+// Grouped build: out-degree of every vertex (internal id) from the counts by original id.
+__global__ void k_part_degrees(int32_t n, const uint32_t *__restrict__ count, int flag,
+                               const int32_t *__restrict__ new_of, uint32_t *deg) {
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x)
+        deg[new_of ? new_of[x] : x] = flag ? count[2 * x] + count[2 * x + 1] : count[x];
+}
+// Grouped build: the counts by original id become write positions: row v's
+// first edge, then (flag) its first flagged one; skip: edges that row v holds
+// already (the out-edges of the symmetrised view), from row offsets.
+__global__ void k_part_cursors(int32_t n, uint32_t *count, int flag, const uint32_t *__restrict__ ro,
+                               const uint32_t *__restrict__ skip_ro, const int32_t *__restrict__ new_of) {
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t v = new_of ? new_of[x] : x;
+        uint32_t at = ro[v];
+        if (skip_ro) at += skip_ro[v + 1] - skip_ro[v];
+        if (flag) {
+            const uint32_t c0 = count[2 * x];
+            count[2 * x] = at;
+            count[2 * x + 1] = at + c0;
+        } else {
+            count[x] = at;
+        }
+    }
+}
+// The symmetrised rows' first part: the out-edges, in CSR order.
+__global__ void k_sym_out(int64_t m, const int32_t *__restrict__ src, const int32_t *__restrict__ col,
+                          const uint32_t *__restrict__ ro, const uint32_t *__restrict__ sro, int32_t *scol) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t u = src[e];
+        scol[sro[u] + ((uint32_t)e - ro[u])] = col[e];
     }
 }
 
@@ -493,6 +517,106 @@ struct Builder {
     }
 };
 
+unsigned row_grid(int64_t m) { return (unsigned)((m + kRowTile - 1) / kRowTile); }
+
+// Edges grouped by an id (fg_partition.cuh): after pass 1, by bucket.
+struct Grouped {
+    PartShape sh;
+    PartPlan plan;
+    uint32_t *words = nullptr;    // one allocation: histogram, plan
+    uint16_t *sub = nullptr;
+    int32_t *a = nullptr, *b = nullptr;
+    uint32_t *count = nullptr;    // per sub-digit; then the cursors of pass 2
+    bool ready = false;
+    uint32_t *hist() const { return words; }
+};
+
+template <typename K>
+void part_kernel_smem(Builder &b, K k, size_t bytes) {
+    b.check(cudaFuncSetAttribute((const void *)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes),
+            "shared memory of the grouping kernels");
+}
+
+// The words of a grouping (histogram cleared).
+void group_alloc(Builder &b, Grouped &q, int32_t n, int flag) {
+    q.sh = part_shape(n, flag);
+    const int nb = q.sh.nb;
+    q.words = b.alloc_tmp<uint32_t>(4 * (int64_t)nb + 2);
+    if (b.status != FG_OK) return;
+    q.plan.start = q.words + nb;
+    q.plan.cursor = q.plan.start + nb + 1;
+    q.plan.tile0 = q.plan.cursor + nb;
+    b.check(cudaMemsetAsync(q.words, 0, (size_t)nb * sizeof(uint32_t), b.st), "memset");
+}
+
+void group_free(Builder &b, Grouped &q) {
+    void *all[] = {q.words, q.sub, q.a, q.b, q.count};
+    for (void *p : all)
+        if (p) cudaFreeAsync(p, b.st);
+    q = Grouped();
+}
+
+// Edges per bucket of s into qs, of t (may be null) into qt; VALIDATE as k_part_hist.
+template <bool VALIDATE>
+void group_hist(Builder &b, int32_t n, int64_t m, const int32_t *s, const int32_t *t, const int32_t *w, Grouped &qs,
+                Grouped *qt, int *flags, unsigned long long *wsum) {
+    if (b.status != FG_OK) return;
+    const size_t bytes = 2 * (size_t)qs.sh.nb * sizeof(uint32_t);
+    part_kernel_smem(b, k_part_hist<VALIDATE>, bytes);
+    k_part_hist<VALIDATE><<<grid_for(m, 4 * kPartThreads) > 608 ? 608 : grid_for(m, 4 * kPartThreads), kPartThreads,
+                            bytes, b.st>>>(m, n, s, t, w, qs.sh, qs.hist(), qt ? qt->hist() : nullptr, flags, wsum);
+    count_launch();
+    b.check(cudaGetLastError(), "edges per bucket");
+}
+
+// Pass 1 and the counts per sub-digit, the histogram given.
+void group_pass1(Builder &b, Grouped &q, int64_t m, const int32_t *key, const int32_t *a, const int32_t *w, bool with_w,
+                 int32_t split) {
+    if (b.status != FG_OK) return;
+    q.sub = b.alloc_tmp<uint16_t>(m);
+    q.a = b.alloc_tmp<int32_t>(m);
+    if (with_w) q.b = b.alloc_tmp<int32_t>(m);
+    q.count = b.alloc_tmp<uint32_t>(q.sh.counters());
+    if (b.status != FG_OK) return;
+    b.check(cudaMemsetAsync(q.count, 0, (size_t)q.sh.counters() * sizeof(uint32_t), b.st), "memset");
+    k_part_plan<<<1, 1024, 0, b.st>>>(q.hist(), q.sh.nb, q.plan);
+    count_launch();
+    const unsigned g1 = (unsigned)((m + kPartTile - 1) / kPartTile);
+    const size_t bytes = part_smem(q.sh.nb, with_w ? 12 : 8);
+    if (with_w) {
+        part_kernel_smem(b, k_part_pass1<true>, bytes);
+        k_part_pass1<true><<<g1, kPartThreads, bytes, b.st>>>(m, key, a, w, q.sh, split, q.plan.cursor, q.sub, q.a, q.b);
+    } else {
+        part_kernel_smem(b, k_part_pass1<false>, bytes);
+        k_part_pass1<false><<<g1, kPartThreads, bytes, b.st>>>(m, key, a, nullptr, q.sh, split, q.plan.cursor, q.sub,
+                                                              q.a, nullptr);
+    }
+    count_launch();
+    const size_t cbytes = (size_t)q.sh.sub() * sizeof(uint32_t);
+    k_part_count<<<part_grid2(m, q.sh), kPartThreads, cbytes, b.st>>>(q.plan, q.sh, q.sub, q.count);
+    count_launch();
+    b.check(cudaGetLastError(), "grouping by bucket");
+    q.ready = b.status == FG_OK;
+}
+
+// Pass 2 to out_a (through map) and out_b; q.count holds the cursors.
+void group_pass2(Builder &b, Grouped &q, int64_t m, const int32_t *map, int32_t *out_a, int32_t *out_b) {
+    if (b.status != FG_OK) return;
+    const bool with_w = q.b != nullptr;
+    const size_t bytes = part_smem(q.sh.sub(), with_w ? 10 : 6);
+    if (with_w) {
+        part_kernel_smem(b, k_part_pass2<true>, bytes);
+        k_part_pass2<true><<<part_grid2(m, q.sh), kPartThreads, bytes, b.st>>>(q.plan, q.sh, q.sub, q.a, q.b, map,
+                                                                              q.count, out_a, out_b);
+    } else {
+        part_kernel_smem(b, k_part_pass2<false>, bytes);
+        k_part_pass2<false><<<part_grid2(m, q.sh), kPartThreads, bytes, b.st>>>(q.plan, q.sh, q.sub, q.a, nullptr, map,
+                                                                               q.count, out_a, nullptr);
+    }
+    count_launch();
+    b.check(cudaGetLastError(), "grouping by vertex");
+}
+
 // Degree buckets of one view (row offsets already set).
 void make_buckets(Builder &b, View &v) {
     int32_t n = v.n;
@@ -579,7 +703,7 @@ const T *to_device(Builder &b, const T *p, int64_t count, T **tmp) {
 void build_src(Builder &b, View &v) {
     int32_t *esrc = b.alloc_graph<int32_t>(v.m);
     if (b.status == FG_OK && v.m > 0) {
-        k_src_from_rows<<<grid_for((int64_t)v.n * 32), kBlock, 0, b.st>>>(v.n, v.row_off, esrc);
+        k_row_sources<<<row_grid(v.m), kBlock, 0, b.st>>>(v.n, v.m, v.row_off, esrc);
         count_launch();
         b.check(cudaGetLastError(), "edge sources");
     }
@@ -593,8 +717,10 @@ void build_src(Builder &b, View &v) {
 // The symmetrised view used by connected components: every edge u->v also
 // stored as v->u (the undirected nbrs iterator, Table "foreach iterators"),
 // as CSR plus edge sources.  Needs the directed view's edge sources.
-// indeg: the in-degrees counted at creation (else counted here)
-void build_sym(Builder &b, fg_graph *g, const uint32_t *indeg = nullptr) {
+// indeg: the in-degrees counted at creation (else counted here); by_dst: the
+// edges grouped by their destination's original id at creation (else, on a
+// graph that is large enough, grouped here by the internal one).
+void build_sym(Builder &b, fg_graph *g, const uint32_t *indeg = nullptr, Grouped *by_dst = nullptr) {
     const View &v = g->g;
     const int32_t n = v.n;
     const int64_t m = v.m;
@@ -618,14 +744,34 @@ void build_sym(Builder &b, fg_graph *g, const uint32_t *indeg = nullptr) {
             k_sym_degree<<<grid_for(n), kBlock, 0, b.st>>>(n, v.row_off, deg);
             count_launch();
             b.check(exclusive_scan(deg, sro, n, b.st), "scan");
-            if (g->new_of) {
+            Grouped mine;
+            const bool grouped = (by_dst && by_dst->ready) || part_usable(n, m);
+            if (grouped) {
+                Grouped &q = by_dst && by_dst->ready ? *by_dst : mine;
+                const int32_t *map = &q == &mine ? nullptr : g->new_of;   // original ids, or internal ones
+                if (&q == &mine) {
+                    group_alloc(b, q, n, 0);
+                    group_hist<false>(b, n, m, v.col, nullptr, nullptr, q, nullptr, nullptr, nullptr);
+                    group_pass1(b, q, m, v.col, v.src, nullptr, false, 0);
+                }
+                if (b.status == FG_OK) {
+                    k_part_cursors<<<grid_for(n), kBlock, 0, b.st>>>(n, q.count, 0, sro, v.row_off, map);
+                    count_launch();
+                    group_pass2(b, q, m, map, scol, nullptr);
+                    k_sym_out<<<grid_for(m), kBlock, 0, b.st>>>(m, v.src, v.col, v.row_off, sro, scol);
+                    count_launch();
+                    k_row_sources<<<row_grid(2 * m), kBlock, 0, b.st>>>(n, 2 * m, sro, ssrc);
+                    count_launch();
+                }
+                group_free(b, mine);
+            } else if (g->new_of) {
                 k_sym_cursor_orig<<<grid_for(n), kBlock, 0, b.st>>>(n, sro, v.row_off, g->new_of, cursor);
                 count_launch();
             } else {
                 k_sym_cursor<<<grid_for(n), kBlock, 0, b.st>>>(n, sro, v.row_off, cursor);
                 count_launch();
             }
-            if (m > 0) {
+            if (m > 0 && !grouped) {
                 if (g->new_of) {
                     k_scatter_sym_renum<<<grid_for(m), kBlock, 0, b.st>>>(m, v.src, v.col, v.row_off, sro,
                                                                           g->orig_of, cursor, scol);
@@ -634,7 +780,7 @@ void build_sym(Builder &b, fg_graph *g, const uint32_t *indeg = nullptr) {
                     k_scatter_sym<<<grid_for(m), kBlock, 0, b.st>>>(m, v.src, v.col, v.row_off, sro, cursor, scol);
                     count_launch();
                 }
-                k_src_from_rows<<<grid_for((int64_t)n * 32), kBlock, 0, b.st>>>(n, sro, ssrc);
+                k_row_sources<<<row_grid(2 * m), kBlock, 0, b.st>>>(n, 2 * m, sro, ssrc);
                 count_launch();
             }
             b.check(cudaGetLastError(), "symmetrise");
@@ -670,16 +816,32 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
     if (from_csr) d_ro = to_device(b, row_off_in, (int64_t)n + 1, &t_ro);
     else d_src = to_device(b, src, m, &t_src);
     int *flags = b.alloc_tmp<int>(1);
+    // large edge lists are grouped by source and (unless the symmetrised view
+    // waits) by destination; the validation counts their buckets
+    Grouped by_src, by_dst;
+    bool group = part_usable(n, m);
+    const bool coo_group = group && !from_csr;
+    if (coo_group) {
+        group_alloc(b, by_src, n, 0);
+        group_alloc(b, by_dst, n, 0);
+    }
+    unsigned long long *wsum = b.alloc_tmp<unsigned long long>(1);
+    unsigned long long weights = 0;   // their sum, if the validation formed it
     if (b.status == FG_OK) {
         b.check(cudaMemsetAsync(flags, 0, sizeof(int), b.st), "memset");
-        if (from_csr)
+        b.check(cudaMemsetAsync(wsum, 0, sizeof(unsigned long long), b.st), "memset");
+        if (coo_group)
+            group_hist<true>(b, n, m, d_src, d_dst, d_w, by_src, &by_dst, flags, wsum);
+        else if (from_csr)
             k_validate_csr<<<grid_for(std::max<int64_t>(m, n)), kBlock, 0, b.st>>>(n, m, d_ro, d_dst, d_w, flags);
         else if (m > 0)
             k_validate_coo<<<grid_for(m), kBlock, 0, b.st>>>(m, n, d_src, d_dst, d_w, flags);
-        if (from_csr || m > 0) count_launch();
+        if (!coo_group && (from_csr || m > 0)) count_launch();
         b.check(cudaGetLastError(), "validate");
         int hf = 0;
         b.check(cudaMemcpyAsync(&hf, flags, sizeof(int), cudaMemcpyDeviceToHost, b.st), "copy");
+        if (coo_group)
+            b.check(cudaMemcpyAsync(&weights, wsum, sizeof(weights), cudaMemcpyDeviceToHost, b.st), "copy");
         b.check(cudaStreamSynchronize(b.st), "sync");
         if (b.status == FG_OK && hf) {
             if (hf & kBadOffsets) { b.status = FG_ERR_INVALID_ARG; b.msg = "row offsets are not a valid CSR (row_off[0]=0, non-decreasing, row_off[n]=m)"; }
@@ -692,14 +854,19 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
     uint32_t *indeg = nullptr;     // in-degrees by internal id
     int32_t *t_csrc = nullptr;
     uint32_t *t_ro32 = nullptr;
+    if (coo_group && !(create_flags & FG_GRAPH_LAZY)) group_pass1(b, by_dst, m, d_dst, d_src, nullptr, false, 0);
     if (b.status == FG_OK && !(create_flags & FG_GRAPH_KEEP_IDS)) {
         indeg = b.alloc_tmp<uint32_t>(n);
         unsigned long long *bins = b.alloc_tmp<unsigned long long>(2 * kDegBins);
         unsigned long long hb[2 * kDegBins] = {};
         if (b.status == FG_OK) {
-            b.check(cudaMemsetAsync(indeg, 0, (size_t)n * sizeof(uint32_t), b.st), "memset");
             b.check(cudaMemsetAsync(bins, 0, sizeof(hb), b.st), "memset");
-            if (m > 0) { k_histogram<<<grid_for(m), kBlock, 0, b.st>>>(m, d_dst, indeg); count_launch(); }
+            if (by_dst.ready)   // counted by vertex in id order
+                b.check(cudaMemcpyAsync(indeg, by_dst.count, (size_t)n * sizeof(uint32_t), cudaMemcpyDeviceToDevice,
+                                        b.st), "copy");
+            else
+                b.check(cudaMemsetAsync(indeg, 0, (size_t)n * sizeof(uint32_t), b.st), "memset");
+            if (m > 0 && !by_dst.ready) { k_histogram<<<grid_for(m), kBlock, 0, b.st>>>(m, d_dst, indeg); count_launch(); }
             k_degree_bins<false><<<grid_for(n), kBlock, 0, b.st>>>(n, indeg, bins, bins + kDegBins);
             count_launch();
             b.check(cudaMemcpyAsync(hb, bins, sizeof(hb), cudaMemcpyDeviceToHost, b.st), "copy");
@@ -707,6 +874,12 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
         }
         if (bins) cudaFreeAsync(bins, b.st);
         if (b.status == FG_OK) g->info.in_degree_gini = (float)gini_of_bins(hb, hb + kDegBins);
+    }
+    if (by_dst.ready && !indeg) {
+        indeg = b.alloc_tmp<uint32_t>(n);
+        if (b.status == FG_OK)
+            b.check(cudaMemcpyAsync(indeg, by_dst.count, (size_t)n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, b.st),
+                    "copy");
     }
     const bool relabel = b.status == FG_OK && indeg &&
                          ((create_flags & FG_GRAPH_RELABEL) || g->info.in_degree_gini > kRelabelGini);
@@ -733,8 +906,12 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
                 k_offsets_to_u32<<<grid_for((int64_t)n + 1), kBlock, 0, b.st>>>(n, d_ro, t_ro32);
                 count_launch();
                 if (m > 0) {
-                    k_src_from_rows<<<grid_for((int64_t)n * 32), kBlock, 0, b.st>>>(n, t_ro32, t_csrc);
+                    k_row_sources<<<row_grid(m), kBlock, 0, b.st>>>(n, m, t_ro32, t_csrc);
                     count_launch();
+                    if (group) {
+                        group_alloc(b, by_src, n, 0);
+                        group_hist<false>(b, n, m, t_csrc, nullptr, nullptr, by_src, nullptr, nullptr, nullptr);
+                    }
                 }
                 d_src = t_csrc;
                 from_csr = false;   // built as a COO from here on
@@ -766,8 +943,18 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
         } else {
             uint32_t *cnt = b.alloc_tmp<uint32_t>(n);
             uint32_t *cursor = b.alloc_tmp<uint32_t>((int64_t)n + 1);
-            uint32_t *cnt_o = g->new_of ? b.alloc_tmp<uint32_t>(n) : nullptr;
-            if (b.status == FG_OK && g->new_of) {   // counted and scattered by original source id
+            uint32_t *cnt_o = g->new_of && !group ? b.alloc_tmp<uint32_t>(n) : nullptr;
+            if (group) {
+                group_pass1(b, by_src, m, d_src, d_dst, d_w, true, 0);
+                if (b.status == FG_OK) {
+                    k_part_degrees<<<grid_for(n), kBlock, 0, b.st>>>(n, by_src.count, 0, g->new_of, cnt);
+                    count_launch();
+                    b.check(exclusive_scan(cnt, ro, n, b.st), "scan");
+                    k_part_cursors<<<grid_for(n), kBlock, 0, b.st>>>(n, by_src.count, 0, ro, nullptr, g->new_of);
+                    count_launch();
+                    group_pass2(b, by_src, m, g->new_of, col, wt);
+                }
+            } else if (b.status == FG_OK && g->new_of) {   // counted and scattered by original source id
                 b.check(cudaMemsetAsync(cnt_o, 0, (size_t)n * sizeof(uint32_t), b.st), "memset");
                 if (m > 0) { k_histogram<<<grid_for(m), kBlock, 0, b.st>>>(m, d_src, cnt_o); count_launch(); }
                 k_permute_u32<<<grid_for(n), kBlock, 0, b.st>>>(n, cnt_o, g->new_of, cnt);
@@ -808,8 +995,11 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
     g->info.n_isolated = -1;
     if (!(create_flags & FG_GRAPH_LAZY)) {
         build_src(b, v);
-        build_sym(b, g, indeg);
+        build_sym(b, g, indeg, &by_dst);
     }
+    group_free(b, by_src);
+    group_free(b, by_dst);
+    if (wsum) cudaFreeAsync(wsum, b.st);
 
     if (indeg) cudaFreeAsync(indeg, b.st);
     if (t_csrc) cudaFreeAsync(t_csrc, b.st);
@@ -832,7 +1022,7 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
         unsigned long long *d_sum = nullptr, h[1 + 2 * kDegBins] = {};
         cudaError_t e = cudaMalloc(&d_sum, sizeof(h));
         if (e == cudaSuccess) e = cudaMemset(d_sum, 0, sizeof(h));
-        if (e == cudaSuccess && m > 0) {
+        if (e == cudaSuccess && m > 0 && !coo_group) {
             k_weight_sum<<<grid_for(m), kBlock>>>(m, v.w, d_sum);
             count_launch();
         }
@@ -847,6 +1037,7 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
             delete g;
             return cuda_fail(e, "graph statistics");
         }
+        if (coo_group) h[0] = w ? weights : (unsigned long long)m;
         if (m > 0) g->w_mean = (double)h[0] / (double)m;
         g->degree_gini = gini_of_bins(h + 1, h + 1 + kDegBins);
     }
