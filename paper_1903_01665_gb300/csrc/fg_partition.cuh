@@ -25,8 +25,8 @@
 namespace fg {
 namespace {
 
-constexpr int kPartThreads = 512;
-constexpr int kPartPer = 16;                            // edges a thread
+constexpr int kPartThreads = 1024;
+constexpr int kPartPer = 8;                             // edges a thread
 constexpr int kPartTile = kPartThreads * kPartPer;      // 8192
 constexpr int kPartRankBits = 13;                       // a rank within a tile
 static_assert(kPartTile == 1 << kPartRankBits, "ranks take kPartRankBits");
@@ -278,7 +278,15 @@ __global__ void __launch_bounds__(kPartThreads) k_part_count(PartPlan p, PartSha
     const int nd = sh.sub();
     for (int d = threadIdx.x; d < nd; d += kPartThreads) cnt_s[d] = 0;
     __syncthreads();
-    for (int i = threadIdx.x; i < cnt; i += kPartThreads) atomicAdd(cnt_s + __ldg(sub + e0 + i), 1u);
+    uint32_t x[kPartPer];   // every load before the first count
+#pragma unroll
+    for (int j = 0; j < kPartPer; j++) {
+        const int i = j * kPartThreads + (int)threadIdx.x;
+        x[j] = i < cnt ? __ldg(sub + e0 + i) : 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < kPartPer; j++)
+        if (j * kPartThreads + (int)threadIdx.x < cnt) atomicAdd(cnt_s + x[j], 1u);
     __syncthreads();
     uint32_t *to = count + ((int64_t)bucket << (sh.low + sh.flag));
     for (int d = threadIdx.x; d < nd; d += kPartThreads)
@@ -374,35 +382,56 @@ __global__ void __launch_bounds__(kBlock) k_row_sources(int32_t n, int64_t m, co
     if (threadIdx.x == 0) own[0] = r0;
     // rows after r0 begin after e0; empty rows share the next one's first
     // edge, whose row is the last of them
-    for (int r = r0 + 1 + (int)threadIdx.x; r <= r1; r += kBlock)
-        atomicMax(own + (int)(__ldg(ro + r) - (uint32_t)e0), r);
+    // (a tile of a skewed graph's last rows can span 10^5 of them: eight
+    // loads in flight a thread)
+    for (int r = r0 + 1 + (int)threadIdx.x; r <= r1; r += 8 * kBlock) {
+        uint32_t at[8];
+#pragma unroll
+        for (int j = 0; j < 8; j++) at[j] = r + j * kBlock <= r1 ? __ldg(ro + r + j * kBlock) : 0u;
+#pragma unroll
+        for (int j = 0; j < 8; j++)
+            if (r + j * kBlock <= r1) atomicMax(own + (int)(at[j] - (uint32_t)e0), r + j * kBlock);
+    }
     __syncthreads();
-    int32_t x[kRowPer], top = 0;
+    // a warp's 512 marks, four consecutive ones a lane at a time
+    int32_t x[kRowPer], carry = 0;
 #pragma unroll
     for (int k = 0; k < kRowPer; k += 4) {
-        const int4 q = *reinterpret_cast<const int4 *>(own + threadIdx.x * kRowPer + k);
-        x[k] = top = max(top, q.x);
-        x[k + 1] = top = max(top, q.y);
-        x[k + 2] = top = max(top, q.z);
-        x[k + 3] = top = max(top, q.w);
-    }
-    int32_t inc = top;
+        const int4 q = reinterpret_cast<const int4 *>(own)[wid * (kRowTile / kWarps / 4) + k * 8 + lane_id()];
+        x[k] = q.x;
+        x[k + 1] = max(x[k], q.y);
+        x[k + 2] = max(x[k + 1], q.z);
+        x[k + 3] = max(x[k + 2], q.w);
+        int32_t inc = x[k + 3];
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-        if ((int)lane_id() >= o) inc = max(inc, y);
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+            if ((int)lane_id() >= o) inc = max(inc, y);
+        }
+        int32_t before = __shfl_up_sync(0xffffffffu, inc, 1);
+        before = lane_id() == 0 ? carry : max(carry, before);
+#pragma unroll
+        for (int j = 0; j < 4; j++) x[k + j] = max(x[k + j], before);
+        carry = max(carry, __shfl_sync(0xffffffffu, inc, 31));
     }
-    if (lane_id() == 31) s_max[wid] = inc;
-    int32_t before = __shfl_up_sync(0xffffffffu, inc, 1);
-    if (lane_id() == 0) before = 0;
+    if (lane_id() == 0) s_max[wid] = carry;
     __syncthreads();
+    int32_t before = 0;
     for (int w = 0; w < wid; w++) before = max(before, s_max[w]);
 #pragma unroll
-    for (int k = 0; k < kRowPer; k++) own[threadIdx.x * kRowPer + k] = max(before, x[k]);
-    __syncthreads();
-    int4 *out = reinterpret_cast<int4 *>(src + e0);
-    for (int i = threadIdx.x; i < cnt / 4; i += kBlock) out[i] = reinterpret_cast<const int4 *>(own)[i];
-    for (int i = (cnt & ~3) + (int)threadIdx.x; i < cnt; i += kBlock) src[e0 + i] = own[i];
+    for (int k = 0; k < kRowPer; k += 4) {
+        const int i = (wid * (kRowTile / kWarps / 4) + k * 8 + (int)lane_id()) * 4;
+        int32_t y[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) y[j] = max(x[k + j], before);
+        if (i + 3 < cnt) {
+            *reinterpret_cast<int4 *>(src + e0 + i) = make_int4(y[0], y[1], y[2], y[3]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+                if (i + j < cnt) src[e0 + i + j] = y[j];
+        }
+    }
 }
 
 // CTAs that cover pass 2's tiles: every bucket's last tile may be short.
