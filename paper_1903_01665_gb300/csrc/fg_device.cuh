@@ -1083,6 +1083,40 @@ struct PullMinOp {
     }
 };
 
+// The first round of the synchronous CC modes: every vertex is active and
+// labelled with its own id, so the round's result for v is the smaller of v
+// and its smallest neighbour -- a minimum over the row itself, without a
+// probe.  The symmetrised view is its own transpose, so the vertices of a
+// pull round are the sources of a push round and the values are the same.
+// On R-MAT 22 the round's 134 M probes and MINs took 0.88-0.94 ms in the
+// push and edge forms, this stream over the targets (537 MB) 0.12 ms.
+struct CcFirstOp {
+    int32_t *next;
+    int32_t *snext;
+    static constexpr bool kEarly = false;
+    static constexpr bool kWeights = false;
+
+    __device__ __forceinline__ bool skip(int32_t) const { return false; }
+    __device__ __forceinline__ int32_t weight(uint32_t) const { return 0; }
+    __device__ __forceinline__ int32_t cand(int32_t u, int32_t, Acc &a) const { return u; }
+    __device__ __forceinline__ void finish(int32_t v, int32_t m, Acc &a) const {
+        if (m < v) {
+            stcg(next + v, m);
+            stcg(snext + v, 2);
+            a.changed++;
+            a.updates++;
+        }
+    }
+    __device__ __forceinline__ void finish_part(int32_t v, int32_t m, bool, Acc &a) const {
+        if (m < v) {
+            red_min(next + v, m);
+            stcg(snext + v, 2);
+            a.changed++;
+            a.updates++;
+        }
+    }
+};
+
 // BFS bottom-up step (level lev): an unvisited vertex joins level lev+1 when
 // some in-neighbour is at level lev; its scan stops at the first one.
 struct BfsPullOp {
@@ -2153,7 +2187,11 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
                                  (MODE == kVertexSync && growing);
                 ch_before = ch_prev;
                 SyncOp<ALGO> op{g.w, cur, next, scur, snext, r, dense_prev};
-                if (pull) {
+                if (ALGO == kCC && r == 1) {   // the modes' counts of a round over every edge
+                    pull_vertices(t, g, CcFirstOp{next, snext}, a);
+                    if (!pull) a.edges += a.pulled, a.pulled = 0;
+                    if (tid == 0 && !pull) a.verts += (uint32_t)g.n_nz;
+                } else if (pull) {
                     pull_vertices(t, p.tv, PullMinOp<ALGO>{p.tv.w, cur, next, snext, r}, a);
                 } else if constexpr (MODE == kVertexSync || MODE == kPull) {
                     expand_vertices(t, g.row_off, g.col, g.low, 0, g.mid, g.n_mid, g.high, g.n_high_chunks, op,
