@@ -45,7 +45,13 @@
  *                   processed first; the others wait in a far list, and when
  *                   the near worklist runs empty T moves to the far list's
  *                   smallest distance + delta and the far list is split.
- *                   BFS and CC run as FG_VERTEX_ASYNC.
+ *                   BFS and CC run as FG_VERTEX_ASYNC.  On a renumbered graph
+ *                   (FG_GRAPH_RELABEL below) whose weights allow it, the rows
+ *                   hold their light edges first: those are relaxed until no
+ *                   vertex below T changes, then the heavy ones of the
+ *                   vertices that did, each once; T moves on when that
+ *                   lowers nothing below it, and the last quarter of the edges
+ *                   runs without a threshold.
  *
  * All reach the same unique fixpoint, so their outputs are identical.
  *
@@ -220,8 +226,9 @@ fg_status fg_cc(const fg_graph *g, int32_t *label_out, fg_mode mode);
  * R-MAT, grid and uniform random graphs of 2^10 to 2^24 vertices (deep = more
  * than 32 levels, skewed = Gini above 0.5):
  *   SSSP  deep: FG_BUCKET from 2^21 vertices, else FG_VERTEX_SYNC;
- *         shallow: FG_EDGE_ASYNC if skewed or from 2^19 vertices, else
- *         FG_EDGE_SYNC;
+ *         shallow: FG_BUCKET from 2^17 vertices if the rows are split into
+ *         light and heavy edges, else FG_EDGE_ASYNC if skewed or from 2^19
+ *         vertices, else FG_EDGE_SYNC;
  *   BFS   deep: FG_BUCKET from 2^21 vertices, else FG_VERTEX_SYNC;
  *         shallow: FG_PULL if skewed, else FG_VERTEX_SYNC;
  *   CC    deep: FG_PULL below 2^23 vertices, else FG_VERTEX_SYNC;
@@ -249,7 +256,7 @@ fg_status fg_select_mode(const fg_graph *g, fg_algo algo, fg_mode *out);
 /* Options and statistics of fg_run.  Zero-initialised options mean defaults. */
 typedef struct {
     void *stream;               /* cudaStream_t to run on; NULL = legacy default stream */
-    int32_t max_rounds;         /* round / generation cap; 0 = n + 2 */
+    int32_t max_rounds;         /* round / generation cap; 0 = n + 2 (FG_BUCKET on split rows: 8 n + 64) */
     int32_t wait_timeout_ms;    /* bound on any single device-side wait; 0 = 1000 ms */
     int32_t blocks_per_sm;      /* persistent CTAs per SM; 0 = occupancy limit */
     int32_t inject_missing_arrival; /* testing aid for failure detection: if nonzero, CTA 0
@@ -263,14 +270,16 @@ typedef struct {
                                    round_trace_cap entries; NULL = no tracing */
     int32_t round_trace_cap;
     int32_t delta;              /* FG_BUCKET and fg_run_multi SSSP: bucket width (0 = 5 x the mean edge weight x the
-                                   mean out-degree) */
+                                   mean out-degree; FG_BUCKET on split rows: the bound between light and heavy
+                                   edges, twice the mean weight over the mean out-degree) */
 } fg_options;
 
 typedef struct {
     int32_t mode;               /* mode that ran (FG_AUTO resolved) */
     int32_t rounds;             /* sync rounds or async worklist generations, final
                                    no-change round included (FG_BUCKET: far-list splits
-                                   included; max_rounds counts the other generations) */
+                                   included; max_rounds counts the other generations,
+                                   light and heavy ones alike) */
     int32_t jump_passes;        /* CC pointer-jumping passes */
     int32_t grid_blocks;        /* persistent CTAs launched */
     int64_t vertices_processed; /* active vertices expanded, summed over rounds

@@ -55,28 +55,29 @@ __global__ void __launch_bounds__(kBlock, min_blocks<MODE>()) batch_kernel(Batch
 
 using BatchFn = void (*)(BatchArgs);
 
-// kind = algo * 8 + mode
+// kind = algo * 16 + mode
 BatchFn batch_kernel_for(int kind) {
     switch (kind) {
-        case kSSSP * 8 + kVertexSync: return batch_kernel<kSSSP, kVertexSync>;
-        case kSSSP * 8 + kVertexAsync: return batch_kernel<kSSSP, kVertexAsync>;
-        case kSSSP * 8 + kEdgeSync: return batch_kernel<kSSSP, kEdgeSync>;
-        case kSSSP * 8 + kEdgeAsync: return batch_kernel<kSSSP, kEdgeAsync>;
-        case kBFS * 8 + kVertexSync: return batch_kernel<kBFS, kVertexSync>;
-        case kBFS * 8 + kVertexAsync: return batch_kernel<kBFS, kVertexAsync>;
-        case kBFS * 8 + kEdgeSync: return batch_kernel<kBFS, kEdgeSync>;
-        case kBFS * 8 + kEdgeAsync: return batch_kernel<kBFS, kEdgeAsync>;
-        case kCC * 8 + kVertexSync: return batch_kernel<kCC, kVertexSync>;
-        case kCC * 8 + kVertexAsync: return batch_kernel<kCC, kVertexAsync>;
-        case kCC * 8 + kEdgeSync: return batch_kernel<kCC, kEdgeSync>;
-        case kCC * 8 + kEdgeAsync: return batch_kernel<kCC, kEdgeAsync>;
-        case kSSSP * 8 + kPull: return batch_kernel<kSSSP, kPull>;
-        case kBFS * 8 + kPull: return batch_kernel<kBFS, kPull>;
-        case kCC * 8 + kPull: return batch_kernel<kCC, kPull>;
-        case kSSSP * 8 + kBucket: return batch_kernel<kSSSP, kBucket>;
-        case kBFS * 8 + kBucket: return batch_kernel<kBFS, kBucket>;
-        case kCC * 8 + kBucket: return batch_kernel<kCC, kBucket>;
-        case kAnyAlgo * 8 + kMulti: return batch_kernel<kAnyAlgo, kMulti>;
+        case kSSSP * 16 + kVertexSync: return batch_kernel<kSSSP, kVertexSync>;
+        case kSSSP * 16 + kVertexAsync: return batch_kernel<kSSSP, kVertexAsync>;
+        case kSSSP * 16 + kEdgeSync: return batch_kernel<kSSSP, kEdgeSync>;
+        case kSSSP * 16 + kEdgeAsync: return batch_kernel<kSSSP, kEdgeAsync>;
+        case kBFS * 16 + kVertexSync: return batch_kernel<kBFS, kVertexSync>;
+        case kBFS * 16 + kVertexAsync: return batch_kernel<kBFS, kVertexAsync>;
+        case kBFS * 16 + kEdgeSync: return batch_kernel<kBFS, kEdgeSync>;
+        case kBFS * 16 + kEdgeAsync: return batch_kernel<kBFS, kEdgeAsync>;
+        case kCC * 16 + kVertexSync: return batch_kernel<kCC, kVertexSync>;
+        case kCC * 16 + kVertexAsync: return batch_kernel<kCC, kVertexAsync>;
+        case kCC * 16 + kEdgeSync: return batch_kernel<kCC, kEdgeSync>;
+        case kCC * 16 + kEdgeAsync: return batch_kernel<kCC, kEdgeAsync>;
+        case kSSSP * 16 + kPull: return batch_kernel<kSSSP, kPull>;
+        case kBFS * 16 + kPull: return batch_kernel<kBFS, kPull>;
+        case kCC * 16 + kPull: return batch_kernel<kCC, kPull>;
+        case kSSSP * 16 + kBucket: return batch_kernel<kSSSP, kBucket>;
+        case kSSSP * 16 + kLightHeavy: return batch_kernel<kSSSP, kLightHeavy>;
+        case kBFS * 16 + kBucket: return batch_kernel<kBFS, kBucket>;
+        case kCC * 16 + kBucket: return batch_kernel<kCC, kBucket>;
+        case kAnyAlgo * 16 + kMulti: return batch_kernel<kAnyAlgo, kMulti>;
     }
     return nullptr;
 }
@@ -201,7 +202,7 @@ fg_status batch_launch(const fg_query *qs, int32_t nq, const fg_batch_options *o
             fg_status s = fg_select_mode(q.g, (fg_algo)q.algo, &m);
             if (s != FG_OK) return s;
         }
-        mode[i] = (Mode)m;
+        mode[i] = kernel_mode(q.g, (Algo)q.algo, (Mode)m);
         fg_status vs = ensure_views(q.g, (Algo)q.algo, (int)m);   // lazily built parts, transposed view
         if (vs != FG_OK) return vs;
     }
@@ -222,7 +223,7 @@ fg_status batch_launch(const fg_query *qs, int32_t nq, const fg_batch_options *o
             job.qunit[i] = u;
         }
         // every multi-source sweep, SSSP or BFS, in one kernel (one launch)
-        const int kind = un.mode == kMulti ? kAnyAlgo * 8 + kMulti : un.algo * 8 + (int)un.mode;
+        const int kind = un.mode == kMulti ? kAnyAlgo * 16 + kMulti : un.algo * 16 + (int)un.mode;
         KindPlan &kp = kinds[kind];
         kp.kind = kind;
         kp.queries.push_back(u);
@@ -339,10 +340,10 @@ fg_status batch_launch(const fg_query *qs, int32_t nq, const fg_batch_options *o
         const BatchUnit &un = units[u];
         Params &p = h_params[u];
         if (un.mode == kPull) p.tv = (un.algo == kCC) ? un.g->s : un.g->t;
-        p.delta = default_delta(un.g);
+        p.delta = un.mode == kLightHeavy ? bucket_width(un.g) : default_delta(un.g);
         p.ctrl = job.d_ctrls + u;
         p.source = un.algo == kCC ? 0 : qs[un.q[0]].src;
-        p.max_rounds = view[u]->n > INT32_MAX - 2 ? INT32_MAX : view[u]->n + 2;
+        p.max_rounds = round_cap(un.mode, view[u]->n);
         p.timeout_ns = (unsigned long long)tmo * 1000000ull;
         if (un.mode == kMulti) {
             p.ms_k = (int32_t)un.q.size();
@@ -549,7 +550,7 @@ fg_status batch_finish(BatchJob &job, fg_status *status_out, fg_stats *stats_out
             for (int i : un.q) {
                 fg_stats &s = stats_out[i];
                 s = fg_stats{};
-                s.mode = un.mode == kMulti ? -1 : (int32_t)un.mode;
+                s.mode = un.mode == kMulti ? -1 : public_mode(un.mode);
                 s.rounds = hc.rounds;
                 s.jump_passes = hc.jump_passes;
                 s.vertices_processed = (int64_t)hc.st_vertices;

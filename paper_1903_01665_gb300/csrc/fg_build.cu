@@ -197,18 +197,21 @@ __global__ void k_class_scatter(int32_t n, const uint32_t *__restrict__ indeg, i
 // cursors are indexed by original id (cursor[x] = row_off[new_of[x]]), so the
 // atomics land where they would without renumbering -- spread over the ids --
 // and not on the adjacent counters of the hubs, which renumbering puts first.
-__global__ void k_cursor_of_orig(int32_t n, const uint32_t *__restrict__ ro, const int32_t *__restrict__ new_of,
-                                 uint32_t *cursor) {
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x)
-        cursor[x] = ro[new_of[x]];
+// With a light bound (light > 0), two counters and cursors per source: the
+// edges below it, then the others.
+__global__ void k_count_sources(int64_t m, const int32_t *__restrict__ s, const int32_t *__restrict__ w, int32_t light,
+                                uint32_t *count) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x)
+        atomicAdd(&count[light ? 2 * (int64_t)s[e] + (w[e] >= light) : s[e]], 1u);
 }
 __global__ void k_scatter_coo_renum(int64_t m, const int32_t *__restrict__ s, const int32_t *__restrict__ d,
-                                    const int32_t *__restrict__ w, const int32_t *__restrict__ new_of,
+                                    const int32_t *__restrict__ w, const int32_t *__restrict__ new_of, int32_t light,
                                     uint32_t *cursor, int32_t *col, int32_t *wout) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t pos = atomicAdd(&cursor[s[e]], 1u);
+        const int32_t x = w ? w[e] : 1;
+        const uint32_t pos = atomicAdd(&cursor[light ? 2 * (int64_t)s[e] + (x >= light) : s[e]], 1u);
         col[pos] = new_of[d[e]];
-        wout[pos] = w ? w[e] : 1;
+        wout[pos] = x;
     }
 }
 
@@ -252,7 +255,8 @@ __global__ void k_part_degrees(int32_t n, const uint32_t *__restrict__ count, in
 // first edge, then (flag) its first flagged one; skip: edges that row v holds
 // already (the out-edges of the symmetrised view), from row offsets.
 __global__ void k_part_cursors(int32_t n, uint32_t *count, int flag, const uint32_t *__restrict__ ro,
-                               const uint32_t *__restrict__ skip_ro, const int32_t *__restrict__ new_of) {
+                               const uint32_t *__restrict__ skip_ro, const int32_t *__restrict__ new_of,
+                               uint32_t *split) {
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
         const int64_t v = new_of ? new_of[x] : x;
         uint32_t at = ro[v];
@@ -261,6 +265,7 @@ __global__ void k_part_cursors(int32_t n, uint32_t *count, int flag, const uint3
             const uint32_t c0 = count[2 * x];
             count[2 * x] = at;
             count[2 * x + 1] = at + c0;
+            split[v] = at + c0;
         } else {
             count[x] = at;
         }
@@ -796,7 +801,7 @@ void build_sym(Builder &b, fg_graph *g, const uint32_t *indeg = nullptr, Grouped
                     group_pass1(b, q, m, v.col, v.src, nullptr, false, 0);
                 }
                 if (b.status == FG_OK) {
-                    k_part_cursors<<<grid_for(n), kBlock, 0, b.st>>>(n, q.count, 0, sro, v.row_off, map);
+                    k_part_cursors<<<grid_for(n), kBlock, 0, b.st>>>(n, q.count, 0, sro, v.row_off, map, nullptr);
                     count_launch();
                     group_pass2(b, q, m, map, scol, nullptr);
                     k_sym_out<<<grid_for(m), kBlock, 0, b.st>>>(m, v.src, v.col, v.row_off, sro, scol);
@@ -966,6 +971,28 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
         g->info.relabelled = 1;
     }
 
+    // A renumbered graph's rows are split by weight: the edges below `light`
+    // first (the near-far SSSP relaxes them until nothing changes and the
+    // heavier ones once).  Twice the mean weight over the mean degree: on
+    // R-MAT graphs (weights U[1,1000], 16 edges a vertex: 62) a sixteenth of
+    // the edges, relaxed three times each, and 1.1 relaxations an edge in all;
+    // half of it needs a third more generations, twice of it 1.3 relaxations.
+    // Weights too alike or too small to tell light from heavy: no split.
+    bool mean_known = coo_group;
+    if (relabel && w && m > 0) {
+        if (!coo_group && b.status == FG_OK) {
+            b.check(cudaMemsetAsync(wsum, 0, sizeof(unsigned long long), b.st), "memset");
+            k_weight_sum<<<grid_for(m), kBlock, 0, b.st>>>(m, d_w, wsum);
+            count_launch();
+            b.check(cudaMemcpyAsync(&weights, wsum, sizeof(weights), cudaMemcpyDeviceToHost, b.st), "copy");
+            b.check(cudaStreamSynchronize(b.st), "weight sum");
+            mean_known = true;
+        }
+        const double l = 2.0 * ((double)weights / (double)m) / std::max(1.0, (double)m / (double)n);
+        if (b.status == FG_OK && l >= 2.0) g->light = l < (double)(kInf / 2) ? (int32_t)(l + 0.5) : kInf / 2;
+    }
+    const int flag = g->light > 0 ? 1 : 0;
+    uint32_t *split = flag ? b.alloc_graph<uint32_t>(n) : nullptr;
     View &v = g->g;
     v.n = n;
     v.m = m;
@@ -984,28 +1011,33 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
         } else {
             uint32_t *cnt = b.alloc_tmp<uint32_t>(n);
             uint32_t *cursor = b.alloc_tmp<uint32_t>((int64_t)n + 1);
-            uint32_t *cnt_o = g->new_of && !group ? b.alloc_tmp<uint32_t>(n) : nullptr;
+            uint32_t *cnt_o = g->new_of && !group ? b.alloc_tmp<uint32_t>((int64_t)n << flag) : nullptr;
             if (group) {
-                group_pass1(b, by_src, m, d_src, d_dst, d_w, true, 0);
+                by_src.sh.flag = flag;
+                group_pass1(b, by_src, m, d_src, d_dst, d_w, true, g->light);
                 if (b.status == FG_OK) {
-                    k_part_degrees<<<grid_for(n), kBlock, 0, b.st>>>(n, by_src.count, 0, g->new_of, cnt);
+                    k_part_degrees<<<grid_for(n), kBlock, 0, b.st>>>(n, by_src.count, flag, g->new_of, cnt);
                     count_launch();
                     b.check(exclusive_scan(cnt, ro, n, b.st), "scan");
-                    k_part_cursors<<<grid_for(n), kBlock, 0, b.st>>>(n, by_src.count, 0, ro, nullptr, g->new_of);
+                    k_part_cursors<<<grid_for(n), kBlock, 0, b.st>>>(n, by_src.count, flag, ro, nullptr, g->new_of,
+                                                                     split);
                     count_launch();
                     group_pass2(b, by_src, m, g->new_of, col, wt);
                 }
             } else if (b.status == FG_OK && g->new_of) {   // counted and scattered by original source id
-                b.check(cudaMemsetAsync(cnt_o, 0, (size_t)n * sizeof(uint32_t), b.st), "memset");
-                if (m > 0) { k_histogram<<<grid_for(m), kBlock, 0, b.st>>>(m, d_src, cnt_o); count_launch(); }
-                k_permute_u32<<<grid_for(n), kBlock, 0, b.st>>>(n, cnt_o, g->new_of, cnt);
+                b.check(cudaMemsetAsync(cnt_o, 0, ((size_t)n << flag) * sizeof(uint32_t), b.st), "memset");
+                if (m > 0) {
+                    k_count_sources<<<grid_for(m), kBlock, 0, b.st>>>(m, d_src, d_w, g->light, cnt_o);
+                    count_launch();
+                }
+                k_part_degrees<<<grid_for(n), kBlock, 0, b.st>>>(n, cnt_o, flag, g->new_of, cnt);
                 count_launch();
                 b.check(exclusive_scan(cnt, ro, n, b.st), "scan");
-                k_cursor_of_orig<<<grid_for(n), kBlock, 0, b.st>>>(n, ro, g->new_of, cursor);
+                k_part_cursors<<<grid_for(n), kBlock, 0, b.st>>>(n, cnt_o, flag, ro, nullptr, g->new_of, split);
                 count_launch();
                 if (m > 0) {
-                    k_scatter_coo_renum<<<grid_for(m), kBlock, 0, b.st>>>(m, d_src, d_dst, d_w, g->new_of, cursor,
-                                                                          col, wt);
+                    k_scatter_coo_renum<<<grid_for(m), kBlock, 0, b.st>>>(m, d_src, d_dst, d_w, g->new_of, g->light,
+                                                                          cnt_o, col, wt);
                     count_launch();
                 }
                 b.check(cudaGetLastError(), "scatter");
@@ -1030,6 +1062,7 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
     v.col = col;
     v.w = wt;
     v.src = nullptr;
+    v.split = split;
     if (b.status == FG_OK) make_buckets(b, v);
     g->s.n = n;
     g->s.m = 2 * m;
@@ -1063,7 +1096,7 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
         unsigned long long *d_sum = nullptr, h[1 + 2 * kDegBins] = {};
         cudaError_t e = cudaMalloc(&d_sum, sizeof(h));
         if (e == cudaSuccess) e = cudaMemset(d_sum, 0, sizeof(h));
-        if (e == cudaSuccess && m > 0 && !coo_group) {
+        if (e == cudaSuccess && m > 0 && !mean_known) {
             k_weight_sum<<<grid_for(m), kBlock>>>(m, v.w, d_sum);
             count_launch();
         }
@@ -1078,7 +1111,7 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
             delete g;
             return cuda_fail(e, "graph statistics");
         }
-        if (coo_group) h[0] = w ? weights : (unsigned long long)m;
+        if (mean_known) h[0] = w ? weights : (unsigned long long)m;
         if (m > 0) g->w_mean = (double)h[0] / (double)m;
         g->degree_gini = gini_of_bins(h + 1, h + 1 + kDegBins);
     }

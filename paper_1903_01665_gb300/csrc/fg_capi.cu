@@ -251,6 +251,9 @@ fg_status fg_sweep(const fg_graph *g, fg_mode mode, const int32_t *cur, int32_t 
 // and the bucketed worklist, and depth selects the worklists that pay on
 // long propagation.
 namespace {
+// vertices from which FG_AUTO takes the light-heavy order on split rows
+constexpr int64_t kLightHeavyMin = 1 << 17;
+
 fg_plan model_plan(const fg_graph *g, fg_algo algo, int32_t depth) {
     const int64_t n = g->info.n, m = g->info.m;
     const bool deep = depth > 32;
@@ -259,6 +262,7 @@ fg_plan model_plan(const fg_graph *g, fg_algo algo, int32_t depth) {
     int32_t bps;
     if (algo == FG_ALGO_SSSP) {
         mode = deep ? (n >= (1 << 21) ? FG_BUCKET : FG_VERTEX_SYNC)
+             : g->g.split && n >= kLightHeavyMin ? FG_BUCKET
                     : ((skew || n >= (1 << 19)) ? FG_EDGE_ASYNC : FG_EDGE_SYNC);
         bps = m <= 3000000 ? 2 : 0;
     } else if (algo == FG_ALGO_BFS) {
@@ -277,7 +281,7 @@ fg_plan model_plan(const fg_graph *g, fg_algo algo, int32_t depth) {
     fg_plan p{};
     p.mode = (int32_t)mode;
     p.blocks_per_sm = bps;
-    p.delta = (mode == FG_BUCKET && algo == FG_ALGO_SSSP) ? default_delta(g) : 0;
+    p.delta = (mode == FG_BUCKET && algo == FG_ALGO_SSSP) ? bucket_width(g) : 0;
     p.tuned = 0;
     p.depth_est = depth;
     p.degree_gini = (float)g->degree_gini;
@@ -334,7 +338,7 @@ fg_status fg_select_plan(const fg_graph *g, fg_algo algo, fg_plan *out) {
         if (g->tuned_mode[algo] >= 0) {
             p.mode = g->tuned_mode[algo];
             p.blocks_per_sm = g->tuned_bps[algo];
-            p.delta = (p.mode == FG_BUCKET && algo == FG_ALGO_SSSP) ? default_delta(g) : 0;
+            p.delta = (p.mode == FG_BUCKET && algo == FG_ALGO_SSSP) ? bucket_width(g) : 0;
             p.tuned = 1;
         }
     }

@@ -27,6 +27,7 @@
 #pragma once
 
 #include <algorithm>
+#include <type_traits>
 
 #include "fg_internal.cuh"
 
@@ -131,6 +132,9 @@ __device__ __forceinline__ T block_sum(T x) {
 //   probe(v)        -- the target's current value, to compare against
 //   commit(v, c, pv, a) -- apply a candidate; true if v must be appended to
 //                      the worklist.
+// and optionally, before the probe,
+//   coarse(v)       -- a word of a denser array that may already rule v out,
+//   passes(x, v, c) -- whether candidate c needs the probe, given that word.
 // Splitting a relaxation into cand / probe / commit lets the expansions
 // issue the loads of several edges before using any of them.
 
@@ -443,6 +447,23 @@ struct SweepOp {
     }
 };
 
+template <class OP, class = void>
+struct has_coarse : std::false_type {};
+template <class OP>
+struct has_coarse<OP, std::void_t<decltype(&OP::coarse)>> : std::true_type {};
+// drops the edges that the coarse array rules out
+template <class OP, int N>
+__device__ __forceinline__ void coarse_filter(const OP &op, const int32_t (&v)[N], const int32_t (&c)[N],
+                                              bool (&ok)[N]) {
+    if constexpr (has_coarse<OP>::value) {
+        int32_t x[N];
+#pragma unroll
+        for (int j = 0; j < N; j++) x[j] = ok[j] ? op.coarse(v[j]) : 0;
+#pragma unroll
+        for (int j = 0; j < N; j++) ok[j] = ok[j] && op.passes(x[j], v[j], c[j]);
+    }
+}
+
 // ================================================================ appenders
 struct NoPush {
     __device__ __forceinline__ void operator()(bool, int32_t, Acc &) const {}
@@ -635,6 +656,7 @@ __device__ __forceinline__ void relax_batch(const int32_t *__restrict__ col, con
             ok[j] = op.cand(val[j], e[j], c[j], a);
         }
     }
+    coarse_filter(op, v, c, ok);
 #pragma unroll
     for (int j = 0; j < N; j++) pv[j] = ok[j] ? op.probe(v[j]) : 0;
     bool want[N];
@@ -1854,6 +1876,12 @@ __device__ __forceinline__ void stream_edges_async(const Team &t, const View &g,
 #ifndef FG_MULTI_MIN_BLOCKS
 #define FG_MULTI_MIN_BLOCKS 4
 #endif
+// the light-heavy passes keep a vertex's offsets and distance beside the edges
+// in flight: at 40 registers (6 CTAs) they spilled 670 bytes and ran R-MAT 22
+// in 1.78 ms, at 48 (5) 1.71, at 64 (4) 1.08
+#ifndef FG_LIGHT_MIN_BLOCKS
+#define FG_LIGHT_MIN_BLOCKS 4
+#endif
 template <int MODE>
 constexpr int min_blocks() {
     return MODE == kVertexSync ? FG_SYNC_MIN_BLOCKS
@@ -1861,6 +1889,7 @@ constexpr int min_blocks() {
          : MODE == kPull       ? FG_PULL_MIN_BLOCKS
          : MODE == kBucket     ? FG_BUCKET_MIN_BLOCKS
          : MODE == kMulti      ? FG_MULTI_MIN_BLOCKS
+         : MODE == kLightHeavy ? FG_LIGHT_MIN_BLOCKS
                                : FG_ASYNC_MIN_BLOCKS;
 }
 

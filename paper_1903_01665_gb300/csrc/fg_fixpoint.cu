@@ -70,7 +70,7 @@ KernelFn kernel_for(Algo algo, Mode mode) {
     FG_K(kCC, kVertexSync) FG_K(kCC, kVertexAsync) FG_K(kCC, kEdgeSync) FG_K(kCC, kEdgeAsync)
     FG_K(kSSSP, kPull) FG_K(kBFS, kPull) FG_K(kCC, kPull)
     FG_K(kSSSP, kBucket) FG_K(kBFS, kBucket) FG_K(kCC, kBucket)
-    FG_K(kSSSP, kMulti) FG_K(kBFS, kMulti)
+    FG_K(kSSSP, kMulti) FG_K(kBFS, kMulti) FG_K(kSSSP, kLightHeavy)
 #undef FG_K
     return nullptr;
 }
@@ -204,6 +204,8 @@ int64_t wl_cap_of(const View &g, Mode mode, int k) {
 // aligned.
 size_t query_workspace_bytes(const View &g, Algo algo, Mode mode) {
     const int32_t n = g.n;
+    if (mode == kLightHeavy)   // control block, distances, marks
+        return Workspace::need(1, sizeof(Ctrl)) + Workspace::need(n, 4) + Workspace::need(lh_mark_bytes(n), 1);
     if (mode == kMulti) {
         if (algo == kBFS)   // control block, reached-by masks, three frontier mask arrays
             return Workspace::need(1, sizeof(Ctrl)) + Workspace::need(msb_pad(n), 1) +
@@ -235,6 +237,11 @@ void carve_query_workspace(char *base, const View &g, Algo algo, Mode mode, Para
     const int64_t nwt = (g.m + kWTile - 1) / kWTile;
     p.g = g;
     p.ctrl = ws.take<Ctrl>(1);
+    if (mode == kLightHeavy) {
+        p.A = ws.take<int32_t>(n);
+        p.marks = ws.take<uint8_t>(lh_mark_bytes(n));
+        return;
+    }
     if (mode == kMulti) {
         if (algo == kBFS) {
             p.A = reinterpret_cast<int32_t *>(ws.take<uint8_t>(msb_pad(n)));
@@ -294,8 +301,20 @@ int32_t default_delta(const fg_graph *G) {
     return d >= (double)(kInf / 2) ? kInf / 2 : std::max(1, (int32_t)(d + 0.5));
 }
 
-fg_status run_query(const fg_graph *G, Algo algo, Mode mode, int32_t source, int32_t *out,
+int32_t bucket_width(const fg_graph *G) { return G->g.split ? G->light : default_delta(G); }
+
+// Default round cap: a round of the synchronous modes, or a worklist
+// generation, settles at least one more hop, so n + 1 suffice.  The
+// light-heavy schedule may spend a light generation and a heavy pass that
+// lower nothing on every one that does, and an epoch on a single vertex.
+int32_t round_cap(Mode mode, int32_t n) {
+    const int64_t cap = mode == kLightHeavy ? 8 * (int64_t)n + 64 : (int64_t)n + 2;
+    return cap > INT32_MAX ? INT32_MAX : (int32_t)cap;
+}
+
+fg_status run_query(const fg_graph *G, Algo algo, Mode user_mode, int32_t source, int32_t *out,
                     const fg_options *opt, fg_stats *stats) {
+    const Mode mode = kernel_mode(G, algo, user_mode);
     if (kernel_for(algo, mode)) {   // the parts of a FG_GRAPH_LAZY graph this query reads
         fg_status vs = ensure_views(G, algo, (int)mode);
         if (vs != FG_OK) return vs;
@@ -329,13 +348,13 @@ fg_status run_query(const fg_graph *G, Algo algo, Mode mode, int32_t source, int
     Params p;
     carve_query_workspace(wsbase, g, algo, mode, p);
     if (mode == kPull) p.tv = (algo == kCC) ? G->s : G->t;
-    p.delta = (opt && opt->delta > 0) ? opt->delta : default_delta(G);
+    p.delta = (opt && opt->delta > 0) ? opt->delta : mode == kLightHeavy ? bucket_width(G) : default_delta(G);
     struct {
         char *base;
     } ws{wsbase};
     p.source = source;
     set_relabel(G, p);
-    p.max_rounds = (opt && opt->max_rounds > 0) ? opt->max_rounds : (n > INT32_MAX - 2 ? INT32_MAX : n + 2);
+    p.max_rounds = (opt && opt->max_rounds > 0) ? opt->max_rounds : round_cap(mode, n);
     int tmo = (opt && opt->wait_timeout_ms > 0) ? opt->wait_timeout_ms : 1000;
     p.timeout_ns = (unsigned long long)tmo * 1000000ull;
     p.inject_missing_arrival = (opt && opt->inject_missing_arrival) ? 1 : 0;
@@ -422,7 +441,7 @@ fg_status run_query(const fg_graph *G, Algo algo, Mode mode, int32_t source, int
     cudaEventDestroy(ev1);
     cudaFreeAsync(ws.base, st);
     if (stats) {
-        stats->mode = (int32_t)mode;
+        stats->mode = public_mode(mode);
         stats->rounds = hc.rounds;
         stats->jump_passes = hc.jump_passes;
         stats->grid_blocks = grid;

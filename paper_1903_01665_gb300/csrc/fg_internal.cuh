@@ -43,6 +43,7 @@ struct View {
     const int2 *high = nullptr;         // {vertex, first edge} per 2048-edge chunk of >= 1024
     const int32_t *nz = nullptr;        // all vertices with >= 1 out-edge, ascending
     const int32_t *zero = nullptr;      // vertices with no out-edge, ascending
+    const uint32_t *split = nullptr;    // [n] first heavy edge of each row (rows of a graph with a light bound), else null
     const uint8_t *vclass = nullptr;    // per vertex: 0 no out-edge, 1 low, 2 mid, 3 high
     int32_t n_low = 0, n_mid = 0, n_high = 0, n_high_chunks = 0, n_nz = 0, n_zero = 0;
     int32_t max_deg = 0;
@@ -62,6 +63,7 @@ struct fg_graph {
     // lazily computed diameter estimate and autotuned modes for fg_select_mode
     mutable std::mutex mu;
     mutable int32_t diam_est = -1;
+    int32_t light = 0;          // edges below this weight come first in their row (0: rows are not split)
     double w_mean = 1.0;        // mean edge weight (bucket mode's default width)
     double degree_gini = 0.0;   // Gini coefficient of the out-degrees (the selection model's skew)
     // renumbered vertices (by in-degree class), else null: every view holds
@@ -105,7 +107,14 @@ enum Algo { kSSSP = 0, kBFS = 1, kCC = 2, kAnyAlgo = 3 };
 // kMulti: the multi-source sweep (up to 8 SSSP or BFS sources on one graph in
 // one fixpoint); not a public fg_mode, it is reached through fg_run_multi
 // and the fusion of same-graph queries in batches and the server
-enum Mode { kVertexSync = 0, kVertexAsync = 1, kEdgeSync = 2, kEdgeAsync = 3, kPull = 5, kBucket = 6, kMulti = 7 };
+// kLightHeavy: FG_BUCKET SSSP on a graph whose rows are split by weight
+enum Mode { kVertexSync = 0, kVertexAsync = 1, kEdgeSync = 2, kEdgeAsync = 3, kPull = 5, kBucket = 6, kMulti = 7,
+            kLightHeavy = 8 };
+// the kernel that runs a public mode on a graph, and back
+inline Mode kernel_mode(const fg_graph *g, Algo algo, Mode m) {
+    return m == kBucket && algo == kSSSP && g->g.split ? kLightHeavy : m;
+}
+inline int32_t public_mode(Mode m) { return m == kLightHeavy ? (int32_t)kBucket : (int32_t)m; }
 
 // worklist classes (vertex-async): low, mid, high chunks; edge-async uses class 0 only
 enum { kWlLow = 0, kWlMid = 1, kWlHigh = 2 };
@@ -122,6 +131,7 @@ struct Params {
     uint32_t *lb_off[2] = {};   // edge-async: global edge offset of each worklist item, by parity
     int32_t *eflag = nullptr;   // edge-sync sparse rounds: round stamp per 128-edge warp tile
     uint32_t *vis = nullptr;    // BFS: visited bitmap, bit v set once v has a level
+    uint8_t *marks = nullptr;   // light-heavy: three near and two heavy mark arrays
     int32_t *far[2] = {};       // bucket mode: far lists by epoch parity
     int32_t *far_mark = nullptr; // bucket mode: epoch in whose far list a vertex is
     int32_t far_cap = 0;
@@ -481,6 +491,8 @@ fg_status ensure_src(const fg_graph *g);
 
 // queries (fg_fixpoint.cu)
 int32_t default_delta(const fg_graph *G);
+int32_t bucket_width(const fg_graph *G);   // FG_BUCKET SSSP's default width
+int32_t round_cap(Mode mode, int32_t n);   // default cap on rounds
 // renumbered graphs: an internal-order result to an output in original order
 // (device or host; CC: labels to minimum original ids).  The caller has
 // checked the result; res is left unchanged.

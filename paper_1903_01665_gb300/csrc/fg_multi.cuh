@@ -25,7 +25,7 @@
 // no per-source distances, only which sources have reached a vertex.
 #pragma once
 
-#include "fg_device.cuh"
+#include "fg_light.cuh"
 
 namespace fg {
 namespace {
@@ -808,7 +808,9 @@ __device__ __forceinline__ void multi_bfs_body(const Params &p, const Team &t) {
 // A query of either kind, as the kernels run it.
 template <int ALGO, int MODE>
 __device__ __forceinline__ void query_body(const Params &p, const Team &t, uint32_t &ring_used) {
-    if constexpr (MODE == kMulti) {
+    if constexpr (MODE == kLightHeavy) {
+        light_heavy_body(p, t);
+    } else if constexpr (MODE == kMulti) {
         if constexpr (ALGO == kAnyAlgo) {
             if (p.ms_bfs) multi_bfs_body(p, t);
             else multi_body<kSSSP>(p, t);
