@@ -24,7 +24,7 @@
 //                      When the vertices not below T hold less than a quarter
 //                      of the edges, the rest runs as one phase over all
 //                      their edges without a threshold.
-// R-MAT 22: 1.1 relaxations per edge in about 28 generations, 0.99 ms, against
+// R-MAT 22: 1.1 relaxations per edge in about 28 generations, 0.91 ms, against
 // 4.0 in 17 and 2.10 ms of the dense edge-async form (R-MAT 18 0.26 against
 // 0.40 ms, R-MAT 16 0.22 against 0.32).  It is bound by latency: 0.26 ms are
 // the one large heavy pass, a third the ten light generations that carry
@@ -69,11 +69,12 @@ struct LhOp {
         c = (int32_t)x;
         return true;
     }
-    // an L1 copy is never below the current distance; what it lets through is
-    // checked against L2
+    // an L1 copy is never below the current distance; what an old one lets
+    // through costs a MIN without effect and perhaps a mark too many, less
+    // than checking each against L2 first (R-MAT 22: 0.99 -> 0.91 ms)
     __device__ __forceinline__ int32_t probe(int32_t v) const { return ldca(D + v); }
     __device__ __forceinline__ bool commit(int32_t v, int32_t c, int32_t pv, Acc &a) const {
-        if (c < pv && c < ldcg(D + v)) {
+        if (c < pv) {
             red_min(D + v, c);
             a.updates++;
             if (c < T) {
