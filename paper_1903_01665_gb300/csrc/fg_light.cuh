@@ -122,15 +122,26 @@ __device__ __forceinline__ void lh_edges(const View &g, int32_t v, uint32_t &b, 
 // tests a vertex, all at once, and handed on: loaded per vertex by the warp
 // that expands it, the dependent loads made a light generation of 100 K
 // vertices take 100 us.
+// The compacted vertices' first edge, edge count and distance, per warp or (high
+// class) of the CTA.  One set for all phases: an instantiation each took 24 KB
+// more of what is L1 otherwise.
+struct LhMem {
+    uint32_t rb[kWarps][128], d[kWarps][128];
+    int32_t v[kWarps][128];
+    int n;
+};
+__device__ __forceinline__ LhMem &lh_mem() {
+    __shared__ LhMem m;
+    return m;
+}
+
 template <int PHASE, class OP>
 __device__ __forceinline__ void lh_pass(const Team &t, const View &g, const uint8_t *marks, uint8_t *heavy, bool first,
                                         int32_t T_old, const OP &op, Acc &a) {
-    // the compacted vertices' first edge, edge count and distance: per warp,
-    // or (high class) of the CTA
-    __shared__ uint32_t s_rb[kWarps][128];
-    __shared__ uint32_t s_d[kWarps][128];
-    __shared__ int32_t s_v[kWarps][128];
-    __shared__ int s_n;
+    auto &s_rb = lh_mem().rb;
+    auto &s_d = lh_mem().d;
+    auto &s_v = lh_mem().v;
+    int &s_n = lh_mem().n;
     const unsigned lane = lane_id();
     const int wid = threadIdx.x >> 5;
     const int32_t T = op.T;
