@@ -726,13 +726,21 @@ __device__ __forceinline__ int scan_step(int64_t n, int64_t nw) {
 // compacts the active vertices with 1..31 out-edges into shared memory, and
 // relaxes their edges 32 rows at a time.  Mid and high vertices are expanded
 // from their bucket lists; vertices without out-edges have nothing to expand.
+struct LowMem {   // of either form: a warp's gathered rows
+    uint32_t rb[kWarps][128], d[kWarps][128];
+    int32_t v[kWarps][128];
+};
+__device__ __forceinline__ LowMem &low_mem() {
+    __shared__ LowMem m;
+    return m;
+}
 template <class OP>
 __device__ __forceinline__ void expand_low_dense(const Team &t, const uint32_t *__restrict__ row_off, const int32_t *__restrict__ col,
                                                  const int32_t *actw, int32_t act_val, int32_t n, const OP &op,
                                                  Acc &a) {
-    __shared__ uint32_t s_rb[kWarps][128];
-    __shared__ uint32_t s_d[kWarps][128];
-    __shared__ int32_t s_v[kWarps][128];
+    auto &s_rb = low_mem().rb;
+    auto &s_d = low_mem().d;
+    auto &s_v = low_mem().v;
     const unsigned lane = lane_id();
     const int wid = threadIdx.x >> 5;
     const int64_t gw = (t.rank * (int64_t)kBlock + threadIdx.x) >> 5;
@@ -799,6 +807,105 @@ __device__ __forceinline__ void expand_low_dense(const Team &t, const uint32_t *
         }
         __syncwarp();
     }
+}
+
+// The same for a round with few active vertices (a wavefront on a grid) on a
+// graph that takes every warp several steps: the activity words of four
+// steps are loaded at once and the vertices found are gathered over the steps
+// before their edges are relaxed, so that they share one batch and one chain
+// of dependent loads.  1023^2 grid, BFS, 912 CTAs: rounds of up to 15 K
+// vertices 11 -> 8 us, a query 1.00 -> 0.84 ms.  Dense rounds fill their
+// batches anyway.  BFS only: the SSSP and CC kernels have no registers left
+// for a second form (544 bytes of spills, R-MAT 22 SSSP 5 % slower).
+template <class OP>
+__device__ __forceinline__ void expand_low_sparse(const Team &t, const uint32_t *__restrict__ row_off, const int32_t *__restrict__ col,
+                                                 const int32_t *actw, int32_t act_val, int32_t n, const OP &op,
+                                                 Acc &a) {
+    auto &s_rb = low_mem().rb;
+    auto &s_d = low_mem().d;
+    auto &s_v = low_mem().v;
+    const unsigned lane = lane_id();
+    const int wid = threadIdx.x >> 5;
+    const int64_t gw = (t.rank * (int64_t)kBlock + threadIdx.x) >> 5;
+    const int64_t nw = (int64_t)t.size * kWarps;
+    constexpr int step = 128;
+    unsigned cnt = 0;   // vertices gathered
+    auto flush = [&]() {
+        __syncwarp();
+        for (unsigned g0 = 0; g0 < cnt; g0 += 32) {
+            const unsigned k = g0 + lane;
+            uint32_t r0 = 0, dd = 0;
+            int32_t vv = 0;
+            if (k < cnt) {
+                r0 = s_rb[wid][k];
+                dd = s_d[wid][k];
+                vv = s_v[wid][k];
+            }
+            relax_rows_of_warp(col, op, NoPush{}, r0, dd, vv, a);
+        }
+        __syncwarp();
+        cnt = 0;
+    };
+    constexpr int kAhead = 4;
+    for (int64_t q0 = gw * step; q0 < n; q0 += kAhead * nw * step) {
+        unsigned found = 0;   // bit 4 q + j: the lane's vertex j of step q is active
+#pragma unroll
+        for (int q = 0; q < kAhead; q++) {
+            const int64_t w0 = q0 + q * nw * step;
+            const int64_t v0 = w0 + 4 * lane;
+            unsigned f = 0;
+            if (v0 + 3 < n) {
+                const int4 x = __ldcg(reinterpret_cast<const int4 *>(actw + v0));
+                f = (unsigned)(x.x == act_val) | (unsigned)(x.y == act_val) << 1 | (unsigned)(x.z == act_val) << 2 |
+                    (unsigned)(x.w == act_val) << 3;
+            } else {
+                for (int j = 0; j < 4; j++)
+                    if (v0 + j < n) f |= (unsigned)(ldcg(actw + v0 + j) == act_val) << j;
+            }
+            found |= f << (4 * q);
+        }
+#pragma unroll 1
+        for (int64_t w0 = q0; w0 < min((int64_t)n, q0 + kAhead * nw * step); w0 += nw * step, found >>= 4) {
+            const int64_t v0 = w0 + 4 * lane;
+            if (lane == 0) a.scanned += min((int64_t)step, (int64_t)n - w0);
+            if (!__ballot_sync(0xffffffffu, (found & 15u) != 0)) continue;
+            bool act[4];
+            uint32_t rb[4], d[4];
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                act[j] = (found >> j) & 1u;
+                rb[j] = 0;
+                d[j] = 0;
+                if (act[j]) {
+                    rb[j] = __ldg(row_off + v0 + j);
+                    d[j] = __ldg(row_off + v0 + j + 1) - rb[j];
+                    act[j] = d[j] >= 1 && d[j] < (uint32_t)kLowMax;
+                }
+            }
+            const unsigned cnt_lane = act[0] + act[1] + act[2] + act[3];
+            if (!__ballot_sync(0xffffffffu, cnt_lane != 0)) continue;
+            const unsigned incl = warp_inclusive_scan(cnt_lane);
+            const unsigned tot = __shfl_sync(0xffffffffu, incl, 31);
+            if (cnt + tot > 128) flush();
+            unsigned slot = cnt + incl - cnt_lane;
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                if (act[j]) {
+                    int32_t val;
+                    bool rq;
+                    op.active((int32_t)(v0 + j), val, rq);
+                    op.own((int32_t)(v0 + j), val);
+                    s_rb[wid][slot] = rb[j];
+                    s_d[wid][slot] = d[j];
+                    s_v[wid][slot] = val;
+                    slot++;
+                }
+            }
+            cnt += tot;
+            if (lane == 0) a.verts += tot;
+        }
+    }
+    if (cnt) flush();
 }
 
 // ================================================================ expansions
@@ -2176,6 +2283,8 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
             if (r == 1) return ALGO != kCC;
             return (ch_prev << FG_SPARSE_SHIFT) < (int64_t)n;
         };
+        // few active vertices in a warp step of 128 ids, two steps a warp at least
+        auto few_active = [&]() -> bool { return ch_prev * 16 < (int64_t)n && (int64_t)n > 128 * (nth >> 5); };
         for (int r = 1;; r++) {
             if (r > p.max_rounds) {
                 if (tid == 0) atomicOr(&c->status, kStRoundCap);
@@ -2191,7 +2300,8 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
                 } else if constexpr (MODE == kVertexSync || MODE == kPull) {
                     expand_vertices(t, g.row_off, g.col, g.low, 0, g.mid, g.n_mid, g.high, g.n_high_chunks, op,
                                     NoPush{}, a);
-                    expand_low_dense(t, g.row_off, g.col, p.A, r - 1, n, op, a);
+                    if (few_active()) expand_low_sparse(t, g.row_off, g.col, p.A, r - 1, n, op, a);
+                    else expand_low_dense(t, g.row_off, g.col, p.A, r - 1, n, op, a);
                 } else if (sparse_round(r)) {
                     flag_edge_tiles(t, g, p.A, r - 1, n, p.eflag, r, a);
                     if (!sync_()) break;
