@@ -1284,8 +1284,36 @@ __device__ __forceinline__ void pull_vertices(const Team &t, const View &tv, con
     const int wid = threadIdx.x >> 5;
     const int64_t gw = (int64_t)t.rank * kWarps + wid, nw = (int64_t)t.size * kWarps;
 
+    // With early exit (BFS) the lists' first entries decide nearly every vertex,
+    // so each vertex's chain of loads counts, not the edges: a warp per chunk
+    // and per vertex, whole batches first, took 172 us for R-MAT 22's round of
+    // 1.6 M discoveries (26 M in-edges read); lanes trying their own vertices
+    // first take 62 us (5 M).
+    // High in-degree: a warp per 2048-edge chunk, 32 edges first.
+    if constexpr (OP::kEarly) {
+        for (int64_t ci = gw; ci < tv.n_high_chunks; ci += nw) {
+            const int2 hc = __ldg(tv.high + ci);
+            const uint32_t re = min(__ldg(tv.row_off + hc.x + 1), (uint32_t)hc.y + (uint32_t)kChunk);
+            if (__shfl_sync(0xffffffffu, lane == 0 ? (int)op.skip(hc.x) : 0, 0)) continue;
+            bool found = false;
+            for (uint32_t eb = (uint32_t)hc.y; eb < re && !found;) {
+                const bool head = eb == (uint32_t)hc.y;
+                int32_t u[kU], m = kInf;
+#pragma unroll
+                for (int j = 0; j < kU; j++)
+                    u[j] = (j == 0 || !head) && eb + 32 * j + lane < re ? ld_edge(tv.col + eb + 32 * j + lane) : -1;
+#pragma unroll
+                for (int j = 0; j < kU; j++)
+                    if (u[j] >= 0) m = min(m, op.cand(u[j], 0, a));
+                found = __any_sync(0xffffffffu, m == 0);
+                if (lane == 0) a.pulled += min(re - eb, head ? 32u : 32u * kU);
+                eb += head ? 32 : 32 * kU;
+            }
+            if (lane == 0 && found) op.finish_part(hc.x, 0, false, a);
+        }
+    }
     // high in-degree: a CTA per 2048-edge chunk
-    for (int64_t ci = t.rank; ci < tv.n_high_chunks; ci += t.size) {
+    for (int64_t ci = t.rank; !OP::kEarly && ci < tv.n_high_chunks; ci += t.size) {
         const int2 hc = __ldg(tv.high + ci);
         const int32_t v = hc.x;
         if (threadIdx.x == 0) s_skip = op.skip(v);
@@ -1313,8 +1341,57 @@ __device__ __forceinline__ void pull_vertices(const Team &t, const View &tv, con
         if (threadIdx.x == 0) op.finish_part(v, m, e0 == rb, a);
     }
 
+    // mid in-degree, with early exit: 32 vertices a warp, each lane its own
+    // vertex's first four in-neighbours (hubs come first: most end there); the
+    // others by the whole warp in turn
+    if constexpr (OP::kEarly) {
+        for (int64_t i0 = gw; i0 < tv.n_mid; i0 += nw * 32) {
+            const int64_t i = i0 + (int64_t)lane * nw;
+            int32_t v = 0;
+            uint32_t rb = 0, re = 0;
+            if (i < tv.n_mid) {
+                v = __ldg(tv.mid + i);
+                if (!op.skip(v)) {
+                    rb = __ldg(tv.row_off + v);
+                    re = __ldg(tv.row_off + v + 1);
+                }
+            }
+            bool open = rb < re;
+            if (open) {   // at least kLowMax in-edges
+                int32_t u[4], m = kInf;
+#pragma unroll
+                for (int k = 0; k < 4; k++) u[k] = __ldg(tv.col + rb + k);
+#pragma unroll
+                for (int k = 0; k < 4; k++) m = min(m, op.cand(u[k], 0, a));
+                a.pulled += 4;
+                rb += 4;
+                if (m == 0) {
+                    op.finish(v, 0, a);
+                    open = false;
+                }
+            }
+            for (unsigned bal = __ballot_sync(0xffffffffu, open); bal; bal &= bal - 1) {
+                const int l = __ffs(bal) - 1;
+                const int32_t vv = __shfl_sync(0xffffffffu, v, l);
+                const uint32_t b = __shfl_sync(0xffffffffu, rb, l), e = __shfl_sync(0xffffffffu, re, l);
+                bool found = false;
+                for (uint32_t eb = b; eb < e && !found; eb += 32 * kU) {
+                    int32_t u[kU], m = kInf;
+#pragma unroll
+                    for (int k = 0; k < kU; k++)
+                        u[k] = eb + 32 * k + lane < e ? ld_edge(tv.col + eb + 32 * k + lane) : -1;
+#pragma unroll
+                    for (int k = 0; k < kU; k++)
+                        if (u[k] >= 0) m = min(m, op.cand(u[k], 0, a));
+                    found = __any_sync(0xffffffffu, m == 0);
+                    if (lane == 0) a.pulled += min(e - eb, 32u * kU);
+                }
+                if (lane == 0 && found) op.finish(vv, 0, a);
+            }
+        }
+    }
     // mid in-degree: a warp per vertex
-    for (int64_t i = gw; i < tv.n_mid; i += nw) {
+    for (int64_t i = gw; !OP::kEarly && i < tv.n_mid; i += nw) {
         const int32_t v = __ldg(tv.mid + i);
         if (__shfl_sync(0xffffffffu, lane == 0 ? (int)op.skip(v) : 0, 0)) continue;
         const uint32_t rb = __ldg(tv.row_off + v), re = __ldg(tv.row_off + v + 1);
@@ -1332,26 +1409,59 @@ __device__ __forceinline__ void pull_vertices(const Team &t, const View &tv, con
             for (int j = 0; j < kU; j++)
                 if (u[j] >= 0) m = min(m, op.cand(u[j], wv[j], a));
             seen += 32 * kU;
-            if (OP::kEarly && __any_sync(0xffffffffu, m == 0)) break;
         }
         if (lane == 0) a.pulled += min(seen, re - rb);
         m = warp_min(m);
         if (lane == 0) op.finish(v, m, a);
     }
 
-    // low in-degree: a warp's 32 vertices, their in-edges spread over the lanes
+    // low in-degree: a warp's 32 vertices, their in-edges spread over the lanes.
+    // With early exit a lane first tries its own vertices' first two
+    // in-neighbours, two vertices at a time: most end there.
+    constexpr int kPer = OP::kEarly ? 2 : 1;
     const int64_t nl = tv.n_low;
-    for (int64_t i0 = gw * 32; i0 < nl; i0 += nw * 32) {
-        const int64_t i = i0 + lane;
-        int32_t v = -1;
-        uint32_t rb = 0, d = 0;
-        if (i < nl) {
-            v = __ldg(tv.low + i);
-            if (!op.skip(v)) {
-                rb = __ldg(tv.row_off + v);
-                d = __ldg(tv.row_off + v + 1) - rb;
+    for (int64_t i0 = gw * 32 * kPer; i0 < nl; i0 += nw * 32 * kPer) {
+        int32_t vs[kPer];
+        uint32_t rbs[kPer], ds[kPer];
+#pragma unroll
+        for (int q = 0; q < kPer; q++) {
+            const int64_t i = i0 + 32 * q + lane;
+            vs[q] = i < nl ? __ldg(tv.low + i) : -1;
+            rbs[q] = ds[q] = 0;
+        }
+#pragma unroll
+        for (int q = 0; q < kPer; q++)
+            if (vs[q] >= 0 && !op.skip(vs[q])) {
+                rbs[q] = __ldg(tv.row_off + vs[q]);
+                ds[q] = __ldg(tv.row_off + vs[q] + 1) - rbs[q];
+            }
+        if constexpr (OP::kEarly) {
+            int32_t u0[kPer], u1[kPer];
+#pragma unroll
+            for (int q = 0; q < kPer; q++) {
+                u0[q] = ds[q] > 0 ? __ldg(tv.col + rbs[q]) : -1;
+                u1[q] = ds[q] > 1 ? __ldg(tv.col + rbs[q] + 1) : u0[q];
+            }
+#pragma unroll
+            for (int q = 0; q < kPer; q++) {
+                if (u0[q] < 0) continue;
+                const int32_t c0 = op.cand(u0[q], 0, a), c1 = op.cand(u1[q], 0, a);
+                const uint32_t tried = min(ds[q], 2u);
+                a.pulled += tried;
+                if (c0 == 0 || c1 == 0) {
+                    op.finish(vs[q], 0, a);
+                    ds[q] = 0;
+                } else {
+                    rbs[q] += tried;
+                    ds[q] -= tried;
+                }
             }
         }
+#pragma unroll
+        for (int q = 0; q < kPer; q++) {
+        const int32_t v = vs[q];
+        const uint32_t rb = rbs[q], d = ds[q];
+        if (OP::kEarly && !__any_sync(0xffffffffu, d > 0)) continue;
         s_min[wid][lane] = kInf;
         __syncwarp();
         const uint32_t incl = warp_inclusive_scan(d);
@@ -1387,6 +1497,7 @@ __device__ __forceinline__ void pull_vertices(const Team &t, const View &tv, con
         __syncwarp();
         if (d > 0) op.finish(v, s_min[wid][lane], a);
         __syncwarp();
+        }
     }
 }
 
@@ -2277,6 +2388,14 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
         constexpr int kPullShift = ALGO == kBFS ? FG_PULL_SHIFT_BFS : (ALGO == kCC ? FG_PULL_SHIFT_CC : FG_PULL_SHIFT_SSSP);
         auto pull_round = [&](int r) -> bool {
             if (r == 1) return ALGO == kCC;
+            // BFS on a renumbered graph, whose in-neighbour lists begin with the
+            // hubs: pulling ends at the first few of them, so it pays from a
+            // sixteenth of the vertices on, and while the frontier explodes
+            // (the one or two per cent that a skewed graph's second or third
+            // level holds are its hubs and push half of the edges; R-MAT 22:
+            // that round 119 us pushed, 62 pulled)
+            if (ALGO == kBFS && p.new_of)
+                return (ch_prev << 4) > (int64_t)n || ((ch_prev << 7) > (int64_t)n && ch_prev > 8 * ch_before);
             return kPullShift >= 0 ? (ch_prev << kPullShift) > (int64_t)n : (ch_prev >> -kPullShift) > (int64_t)n;
         };
         auto sparse_round = [&](int r) -> bool {
@@ -2294,6 +2413,7 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
             const bool pull = (MODE == kPull) && pull_round(r);
             if (pull && tid == 0) c->pull_rounds++;
             if constexpr (ALGO == kBFS) {
+                ch_before = ch_prev;
                 BfsSyncOp op{p.A, r - 1, p.vis};
                 if (pull) {
                     pull_vertices(t, p.tv, BfsPullOp{p.A, r - 1, p.vis}, a);
