@@ -338,9 +338,13 @@ fg_status fg_run(const fg_graph *g, fg_algo algo, int32_t src, int32_t *out, fg_
  * a graph.  CC has no source: it runs once (in fg_select_mode's mode) and is
  * copied to every output.
  *
+ * On a renumbered graph with split rows (FG_BUCKET above) the light edges of
+ * all sources go first, each source below its own threshold, then the heavy
+ * ones once.
+ *
  * Options: stream, max_rounds (0 = n + 2 for BFS and CC, 2 k n + 2 for
- * SSSP, whose epochs add rounds), wait_timeout_ms, blocks_per_sm, delta (the
- * SSSP width; 0 = FG_BUCKET's default, 5 x mean weight x mean out-degree);
+ * SSSP, whose epochs add rounds, 8 k n + 64 on split rows), wait_timeout_ms,
+ * blocks_per_sm, delta (the SSSP width; 0 = FG_BUCKET's default);
  * the other fields are ignored.  status_out[k] (may be NULL) receives each
  * query's status: they differ only when some SSSP sources overflow
  * (FG_ERR_OVERFLOW for those, FG_OK and their outputs for the others).

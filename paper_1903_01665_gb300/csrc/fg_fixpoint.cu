@@ -284,9 +284,13 @@ void carve_query_workspace(char *base, const View &g, Algo algo, Mode mode, Para
 // slot).  With the near-far order (SSSP) the rounds of one epoch that lower
 // something are at most the vertex-slot pairs the epoch settles, and each
 // epoch ends with one round that lowers nothing: 2 k n + 2 bounds the sum.
-int32_t ms_default_rounds(int32_t n, int k, bool near_far) {
-    const int64_t cap = near_far ? 2 * (int64_t)k * n + 2 : (int64_t)n + 2;
+int32_t ms_default_rounds(int32_t n, int k, bool near_far, bool light) {
+    const int64_t cap = light ? 8 * (int64_t)k * n + 64 : near_far ? 2 * (int64_t)k * n + 2 : (int64_t)n + 2;
     return cap > INT32_MAX ? INT32_MAX : (int32_t)cap;
+}
+
+int32_t ms_light_width(const fg_graph *G, Algo algo, int32_t delta) {
+    return algo == kSSSP && G->g.split ? (delta > 0 ? delta : G->light) : 0;
 }
 
 // bucket mode: 5 x the mean edge weight x the mean out-degree unless the
@@ -516,13 +520,14 @@ fg_status run_multi(const fg_graph *G, Algo algo, int32_t k, const int32_t *srcs
     p.ms_bfs = algo == kBFS ? 1 : 0;
     set_relabel(G, p);
     p.delta = (opt && opt->delta > 0) ? opt->delta : default_delta(G);   // the SSSP sweep's near-far width
+    p.ms_light = ms_light_width(G, algo, opt ? opt->delta : 0);
     int32_t *dout[kMsMax] = {};
     for (int j = 0, h = 0; j < k; j++) {
         p.ms_src[j] = srcs[j];
         dout[j] = on_dev[j] ? outs[j] : reinterpret_cast<int32_t *>(base + qbytes + (size_t)(h++) * sbytes);
         p.ms_out[j] = dout[j];
     }
-    p.max_rounds = (opt && opt->max_rounds > 0) ? opt->max_rounds : ms_default_rounds(n, k, algo == kSSSP);
+    p.max_rounds = (opt && opt->max_rounds > 0) ? opt->max_rounds : ms_default_rounds(n, k, algo == kSSSP, p.ms_light > 0);
     const int tmo = (opt && opt->wait_timeout_ms > 0) ? opt->wait_timeout_ms : 1000;
     p.timeout_ns = (unsigned long long)tmo * 1000000ull;
 

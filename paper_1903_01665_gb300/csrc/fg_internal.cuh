@@ -98,6 +98,7 @@ struct Ctrl {
     int pull_rounds;            // pull mode: rounds that pulled
     int far_size[3];            // bucket mode: far-list sizes, rotating by epoch
     int far_min[3];             // bucket mode: smallest distance in each epoch's far list
+    int ms_min[3][8];           // multi-source light-heavy: each slot's smallest waiting distance, by split
     int splits;                 // bucket mode: far-list splits (threshold moves)
 };
 
@@ -142,6 +143,7 @@ struct Params {
     int32_t inject_missing_arrival = 0;
     int32_t *out = nullptr;                // batch: device output the team copies the result to
     int32_t ms_k = 0;                      // multi-source: sources in the sweep (A = rows of 8 values, S0 = stamps)
+    int32_t ms_light = 0;                  // multi-source SSSP: the light-heavy order's first width (0: plain near-far)
     int32_t ms_bfs = 0;                    // multi-source: unit weights (BFS levels)
     int32_t ms_src[8] = {};                // multi-source: source of each slot
     int32_t *ms_out[8] = {};               // multi-source: device output of each slot (null: not written)
@@ -499,7 +501,9 @@ int32_t round_cap(Mode mode, int32_t n);   // default cap on rounds
 fg_status relabel_output(const fg_graph *G, Algo algo, const int32_t *res, int32_t *out, cudaStream_t st);
 // fills the relabelling fields of a query's Params from its graph
 void set_relabel(const fg_graph *G, Params &p);
-int32_t ms_default_rounds(int32_t n, int k, bool near_far);
+int32_t ms_default_rounds(int32_t n, int k, bool near_far, bool light);
+// the width of the light-heavy order for a multi-source SSSP sweep, 0 if the graph's rows are not split
+int32_t ms_light_width(const fg_graph *G, Algo algo, int32_t delta);
 fg_status run_multi(const fg_graph *g, Algo algo, int32_t k, const int32_t *srcs, int32_t *const *outs,
                     const fg_options *opt, fg_status *status_out, fg_stats *stats);
 fg_status run_query(const fg_graph *g, Algo algo, Mode mode, int32_t source, int32_t *out,

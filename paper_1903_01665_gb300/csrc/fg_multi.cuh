@@ -164,6 +164,21 @@ __device__ __forceinline__ void ms_relax_one_source(const View &g, int32_t *D, i
     }
 }
 
+// Shared memory of the sweeps, one set for all their forms: the thresholds of
+// the light-heavy order, and the rows that a warp (or the CTA) gathered --
+// first edge, edges, vertex (or BFS frontier mask).
+struct MsLight {
+    int32_t T[kMsMax], T_old[kMsMax];
+    int32_t mn[kMsMax];
+    uint32_t rb[kWarps][128], d[kWarps][128];
+    int32_t u[kWarps][128];
+    int n;
+};
+__device__ __forceinline__ MsLight &ms_light() {
+    __shared__ __align__(16) MsLight m;
+    return m;
+}
+
 #ifndef FG_MULTI_EDGES_PER_LANE
 #define FG_MULTI_EDGES_PER_LANE 2
 #endif
@@ -177,9 +192,9 @@ __device__ __forceinline__ void ms_round(const Team &t, const View &g, int32_t *
                                          const MsNear &nf, Acc &a) {
     __shared__ int32_t s_list[kBlock];
     __shared__ int s_n;
-    __shared__ uint32_t s_rb[kWarps][128];
-    __shared__ uint32_t s_d[kWarps][128];
-    __shared__ int32_t s_u[kWarps][128];
+    auto &s_rb = ms_light().rb;
+    auto &s_d = ms_light().d;
+    auto &s_u = ms_light().u;
     const unsigned lane = lane_id();
     const int wid = threadIdx.x >> 5;
     // ---- high-degree chunks: dealt to the team's CTAs round-robin
@@ -365,6 +380,417 @@ __device__ __forceinline__ int32_t ms_far_min(const int32_t (&x)[kMsMax], int32_
     return m;
 }
 
+// ================================================================ light and heavy edges for k sources
+// On a graph whose rows are split by weight the SSSP sweep runs in the order of
+// fg_light.cuh -- light generations to a fixpoint below a threshold, one
+// heavy pass, the threshold moved -- for all sources at once: a vertex is
+// near if any slot was lowered below its own threshold.  Each slot has its own
+// (every source reaches the hubs at another distance), in shared memory,
+// written by thread 0 between barriers; a source row's slots at or above it
+// are masked on load, so the relaxation itself does not ask.  R-MAT 24, 8
+// sources: 1.69 G edge visits in 17 rounds and 17.3 ms in the plain near-far
+// order, 0.60 G in 39 and 10.0 ms in this one (R-MAT 22 4.5 -> 2.8 ms).  It is
+// bound by the rows' probes: 32 bytes of 537 MB each.  Measured and left out:
+// a bit per vertex whose slots are all settled, tested before a heavy edge's
+// row (11.0 ms: the slots settle at different times), 3 or 2 CTAs per SM
+// instead of 4 (11.7, 14.4 ms), one edge a lane (11.3 ms), the passes as
+// functions of their own (10.9 ms).
+// A source row as it is relaxed: slots at or above their threshold have no candidate.
+__device__ __forceinline__ void ml_load_source(const int32_t *row, int32_t (&x)[kMsMax], bool fresh) {
+    ms_load_row(row, x, fresh);
+    const int32_t *T = ms_light().T;
+#pragma unroll
+    for (int s = 0; s < kMsMax; s++)
+        if (x[s] >= T[s]) x[s] = kInf;
+}
+
+// Relaxes up to N edges per lane, edge j from the source row src(j).
+template <int N, class SRC>
+__device__ __forceinline__ void ml_relax(const View &g, int32_t *D, uint8_t *near, const uint32_t (&e)[N],
+                                         const bool (&in)[N], const SRC &src, Acc &a) {
+    int32_t v[N], wv[N], pv[N][kMsMax];
+#pragma unroll
+    for (int j = 0; j < N; j++) {
+        v[j] = 0;
+        wv[j] = 0;
+        if (in[j]) {
+            v[j] = ld_edge(g.col + e[j]);
+            wv[j] = ld_edge(g.w + e[j]);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < N; j++) {
+        if (in[j]) {
+            ms_load_row(D + (size_t)v[j] * kMsMax, pv[j], false);
+        } else {
+#pragma unroll
+            for (int s = 0; s < kMsMax; s++) pv[j][s] = 0;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < N; j++) {
+        if (!in[j]) continue;
+        const int32_t(&du)[kMsMax] = src(j);
+        int32_t *row = D + (size_t)v[j] * kMsMax;
+        bool lowered = false, is_near = false;
+#pragma unroll
+        for (int s = 0; s < kMsMax; s++) {
+            const uint32_t c = (uint32_t)du[s] + (uint32_t)wv[j];
+            if ((int32_t)min(c, (uint32_t)kInf) >= pv[j][s]) {
+                if (c >= (uint32_t)kInf && du[s] != kInf) a.overflow = 1;
+                continue;
+            }
+            red_min(row + s, (int32_t)c);   // c < pv <= INF
+            lowered = true;
+            is_near |= (int32_t)c < ms_light().T[s];
+        }
+        if (is_near) {
+            mark_byte(near + v[j]);
+            a.changed++;
+        }
+        a.updates += lowered;
+    }
+}
+
+template <int PHASE>
+__device__ __forceinline__ void ml_pass(const Team &t, const View &g, int32_t *D, const uint8_t *marks, uint8_t *near,
+                                        uint8_t *heavy, Acc &acc) {
+    Acc a;
+    MsLight &m = ms_light();
+    auto &s_rb = m.rb;
+    auto &s_d = m.d;
+    auto &s_u = m.u;
+    const unsigned lane = lane_id();
+    const int wid = threadIdx.x >> 5;
+    // the rows given per lane, their edges spread over the warp
+    auto relax_rows = [&](uint32_t rb, uint32_t d, int32_t u) {
+        const uint32_t inc = warp_inclusive_scan(d);
+        const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
+        const uint32_t exc = inc - d;
+        if (lane == 0) a.edges += total;
+        for (uint32_t k0 = 0; k0 < total; k0 += 32 * kMsU) {
+            uint32_t e[kMsU];
+            bool in[kMsU];
+            int32_t du[kMsU][kMsMax];
+#pragma unroll
+            for (int j = 0; j < kMsU; j++) {
+                const uint32_t x = k0 + 32 * j + lane;
+                int owner = 0;
+#pragma unroll
+                for (int step = 16; step > 0; step >>= 1) {
+                    const uint32_t pv = __shfl_sync(0xffffffffu, inc, owner + step - 1);
+                    if (pv <= x) owner += step;
+                }
+                const uint32_t ob = __shfl_sync(0xffffffffu, rb, owner);
+                const uint32_t oe = __shfl_sync(0xffffffffu, exc, owner);
+                const int32_t ou = __shfl_sync(0xffffffffu, u, owner);
+                in[j] = x < total;
+                e[j] = ob + (x - oe);
+                if (in[j]) {
+                    ml_load_source(D + (size_t)ou * kMsMax, du[j], false);
+                } else {
+#pragma unroll
+                    for (int s = 0; s < kMsMax; s++) du[j][s] = kInf;
+                }
+            }
+            ml_relax(g, D, near, e, in, [&](int j) -> const int32_t(&)[kMsMax] { return du[j]; }, a);
+        }
+    };
+    // edges [e0, e1) of u, by `lanes` threads, x the thread's place
+    auto relax_range = [&](int32_t u, uint32_t e0, uint32_t e1, int x, int lanes) {
+        int32_t du[kMsMax];
+        ml_load_source(D + (size_t)u * kMsMax, du, true);
+        for (uint32_t eb = e0; eb < e1; eb += lanes * kMsU) {
+            uint32_t e[kMsU];
+            bool in[kMsU];
+#pragma unroll
+            for (int j = 0; j < kMsU; j++) {
+                e[j] = eb + j * lanes + x;
+                in[j] = e[j] < e1;
+            }
+            ml_relax(g, D, near, e, in, [&](int) -> const int32_t(&)[kMsMax] { return du; }, a);
+        }
+    };
+    const int64_t G = t.size;
+    for (int64_t base = t.rank; base < g.n_high_chunks; base += G * kBlock) {
+        const int64_t ci = base + (int64_t)threadIdx.x * G;
+        bool act = false;
+        uint32_t b = 0, e = 0;
+        int32_t u = 0;
+        if (ci < g.n_high_chunks) {
+            const int2 hc = __ldg(g.high + ci);
+            u = hc.x;
+            if (__ldcg(marks + u)) {
+                const uint32_t cb = (uint32_t)hc.y, rb = __ldg(g.row_off + u);
+                lh_edges<PHASE>(g, u, b, e);
+                b = max(b, cb);
+                e = min(e, cb + (uint32_t)kChunk);
+                act = b < e;
+                if (cb == rb) {
+                    a.verts++;
+                    if (PHASE == kLight) mark_byte(heavy + u);
+                }
+            }
+        }
+        if (threadIdx.x == 0) m.n = 0;
+        __syncthreads();
+        const unsigned bal = __ballot_sync(0xffffffffu, act);
+        int at = 0;
+        if (lane == 0 && bal) at = atomicAdd(&m.n, __popc(bal));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(bal & lanemask_lt());
+        if (act) {
+            (&s_rb[0][0])[at] = b;
+            (&s_d[0][0])[at] = e;
+            (&s_u[0][0])[at] = u;
+            a.edges += e - b;
+        }
+        __syncthreads();
+        const int na = m.n;
+        auto small = [&](int i) { return PHASE == kLight && (&s_d[0][0])[i] - (&s_rb[0][0])[i] <= 256u; };
+        for (int i = 0; i < na; i++)
+            if (!small(i))
+                relax_range((&s_u[0][0])[i], (&s_rb[0][0])[i], (&s_d[0][0])[i], (int)threadIdx.x, kBlock);
+        if (PHASE == kLight)
+            for (int i = wid; i < na; i += kWarps)
+                if (small(i)) relax_range((&s_u[0][0])[i], (&s_rb[0][0])[i], (&s_d[0][0])[i], (int)lane, 32);
+        __syncthreads();
+    }
+    const int gw = (int)((t.rank * (unsigned)kBlock + threadIdx.x) >> 5);
+    const int nw = (int)(t.size * (unsigned)kWarps);
+    for (int base = gw; base < g.n_mid; base += nw * 32) {
+        const int i = base + (int)lane * nw;
+        uint32_t vb = 0, ve = 0;
+        int32_t u = 0;
+        bool act = false;
+        if (i < g.n_mid) {
+            u = __ldg(g.mid + i);
+            act = __ldcg(marks + u) != 0;
+            if (act) {
+                lh_edges<PHASE>(g, u, vb, ve);
+                if (PHASE == kLight) mark_byte(heavy + u);
+            }
+        }
+        unsigned bal = __ballot_sync(0xffffffffu, act);
+        if (lane == 0) a.verts += __popc(bal);
+        if (PHASE == kLight) {
+            if (bal) relax_rows(vb, ve - vb, u);
+            bal = 0;
+        }
+        while (bal) {
+            const int l = __ffs(bal) - 1;
+            bal &= bal - 1;
+            const uint32_t b = __shfl_sync(0xffffffffu, vb, l), en = __shfl_sync(0xffffffffu, ve, l);
+            if (lane == 0) a.edges += en - b;
+            relax_range(__shfl_sync(0xffffffffu, u, l), b, en, (int)lane, 32);
+        }
+    }
+    const int32_t n = g.n;
+    const int step = scan_step(n, nw);
+    unsigned cnt = 0;
+    auto flush = [&]() {
+        __syncwarp();
+        for (unsigned g0 = 0; g0 < cnt; g0 += 32) {
+            const unsigned k = g0 + lane;
+            relax_rows(k < cnt ? s_rb[wid][k] : 0u, k < cnt ? s_d[wid][k] : 0u, k < cnt ? s_u[wid][k] : 0);
+        }
+        __syncwarp();
+        cnt = 0;
+    };
+    for (int64_t q0 = (int64_t)gw * step; q0 < n; q0 += 4 * (int64_t)nw * step) {
+        uint32_t m4 = 0;   // a nibble a step: the lane's marked vertices
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const int64_t v0 = q0 + (int64_t)q * nw * step + (step == 128 ? 4 * lane : lane);
+            uint32_t x = 0;
+            if (step == 128) {
+                if (v0 < n) x = (uint32_t)__ldcg(reinterpret_cast<const int32_t *>(marks + v0));   // padded to 16
+            } else if ((int)lane < step && v0 < n) {
+                x = __ldcg(marks + v0);
+            }
+            m4 |= ((x & 1u) | ((x >> 7) & 2u) | ((x >> 14) & 4u) | ((x >> 21) & 8u)) << (4 * q);   // marks are 0 or 1
+        }
+#pragma unroll 1
+        for (int q = 0; q < 4; q++, m4 >>= 4) {
+            const int64_t w0 = q0 + (int64_t)q * nw * step;
+            if (w0 >= n) break;
+            const int64_t v0 = w0 + (step == 128 ? 4 * lane : lane);
+            if (lane == 0) a.scanned += min((int64_t)step, (int64_t)n - w0);
+            if (!__ballot_sync(0xffffffffu, (m4 & 15u) != 0)) continue;
+            bool act[4];
+            uint32_t rb[4], d[4];
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                act[j] = (m4 >> j) & 1u;
+                rb[j] = d[j] = 0;
+                if (act[j]) {
+                    const int32_t v = (int32_t)(v0 + j);
+                    const uint32_t deg = __ldg(g.row_off + v + 1) - __ldg(g.row_off + v);
+                    uint32_t e;
+                    lh_edges<PHASE>(g, v, rb[j], e);
+                    d[j] = e - rb[j];
+                    act[j] = deg >= 1 && deg < (uint32_t)kLowMax;
+                    if (act[j] && PHASE == kLight) mark_byte(heavy + v);
+                    act[j] = act[j] && d[j] > 0;
+                }
+            }
+            const unsigned cnt_lane = act[0] + act[1] + act[2] + act[3];
+            if (!__ballot_sync(0xffffffffu, cnt_lane != 0)) continue;
+            const unsigned incl = warp_inclusive_scan(cnt_lane);
+            const unsigned tot = __shfl_sync(0xffffffffu, incl, 31);
+            if (cnt + tot > 128) flush();
+            unsigned slot = cnt + incl - cnt_lane;
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                if (act[j]) {
+                    s_rb[wid][slot] = rb[j];
+                    s_d[wid][slot] = d[j];
+                    s_u[wid][slot] = (int32_t)(v0 + j);
+                    slot++;
+                }
+            }
+            cnt += tot;
+            if (lane == 0) a.verts += tot;
+        }
+    }
+    if (cnt) flush();
+    acc.edges += a.edges;
+    acc.verts += a.verts;
+    acc.updates += a.updates;
+    acc.scanned += a.scanned;
+    acc.changed += a.changed;
+    acc.overflow |= a.overflow;
+}
+
+// The generations of the light-heavy sweep, after the rows' initialisation.
+// Returns whether the fixpoint was reached.
+template <class SYNC>
+__device__ __forceinline__ bool ml_sweep(const Params &p, const Team &t, const int32_t (&msrc)[kMsMax], Acc &a,
+                                         int &rounds, int &splits, const SYNC &sync_) {
+    Ctrl *c = p.ctrl;
+    const View &g = p.g;
+    const int32_t n = g.n;
+    const int k = p.ms_k;
+    const int64_t np = lh_pad(n);
+    int32_t *D = p.A;
+    uint8_t *F = reinterpret_cast<uint8_t *>(p.S0);         // three near arrays (n int32 hold them)
+    uint8_t *H = reinterpret_cast<uint8_t *>(p.far_mark);   // two heavy ones
+    const int64_t tid = t.rank * (int64_t)kBlock + threadIdx.x;
+    const int64_t nth = (int64_t)t.size * kBlock;
+    MsLight &m = ms_light();
+    auto clear = [&](uint8_t *x, int64_t arrays) {
+        for (int64_t i = tid; i < arrays * np / 16; i += nth) reinterpret_cast<int4 *>(x)[i] = make_int4(0, 0, 0, 0);
+    };
+    clear(F, 3);
+    clear(H, 2);
+    if (tid < 3 * kMsMax) (&c->ms_min[0][0])[tid] = kInf;
+    if (threadIdx.x < kMsMax) {
+        m.T[threadIdx.x] = p.ms_light;
+        m.T_old[threadIdx.x] = 0;
+    }
+    if (!sync_()) return false;
+    if (tid == 0)
+        for (int s = 0; s < k; s++) F[np + msrc[s]] = 1;   // F[1]: the sources are near in generation 1
+    if (!sync_()) return false;
+    int phase = kLight, hp = 0, work = 0;
+    int32_t width = p.ms_light;
+    bool h_used = false;
+    for (int gen = 1;; gen++) {
+        if (work >= p.max_rounds) {
+            if (tid == 0) atomicOr(&c->status, kStRoundCap);
+            return false;
+        }
+        work++;
+        rounds++;
+        const uint8_t *cur = F + (gen % 3) * np;
+        uint8_t *next = F + ((gen + 1) % 3) * np, *heavy = H + (hp & 1) * np;
+        clear(F + ((gen + 2) % 3) * np, 1);
+        if (phase == kLight) {
+            if (h_used) clear(H + ((hp + 1) & 1) * np, 1);
+            h_used = false;
+            ml_pass<kLight>(t, g, D, cur, next, heavy, a);
+        } else if (phase == kHeavy) {
+            ml_pass<kHeavy>(t, g, D, heavy, next, nullptr, a);
+            hp++;
+            h_used = true;
+        } else {
+            ml_pass<kBoth>(t, g, D, cur, next, nullptr, a);
+        }
+        if (a.overflow) atomicOr(&c->status, kStOverflow);
+        a.overflow = 0;
+        if (!sync_(a.changed)) return false;
+        a.changed = 0;
+        if (team_total() != 0) {
+            if (phase == kHeavy) phase = kLight;
+            continue;
+        }
+        if (phase == kBoth) return true;
+        if (phase == kLight) {
+            phase = kHeavy;
+            continue;
+        }
+        // ---- split: each slot's smallest distance not below its threshold,
+        // and the edges of the vertices not below it, over all slots
+        rounds++;
+        if (threadIdx.x < kMsMax) m.mn[threadIdx.x] = kInf;
+        if (tid < kMsMax) c->ms_min[(splits + 1) % 3][tid] = kInf;
+        __syncthreads();
+        uint32_t left = 0;
+        int32_t mn[kMsMax];
+#pragma unroll
+        for (int s = 0; s < kMsMax; s++) mn[s] = kInf;
+        for (int64_t v = tid; v < n; v += nth) {
+            int32_t x[kMsMax];
+            ms_load_row(D + (size_t)v * kMsMax, x, true);
+            int open = 0;
+#pragma unroll
+            for (int s = 0; s < kMsMax; s++) {
+                const bool wait = s < k && x[s] >= m.T[s];
+                open += wait;
+                if (wait) mn[s] = min(mn[s], x[s]);
+            }
+            if (open) left += open * (__ldg(g.row_off + v + 1) - __ldg(g.row_off + v));
+        }
+#pragma unroll
+        for (int s = 0; s < kMsMax; s++) {
+            const int32_t x = warp_min(mn[s]);
+            if (lane_id() == 0 && x < kInf) atomicMin(&m.mn[s], x);
+        }
+        __syncthreads();
+        if (threadIdx.x < kMsMax && m.mn[threadIdx.x] < kInf)
+            atomicMin(&c->ms_min[splits % 3][threadIdx.x], m.mn[threadIdx.x]);
+        if (!sync_((int)(left >> 4))) return false;   // sixteenths, so that a warp's sum stays in 32 bits
+        const bool both = 64 * team_total() < (int64_t)k * g.m;
+        int32_t low = kInf;
+        __syncthreads();   // every warp has read m.T
+        if (threadIdx.x < kMsMax) {
+            const int s = threadIdx.x;
+            const int32_t x = __ldcg(&c->ms_min[splits % 3][s]);
+            m.mn[s] = x;
+            m.T_old[s] = m.T[s];
+            if (both) m.T[s] = kInf;
+            else if (x < kInf) m.T[s] = x >= kInf - width ? kInf : x + width;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int s = 0; s < kMsMax; s++) low = min(low, m.mn[s]);
+        splits++;
+        if (low >= kInf) return true;
+        phase = both ? kBoth : kLight;
+        width = width > kInf / 2 ? kInf : 2 * width;
+        // the vertices with a slot in between are near in the next generation
+        uint8_t *mark = F + ((gen + 1) % 3) * np;
+        for (int64_t v = tid; v < n; v += nth) {
+            int32_t x[kMsMax];
+            ms_load_row(D + (size_t)v * kMsMax, x, true);
+            bool now = false;
+#pragma unroll
+            for (int s = 0; s < kMsMax; s++) now |= x[s] >= m.T_old[s] && x[s] < m.T[s];
+            if (now) mark[v] = 1;
+        }
+        if (!sync_()) return false;
+    }
+}
+
 // The whole multi-source query run by one team: init, rounds until one
 // lowers nothing and no vertex is far-pending, then the rows are written out
 // per source (unless a candidate overflowed: the host then checks which
@@ -405,8 +831,10 @@ __device__ __forceinline__ void multi_body(const Params &p, const Team &t) {
         int4 *row = reinterpret_cast<int4 *>(D + (size_t)v * kMsMax);
         row[0] = make_int4(x[0], x[1], x[2], x[3]);
         row[1] = make_int4(x[4], x[5], x[6], x[7]);
-        stamp[v] = src ? 1 : 0;
-        p.far_mark[v] = 0;   // rounds start at 1
+        if (!p.ms_light) {
+            stamp[v] = src ? 1 : 0;
+            p.far_mark[v] = 0;   // rounds start at 1
+        }
     }
     if (tid == 0)
         for (int e = 0; e < 3; e++) c->far_min[e] = kInf;
@@ -418,7 +846,12 @@ __device__ __forceinline__ void multi_body(const Params &p, const Team &t) {
         s_epoch0 = 1;
         s_splits = 0;
     }
-    bool ok = sync_();
+    if (p.ms_light) {
+        int splits = 0;
+        done = ml_sweep(p, t, msrc, a, rounds, splits, sync_);
+        if (threadIdx.x == 0) s_splits = splits;
+    }
+    bool ok = !p.ms_light && sync_();
     for (int r = 1; ok; r++) {
         if (r > p.max_rounds) {
             if (tid == 0) atomicOr(&c->status, kStRoundCap);
@@ -586,9 +1019,9 @@ __device__ __forceinline__ void msb_round(const Team &t, const View &g, const Pa
                                           const uint8_t *cur, uint8_t *nxt, int32_t r, Acc &a) {
     __shared__ int32_t s_list[kBlock];
     __shared__ int s_n;
-    __shared__ uint32_t s_rb[kWarps][128];
-    __shared__ uint32_t s_d[kWarps][128];
-    __shared__ uint32_t s_f[kWarps][128];
+    auto &s_rb = ms_light().rb;
+    auto &s_d = ms_light().d;
+    auto &s_f = ms_light().u;
     const unsigned lane = lane_id();
     const int wid = threadIdx.x >> 5;
     // ---- high-degree chunks: dealt to the team's CTAs round-robin
@@ -690,7 +1123,7 @@ __device__ __forceinline__ void msb_round(const Team &t, const View &g, const Pa
             if (act[j]) {
                 s_rb[wid][slot] = rb[j];
                 s_d[wid][slot] = d[j];
-                s_f[wid][slot] = fm[j];
+                s_f[wid][slot] = (int32_t)fm[j];
                 slot++;
             }
         }
@@ -702,7 +1135,7 @@ __device__ __forceinline__ void msb_round(const Team &t, const View &g, const Pa
             if (k < tot) {
                 r0 = s_rb[wid][k];
                 dd = s_d[wid][k];
-                f0 = s_f[wid][k];
+                f0 = (uint32_t)s_f[wid][k];
             }
             const uint32_t inc = warp_inclusive_scan(dd);
             const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
