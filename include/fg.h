@@ -430,8 +430,8 @@ uint64_t fg_kernel_launches(void);
  * (algorithm, mode) kind present, the kinds running concurrently -- the
  * runtime form of the paper's barrier-free kernels on separate streams
  * (Sec. 3.2) and independent parallel sections (Sec. 3.4).  Each launch is
- * a persistent kernel split into teams of CTAs (team size from the query's
- * edge count, CTA share from its estimated work); teams pull queries from
+ * a persistent kernel split into teams of CTAs (sizes and numbers planned from
+ * a cost model for one common makespan); teams pull queries from
  * size-class queues and run each fixpoint with a team-local barrier.
  * Results are identical to fg_run's.
  */

@@ -9,8 +9,8 @@
 // Each launch is a persistent cooperative kernel whose CTAs are split into
 // teams; every team pulls units from the queue of its size class and runs
 // the whole fixpoint of each with a team-local barrier (a one-CTA team needs
-// only __syncthreads).  The team size of a unit comes from its edge count,
-// the CTA budget of each kind and class from its estimated work.  Kinds run
+// only __syncthreads).  The team sizes and their number come from a cost model
+// of the units and a makespan common to all kinds (plan_teams).  Kinds run
 // concurrently on forked streams, optionally captured in one CUDA graph.
 #include <algorithm>
 #include <map>
@@ -82,25 +82,49 @@ BatchFn batch_kernel_for(int kind) {
     return nullptr;
 }
 
-// CTAs a query's team gets: one per ~128K edges, a power of two in [1, 128].
-int team_size_for(int64_t m) {
-    int s = 1;
-    while (s < 128 && (int64_t)s * (1 << 17) < m) s <<= 1;
-    return s;
-}
-
-// relative work of a query (SSSP relaxes each edge several times)
-double work_of(int algo, const View &v) {
-    return (double)v.m * (algo == kSSSP ? 4.0 : 1.0) + (double)v.n;
-}
-
-// relative work of a unit: a fused sweep of k sources costs a fraction of k
-// separate sweeps (R-MAT 22, 8 sources: SSSP about 2x one query, BFS about 4x)
-double unit_work(const BatchUnit &u, const View &v) {
-    const double one = work_of(u.algo, v);
-    if (u.mode != kMulti) return one;
-    const double k = (double)u.q.size();
-    return one * (1.0 + (k - 1.0) * (u.algo == kSSSP ? 0.15 : 0.45));
+// The cost model of the planner: a unit on a team of p CTAs takes about
+// a + b / p ms.  a: its rounds, each a chain of dependent loads and a barrier;
+// b: the edges it visits and the vertices its rounds scan, in CTA-ms.  Fitted to
+// four-source sweeps and single queries on 152 to 608 CTAs (grids of 64^2 to
+// 1484^2, R-MAT of 2^11 to 2^20 vertices; a 1484^2 grid's SSSP: 7.6, 4.6 and
+// 3.2 ms on 152, 304 and 608 CTAs), b half as much again for the teams that
+// run beside it (a batch of 24 units: measured 1.0 to 1.6 times the fit).
+struct UnitCost {
+    double a = 0, b = 0;
+    double ms(int p) const { return a + b / p; }
+};
+UnitCost unit_cost(const BatchUnit &u, const View &v) {
+    int depth;
+    {
+        std::lock_guard<std::mutex> lk(u.g->mu);
+        depth = u.g->diam_est;   // known if a query of the graph was FG_AUTO
+    }
+    const bool skew = u.g->degree_gini > 0.5;
+    if (depth < 0) depth = skew ? 10 : 100;
+    const bool deep = depth > 32;
+    const double k = (double)u.q.size(), m = (double)v.m, n = (double)v.n;
+    double rounds, round_us, visits, visit_ns, scan;   // scan: vertices' words read per round, in int32
+    if (u.mode == kMulti) {
+        const bool sssp = u.algo == kSSSP;
+        rounds = sssp ? (deep ? 1.5 * depth : 40) : depth + 1;
+        round_us = deep ? 7 : sssp ? 20 : 12;
+        visits = m * (sssp ? (deep ? 1.2 + 2.2 * k : 2.3) : (deep ? 0.97 * k : 2.2));
+        visit_ns = deep ? (sssp ? 7.4 : 8.7) : (sssp ? 4.9 : 2.7);
+        scan = sssp ? n : n / 2;
+    } else {
+        rounds = u.algo == kSSSP ? 1.4 * depth + 12 : u.algo == kBFS ? depth + 1 : 8;
+        round_us = u.mode == kVertexSync || u.mode == kPull ? 6 : 9;
+        visits = m * (u.algo == kBFS ? 1.0 : u.algo == kCC ? 2.0 : u.mode == kLightHeavy ? 1.2
+                                                             : u.mode == kBucket         ? 2.2
+                                                             : deep                      ? 9.0
+                                                                                         : 5.0);
+        visit_ns = 3.5;
+        scan = u.mode == kVertexAsync || u.mode == kEdgeAsync || u.mode == kBucket ? 0 : n;
+    }
+    UnitCost c;
+    c.a = 1e-3 * rounds * round_us;
+    c.b = 1.5 * (1e-6 * visits * visit_ns + 6e-7 * rounds * scan);
+    return c;
 }
 
 struct KindPlan {
@@ -109,9 +133,54 @@ struct KindPlan {
     std::vector<int> class_size;              // team size per class
     std::vector<std::vector<int>> class_q;    // units per class, largest work first
     std::vector<int> class_teams;             // teams per class
-    double work = 0;
+    int capacity = 1;                         // co-resident CTAs
     int ctas = 0;
 };
+
+// Team sizes: 1, 2, 3, 4, 6, 8, 12, 16, ...
+int next_team(int p) { return p < 2 ? 2 : (p & (p - 1)) == 0 ? p + p / 2 : p / 3 * 4; }
+
+// Plans the teams of every kind for a common makespan T ms: each unit gets the
+// smallest team that finishes it in T, the units of one size
+// share as many teams as their times fill, and T is the smallest at which all
+// teams are resident together.  (Team sizes by edge count and CTAs by a guess
+// of the work, as before, left the longest unit of a mixed batch on a fifth
+// of the device while a third of it idled: 12 graphs, 15.6 ms.)
+void plan_teams(std::map<int, KindPlan> &kinds, const std::vector<UnitCost> &cost) {
+    double t0 = 1e30, tmax = 0;
+    for (auto &kv : kinds)
+        for (int u : kv.second.queries) tmax = std::max(tmax, cost[u].ms(kv.second.capacity));
+    t0 = std::max(tmax, 1e-3);
+    for (double T = t0;; T *= 1.06) {
+        double used = 0;
+        for (auto &kv : kinds) {
+            KindPlan &kp = kv.second;
+            std::map<int, std::vector<int>> by_size;
+            std::map<int, double> load;
+            for (int u : kp.queries) {
+                int p = 1;
+                while (p < kp.capacity && cost[u].ms(p) > T) p = std::min(kp.capacity, next_team(p));
+                by_size[p].push_back(u);
+                load[p] += cost[u].ms(p);
+            }
+            kp.class_size.clear();
+            kp.class_q.clear();
+            kp.class_teams.clear();
+            kp.ctas = 0;
+            for (auto &c : by_size) {
+                std::vector<int> v = c.second;
+                std::sort(v.begin(), v.end(), [&](int x, int y) { return cost[x].ms(c.first) > cost[y].ms(c.first); });
+                const int teams = std::min((int)v.size(), std::max(1, (int)(1.1 * load[c.first] / T + 0.999)));
+                kp.class_size.push_back(c.first);
+                kp.class_q.push_back(v);
+                kp.class_teams.push_back(teams);
+                kp.ctas += teams * c.first;
+            }
+            used += (double)kp.ctas / kp.capacity;
+        }
+        if (used <= 1.0 || T > 1e4 * t0) break;
+    }
+}
 
 }  // namespace
 
@@ -214,7 +283,7 @@ fg_status batch_launch(const fg_query *qs, int32_t nq, const fg_batch_options *o
     job.qmode.assign(nq, kVertexSync);
     job.qunit.assign(nq, 0);
     std::map<int, KindPlan> kinds;
-    double total_work = 0;
+    std::vector<UnitCost> cost(nu);
     for (int u = 0; u < nu; u++) {
         const BatchUnit &un = units[u];
         view[u] = (un.algo == kCC) ? &un.g->s : &un.g->g;
@@ -227,61 +296,17 @@ fg_status batch_launch(const fg_query *qs, int32_t nq, const fg_batch_options *o
         KindPlan &kp = kinds[kind];
         kp.kind = kind;
         kp.queries.push_back(u);
-        const double w = unit_work(un, *view[u]);
-        kp.work += w;
-        total_work += w;
+        cost[u] = unit_cost(un, *view[u]);
     }
     for (auto &kv : kinds) {
         KindPlan &kp = kv.second;
-        std::map<int, std::vector<int>> by_size;
-        // a kind with few units (at most 8) gives each a larger team (a lone
-        // unit the whole budget); otherwise the size follows its edge count
-        int per_sm0 = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm0, (const void *)batch_kernel_for(kp.kind), kBlock, 0);
-        const int cap0 = std::max(1, (int)(std::max(1, std::min(per_sm0 * sms, kMaxGrid)) * cta_fraction *
-                                           std::max(kp.work / std::max(total_work, 1.0), 0.0)));
-        int share = 1;
-        if (kp.queries.size() <= 8)
-            while (share * 2 <= cap0 / (int)kp.queries.size()) share *= 2;
-        for (int u : kp.queries) by_size[std::max(team_size_for(view[u]->m), share)].push_back(u);
-        std::vector<double> cw;
-        for (auto &c : by_size) {
-            std::vector<int> v = c.second;
-            std::sort(v.begin(), v.end(), [&](int a, int b) {
-                return unit_work(units[a], *view[a]) > unit_work(units[b], *view[b]);
-            });
-            double w = 0;
-            for (int u : v) w += unit_work(units[u], *view[u]);
-            kp.class_size.push_back(c.first);
-            kp.class_q.push_back(v);
-            cw.push_back(w);
-        }
         int per_sm = 0;
-        BatchFn fn = batch_kernel_for(kp.kind);
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)fn, kBlock, 0);
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &per_sm, (const void *)batch_kernel_for(kp.kind), kBlock, 0);
         if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
-        int capacity = std::max(1, std::min(per_sm * sms, kMaxGrid));
-        capacity = std::max(1, (int)(capacity * cta_fraction));
-        int min_ctas = 0;
-        for (int s : kp.class_size) min_ctas += std::min(s, capacity);
-        int budget = (int)(capacity * (kp.work / std::max(total_work, 1.0)));
-        budget = std::min(capacity, std::max(budget, min_ctas));
-        // one team per class, the rest of the budget by class work
-        int used = 0;
-        for (size_t c = 0; c < kp.class_size.size(); c++) {
-            kp.class_size[c] = std::min(kp.class_size[c], capacity);
-            kp.class_teams.push_back(1);
-            used += kp.class_size[c];
-        }
-        const int rest = std::max(0, budget - used);
-        for (size_t c = 0; c < kp.class_size.size(); c++) {
-            int extra = (int)(rest * (cw[c] / std::max(kp.work, 1.0)) / kp.class_size[c]);
-            extra = std::min(extra, (int)kp.class_q[c].size() - 1);
-            kp.class_teams[c] += std::max(0, extra);
-        }
-        kp.ctas = 0;
-        for (size_t c = 0; c < kp.class_size.size(); c++) kp.ctas += kp.class_teams[c] * kp.class_size[c];
+        kp.capacity = std::max(1, (int)(std::max(1, std::min(per_sm * sms, kMaxGrid)) * cta_fraction));
     }
+    plan_teams(kinds, cost);
 
     // ---- one device allocation: zeroed region | tables | unit workspaces | staging
     size_t zero_bytes = Workspace::need(1, sizeof(Ctrl)) + Workspace::need(nu, sizeof(Ctrl));
