@@ -1070,6 +1070,7 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
     if (!(create_flags & FG_GRAPH_LAZY)) {
         build_src(b, v);
         build_sym(b, g, indeg, &by_dst);
+        g->sym_built = b.status == FG_OK;
     }
     group_free(b, by_src);
     group_free(b, by_dst);

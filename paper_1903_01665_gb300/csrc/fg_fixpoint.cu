@@ -518,6 +518,7 @@ fg_status run_multi(const fg_graph *G, Algo algo, int32_t k, const int32_t *srcs
     carve_query_workspace(base, g, algo, kMulti, p);
     p.ms_k = k;
     p.ms_bfs = algo == kBFS ? 1 : 0;
+    if (algo == kBFS && G->sym_built && G->new_of) p.tv = G->s;   // its rows end with the in-edges: pull rounds
     set_relabel(G, p);
     p.delta = (opt && opt->delta > 0) ? opt->delta : default_delta(G);   // the SSSP sweep's near-far width
     p.ms_light = ms_light_width(G, algo, opt ? opt->delta : 0);

@@ -57,6 +57,7 @@ struct fg_graph {
     fg::View s;      // symmetrised
     fg::View t;      // transposed (in-neighbours), built on the first pull query
     bool t_ready = false;
+    bool sym_built = false;     // the symmetrised view was built at creation (never changes after)
     fg_graph_info_t info{};
     void *allocs[48] = {};
     int n_allocs = 0;
@@ -98,6 +99,7 @@ struct Ctrl {
     int pull_rounds;            // pull mode: rounds that pulled
     int far_size[3];            // bucket mode: far-list sizes, rotating by epoch
     int far_min[3];             // bucket mode: smallest distance in each epoch's far list
+    unsigned ms_front[3];       // multi-source BFS: sources with a frontier, by round
     int ms_min[3][8];           // multi-source light-heavy: each slot's smallest waiting distance, by split
     int splits;                 // bucket mode: far-list splits (threshold moves)
 };

@@ -989,7 +989,7 @@ __device__ __forceinline__ uint32_t ldcg_u32(const uint8_t *p) {
 template <int N>
 __device__ __forceinline__ void msb_relax(const View &g, const Params &p, uint8_t *vis, uint8_t *nxt, int32_t r,
                                           const uint32_t (&e)[N], const bool (&in)[N], const uint32_t (&f)[N],
-                                          Acc &a) {
+                                          uint32_t &found, Acc &a) {
     int32_t v[N];
     uint32_t seen[N];
 #pragma unroll
@@ -1010,13 +1010,14 @@ __device__ __forceinline__ void msb_relax(const View &g, const Params &p, uint8_
 #pragma unroll
         for (int s = 0; s < kMsMax; s++)
             if ((newly >> s) & 1u) stcg(p.ms_out[s] + ov, r);
+        found |= newly;
         a.changed++;
         a.updates++;
     }
 }
 
 __device__ __forceinline__ void msb_round(const Team &t, const View &g, const Params &p, uint8_t *vis,
-                                          const uint8_t *cur, uint8_t *nxt, int32_t r, Acc &a) {
+                                          const uint8_t *cur, uint8_t *nxt, int32_t r, uint32_t &found, Acc &a) {
     __shared__ int32_t s_list[kBlock];
     __shared__ int s_n;
     auto &s_rb = ms_light().rb;
@@ -1051,7 +1052,7 @@ __device__ __forceinline__ void msb_round(const Team &t, const View &g, const Pa
                     in[j] = e[j] < e1;
                     f[j] = fu;
                 }
-                msb_relax(g, p, vis, nxt, r, e, in, f, a);
+                msb_relax(g, p, vis, nxt, r, e, in, f, found, a);
             }
         }
         __syncthreads();
@@ -1085,7 +1086,7 @@ __device__ __forceinline__ void msb_round(const Team &t, const View &g, const Pa
                     in[j] = e[j] < en;
                     f[j] = ff;
                 }
-                msb_relax(g, p, vis, nxt, r, e, in, f, a);
+                msb_relax(g, p, vis, nxt, r, e, in, f, found, a);
             }
         }
     }
@@ -1159,10 +1160,106 @@ __device__ __forceinline__ void msb_round(const Team &t, const View &g, const Pa
                     in[j] = x < total;
                     e[j] = ob + (x - oe);
                 }
-                msb_relax(g, p, vis, nxt, r, e, in, f, a);
+                msb_relax(g, p, vis, nxt, r, e, in, f, found, a);
             }
         }
         __syncwarp();
+    }
+}
+
+// A pull round: every vertex that some source of `front` (those with a frontier)
+// has not reached ORs its in-neighbours' frontier masks until they hold all it
+// can get.  The in-edges of v are the end of its symmetrised row, after its
+// out-edges, so no transposed view is built.  A lane tries its own vertex's
+// first four in-neighbours; rows with more to read are taken by the warp in
+// turn, hubs (1024 symmetrised edges and more) by chunks.  Only its owner
+// writes a vertex's bytes, but for the hubs, whose chunks claim by atomic OR.
+__device__ __forceinline__ void msb_reached(const Params &p, int32_t v, uint32_t newly, int32_t r, Acc &a) {
+    const int32_t ov = p.orig_of ? __ldg(p.orig_of + v) : v;
+#pragma unroll
+    for (int s = 0; s < kMsMax; s++)
+        if ((newly >> s) & 1u) stcg(p.ms_out[s] + ov, r);
+    a.changed++;
+    a.updates++;
+}
+__device__ __forceinline__ void msb_pull_round(const Team &t, const View &g, const View &sv, const Params &p,
+                                               uint8_t *vis, const uint8_t *cur, uint8_t *nxt, uint32_t front,
+                                               int32_t r, uint32_t &found, Acc &a) {
+    const unsigned lane = lane_id();
+    const int64_t gw = ((int64_t)t.rank * kBlock + threadIdx.x) >> 5, nw = (int64_t)t.size * kWarps;
+    // frontier masks of the in-edges [b, e), by the warp, until they hold `need`
+    auto gather = [&](uint32_t b, uint32_t e, uint32_t need) -> uint32_t {
+        uint32_t got = 0;
+        for (uint32_t eb = b; eb < e && (got & need) != need; eb += 128) {
+            int32_t u[4];
+            uint32_t f = 0;
+#pragma unroll
+            for (int k = 0; k < 4; k++) u[k] = eb + 32 * k + lane < e ? ld_edge(sv.col + eb + 32 * k + lane) : -1;
+#pragma unroll
+            for (int k = 0; k < 4; k++)
+                if (u[k] >= 0) f |= (uint32_t)__ldca(cur + u[k]);
+            got |= __reduce_or_sync(0xffffffffu, f);
+            if (lane == 0) a.edges += min(e - eb, 128u);
+        }
+        return got;
+    };
+    for (int64_t i = gw; i < sv.n_high_chunks; i += nw) {
+        const int2 hc = __ldg(sv.high + i);
+        const int32_t v = hc.x;
+        const uint32_t need = front & ~(uint32_t)__ldcg(vis + v);
+        const uint32_t in0 = __ldg(sv.row_off + v) + (__ldg(g.row_off + v + 1) - __ldg(g.row_off + v));
+        const uint32_t b = max((uint32_t)hc.y, in0), e = min((uint32_t)hc.y + (uint32_t)kChunk, __ldg(sv.row_off + v + 1));
+        if (need == 0 || b >= e) continue;
+        const uint32_t bits = gather(b, e, need) & need;
+        if (lane == 0 && bits) {
+            const int sh = (v & 3) * 8;
+            const uint32_t old = atomicOr(reinterpret_cast<uint32_t *>(vis + (v & ~3)), bits << sh);
+            const uint32_t newly = bits & ~(old >> sh) & 0xffu;
+            if (newly) {
+                red_or(reinterpret_cast<uint32_t *>(nxt + (v & ~3)), newly << sh);
+                found |= newly;
+                msb_reached(p, v, newly, r, a);
+            }
+        }
+    }
+    const int32_t n = g.n;
+    for (int64_t v0 = gw * 32; v0 < n; v0 += nw * 32) {
+        const int64_t v = v0 + lane;
+        uint32_t need = 0, seen = 0, got = 0, b = 0, e = 0;
+        if (lane == 0) a.scanned += min((int64_t)32, (int64_t)n - v0);
+        if (v < n) {
+            seen = __ldcg(vis + v);
+            need = front & ~seen;
+            if (need) {
+                const uint32_t rb = __ldg(sv.row_off + v);
+                e = __ldg(sv.row_off + v + 1);
+                b = rb + (__ldg(g.row_off + v + 1) - __ldg(g.row_off + v));
+                if (e - rb >= (uint32_t)kMidMax) need = 0;   // by chunks, above
+            }
+        }
+        if (need && b < e) {
+            int32_t u[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) u[k] = b + k < e ? __ldg(sv.col + b + k) : -1;
+#pragma unroll
+            for (int k = 0; k < 4; k++)
+                if (u[k] >= 0) got |= (uint32_t)__ldca(cur + u[k]);
+            a.edges += min(e - b, 4u);
+            b += 4;
+        }
+        for (unsigned bal = __ballot_sync(0xffffffffu, need && b < e && (got & need) != need); bal; bal &= bal - 1) {
+            const int l = __ffs(bal) - 1;
+            const uint32_t x = gather(__shfl_sync(0xffffffffu, b, l), __shfl_sync(0xffffffffu, e, l),
+                                      __shfl_sync(0xffffffffu, need & ~got, l));
+            if ((int)lane == l) got |= x;
+        }
+        const uint32_t newly = got & need;
+        if (newly) {
+            vis[v] = (uint8_t)(seen | newly);
+            nxt[v] = (uint8_t)newly;
+            found |= newly;
+            msb_reached(p, (int32_t)v, newly, r, a);
+        }
     }
 }
 
@@ -1212,6 +1309,8 @@ __device__ __forceinline__ void multi_bfs_body(const Params &p, const Team &t) {
                 if (s < k) p.ms_out[s][v] = p.ms_src[s] == (int32_t)v ? 0 : kInf;
     }
     bool ok = sync_();
+    int64_t ch_prev = 0, ch_before = 0;   // changes of the last two rounds
+    uint32_t found = 0;                   // sources that the thread's claims of the round belong to
     for (int r = 1; ok; r++) {
         if (r > p.max_rounds) {
             if (tid == 0) atomicOr(&c->status, kStRoundCap);
@@ -1222,10 +1321,26 @@ __device__ __forceinline__ void multi_bfs_body(const Params &p, const Team &t) {
         uint8_t *nxt = F + ((r + 1) % 3) * np;
         int4 *clr = reinterpret_cast<int4 *>(F + ((r + 2) % 3) * np);   // the previous round's frontier
         for (int64_t i = tid; i < np / 16; i += nth) clr[i] = make_int4(0, 0, 0, 0);
-        msb_round(t, g, p, vis, cur, nxt, r, a);
+        // pulls like FG_PULL's BFS on a renumbered graph: after many changes
+        // or while the frontier explodes (R-MAT of 3 M vertices, 5 sources:
+        // those two rounds 230 us each pushed)
+        const int64_t ch = ch_prev;
+        const bool pull = p.tv.row_off && ((ch << 4) > (int64_t)n || ((ch << 7) > (int64_t)n && ch > 8 * ch_before));
+        ch_before = ch;
+        if (pull) {
+            if (tid == 0) c->pull_rounds++;
+            msb_pull_round(t, g, p.tv, p, vis, cur, nxt, __ldcg(&c->ms_front[r % 3]), r, found, a);
+        } else {
+            msb_round(t, g, p, vis, cur, nxt, r, found, a);
+        }
+        if (tid == 0) c->ms_front[(r + 2) % 3] = 0;
+        found = __reduce_or_sync(0xffffffffu, found);
+        if (lane_id() == 0 && found) atomicOr(&c->ms_front[(r + 1) % 3], found);
+        found = 0;
         if (!sync_(a.changed)) break;
         a.changed = 0;
-        if (team_total() == 0) {
+        ch_prev = team_total();
+        if (ch_prev == 0) {
             done = true;
             break;
         }
