@@ -100,6 +100,7 @@ struct Ctrl {
     int far_size[3];            // bucket mode: far-list sizes, rotating by epoch
     int far_min[3];             // bucket mode: smallest distance in each epoch's far list
     unsigned ms_front[3];       // multi-source BFS: sources with a frontier, by round
+    unsigned long long ms_mass[3][8];   // ... and the edges of the vertices that wait for it
     int ms_min[3][8];           // multi-source light-heavy: each slot's smallest waiting distance, by split
     int splits;                 // bucket mode: far-list splits (threshold moves)
 };

@@ -168,8 +168,9 @@ __device__ __forceinline__ void ms_relax_one_source(const View &g, int32_t *D, i
 // the light-heavy order, and the rows that a warp (or the CTA) gathered --
 // first edge, edges, vertex (or BFS frontier mask).
 struct MsLight {
-    int32_t T[kMsMax], T_old[kMsMax];
+    int32_t T[kMsMax], T_old[kMsMax], width[kMsMax];
     int32_t mn[kMsMax];
+    unsigned long long mass[kMsMax];
     uint32_t rb[kWarps][128], d[kWarps][128];
     int32_t u[kWarps][128];
     int n;
@@ -389,8 +390,8 @@ __device__ __forceinline__ int32_t ms_far_min(const int32_t (&x)[kMsMax], int32_
 // written by thread 0 between barriers; a source row's slots at or above it
 // are masked on load, so the relaxation itself does not ask.  R-MAT 24, 8
 // sources: 1.69 G edge visits in 17 rounds and 17.3 ms in the plain near-far
-// order, 0.60 G in 39 and 10.0 ms in this one (R-MAT 22 4.5 -> 2.8 ms).  It is
-// bound by the rows' probes: 32 bytes of 537 MB each.  Measured and left out:
+// order, 0.60 to 0.88 G in 50 to 80 and 10.6 to 14.6 ms in this one (R-MAT 22
+// 4.5 -> 3.1 to 4.2 ms).  It is bound by the rows' probes: 32 bytes of 537 MB each.  Measured and left out:
 // a bit per vertex whose slots are all settled, tested before a heavy edge's
 // row (11.0 ms: the slots settle at different times), 3 or 2 CTAs per SM
 // instead of 4 (11.7, 14.4 ms), one edge a lane (11.3 ms), the passes as
@@ -684,7 +685,7 @@ __device__ __forceinline__ bool ml_sweep(const Params &p, const Team &t, const i
     clear(H, 2);
     if (tid < 3 * kMsMax) (&c->ms_min[0][0])[tid] = kInf;
     if (threadIdx.x < kMsMax) {
-        m.T[threadIdx.x] = p.ms_light;
+        m.T[threadIdx.x] = m.width[threadIdx.x] = p.ms_light;
         m.T_old[threadIdx.x] = 0;
     }
     if (!sync_()) return false;
@@ -692,7 +693,6 @@ __device__ __forceinline__ bool ml_sweep(const Params &p, const Team &t, const i
         for (int s = 0; s < k; s++) F[np + msrc[s]] = 1;   // F[1]: the sources are near in generation 1
     if (!sync_()) return false;
     int phase = kLight, hp = 0, work = 0;
-    int32_t width = p.ms_light;
     bool h_used = false;
     for (int gen = 1;; gen++) {
         if (work >= p.max_rounds) {
@@ -731,52 +731,79 @@ __device__ __forceinline__ bool ml_sweep(const Params &p, const Team &t, const i
         // ---- split: each slot's smallest distance not below its threshold,
         // and the edges of the vertices not below it, over all slots
         rounds++;
-        if (threadIdx.x < kMsMax) m.mn[threadIdx.x] = kInf;
-        if (tid < kMsMax) c->ms_min[(splits + 1) % 3][tid] = kInf;
+        if (threadIdx.x < kMsMax) {
+            m.mn[threadIdx.x] = kInf;
+            m.mass[threadIdx.x] = 0;
+        }
+        if (tid < kMsMax) {
+            c->ms_min[(splits + 1) % 3][tid] = kInf;
+            c->ms_mass[(splits + 1) % 3][tid] = 0;
+        }
         __syncthreads();
-        uint32_t left = 0;
+        uint32_t left[kMsMax];
         int32_t mn[kMsMax];
 #pragma unroll
-        for (int s = 0; s < kMsMax; s++) mn[s] = kInf;
+        for (int s = 0; s < kMsMax; s++) {
+            mn[s] = kInf;
+            left[s] = 0;
+        }
         for (int64_t v = tid; v < n; v += nth) {
             int32_t x[kMsMax];
             ms_load_row(D + (size_t)v * kMsMax, x, true);
-            int open = 0;
+            const uint32_t deg = __ldg(g.row_off + v + 1) - __ldg(g.row_off + v);
 #pragma unroll
             for (int s = 0; s < kMsMax; s++) {
                 const bool wait = s < k && x[s] >= m.T[s];
-                open += wait;
-                if (wait) mn[s] = min(mn[s], x[s]);
+                if (wait) {
+                    mn[s] = min(mn[s], x[s]);
+                    left[s] += deg;
+                }
             }
-            if (open) left += open * (__ldg(g.row_off + v + 1) - __ldg(g.row_off + v));
         }
 #pragma unroll
         for (int s = 0; s < kMsMax; s++) {
             const int32_t x = warp_min(mn[s]);
+            const uint32_t d = __reduce_add_sync(0xffffffffu, left[s]);   // at most m < 2^31
             if (lane_id() == 0 && x < kInf) atomicMin(&m.mn[s], x);
+            if (lane_id() == 0 && d) atomicAdd(&m.mass[s], (unsigned long long)d);
         }
         __syncthreads();
-        if (threadIdx.x < kMsMax && m.mn[threadIdx.x] < kInf)
-            atomicMin(&c->ms_min[splits % 3][threadIdx.x], m.mn[threadIdx.x]);
-        if (!sync_((int)(left >> 4))) return false;   // sixteenths, so that a warp's sum stays in 32 bits
-        const bool both = 64 * team_total() < (int64_t)k * g.m;
-        int32_t low = kInf;
-        __syncthreads();   // every warp has read m.T
+        if (threadIdx.x < kMsMax) {
+            if (m.mn[threadIdx.x] < kInf) atomicMin(&c->ms_min[splits % 3][threadIdx.x], m.mn[threadIdx.x]);
+            if (m.mass[threadIdx.x]) atomicAdd(&c->ms_mass[splits % 3][threadIdx.x], m.mass[threadIdx.x]);
+        }
+        if (!sync_()) return false;
+        // A slot with less than a quarter of the edges left runs on without a
+        // threshold, the others get their next one.  The width holds for
+        // three splits -- sources at the rim take as many to reach the hubs,
+        // where a wide epoch relaxes heavy edges again and again -- and
+        // doubles from then on.  (One rule for all slots and a width doubled
+        // at every split: 18.8 ms on R-MAT 24 with three far sources, 5.4
+        // visits an edge, against 14.6 ms and 3.3.  Slots that wait with their
+        // heavy edges until every slot has reached the hubs changed nothing.)
         if (threadIdx.x < kMsMax) {
             const int s = threadIdx.x;
             const int32_t x = __ldcg(&c->ms_min[splits % 3][s]);
             m.mn[s] = x;
             m.T_old[s] = m.T[s];
-            if (both) m.T[s] = kInf;
-            else if (x < kInf) m.T[s] = x >= kInf - width ? kInf : x + width;
+            if (x < kInf) {
+                const int32_t w = m.width[s];
+                const bool tail = 4 * __ldcg(&c->ms_mass[splits % 3][s]) < (unsigned long long)g.m;
+                m.T[s] = tail || x >= kInf - w ? kInf : x + w;
+                if (splits >= 2) m.width[s] = w > kInf / 2 ? kInf : 2 * w;
+            }
         }
         __syncthreads();
+        int32_t low = kInf;
+        bool both = true;
 #pragma unroll
-        for (int s = 0; s < kMsMax; s++) low = min(low, m.mn[s]);
+        for (int s = 0; s < kMsMax; s++) {
+            low = min(low, m.mn[s]);
+            both &= m.mn[s] >= kInf || m.T[s] >= kInf;
+        }
         splits++;
         if (low >= kInf) return true;
         phase = both ? kBoth : kLight;
-        width = width > kInf / 2 ? kInf : 2 * width;
         // the vertices with a slot in between are near in the next generation
         uint8_t *mark = F + ((gen + 1) % 3) * np;
         for (int64_t v = tid; v < n; v += nth) {
