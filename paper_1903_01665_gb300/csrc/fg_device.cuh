@@ -352,7 +352,7 @@ struct BucketOp : AsyncOp<kSSSP> {
     Ctrl *ctrl;
 
     __device__ __forceinline__ bool commit(int32_t v, int32_t c, int32_t pv, Acc &a) const {
-        if (c < pv && c < ldcg(D + v)) {
+        if (c < pv) {   // without AsyncOp's second look: the grids' generations are chains of loads
             red_min(D + v, c);
             a.updates++;
             if (c < T) return atomicExch(stamp + v, gen + 1) != gen + 1;
@@ -2080,9 +2080,10 @@ __device__ __forceinline__ void stream_edges_async(const Team &t, const View &g,
 #define FG_SPARSE_SHIFT 0
 #endif
 // the bucketed mode runs many generations with small worklists: fewer CTAs
-// pay less per barrier (4 CTAs: 10.6 ms on the 4096^2 grid, 6: 11.9 ms)
+// pay less per barrier (SSSP on the 1500^2 / 4096^2 grid, 5, 4 and 3 CTAs per
+// SM: 2.44 / 8.47, 2.16 / 8.03 and 1.99 / 8.03 ms)
 #ifndef FG_BUCKET_MIN_BLOCKS
-#define FG_BUCKET_MIN_BLOCKS 4
+#define FG_BUCKET_MIN_BLOCKS 3
 #endif
 #ifndef FG_PULL_MIN_BLOCKS
 #define FG_PULL_MIN_BLOCKS 6
