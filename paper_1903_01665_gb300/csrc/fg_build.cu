@@ -631,7 +631,7 @@ void group_hist(Builder &b, int32_t n, int64_t m, const int32_t *s, const int32_
 
 // Pass 1 and the counts per sub-digit, the histogram given.
 void group_pass1(Builder &b, Grouped &q, int64_t m, const int32_t *key, const int32_t *a, const int32_t *w, bool with_w,
-                 int32_t split) {
+                 int32_t split, bool by_a = false) {
     if (b.status != FG_OK) return;
     q.sub = b.alloc_tmp<uint16_t>(m);
     q.a = b.alloc_tmp<int32_t>(m);
@@ -645,10 +645,10 @@ void group_pass1(Builder &b, Grouped &q, int64_t m, const int32_t *key, const in
     const size_t bytes = part_smem(q.sh.nb, with_w ? 12 : 8);
     if (with_w) {
         part_kernel_smem(b, k_part_pass1<true>, bytes);
-        k_part_pass1<true><<<g1, kPartThreads, bytes, b.st>>>(m, key, a, w, q.sh, split, q.plan.cursor, q.sub, q.a, q.b);
+        k_part_pass1<true><<<g1, kPartThreads, bytes, b.st>>>(m, key, a, w, q.sh, split, by_a, q.plan.cursor, q.sub, q.a, q.b);
     } else {
         part_kernel_smem(b, k_part_pass1<false>, bytes);
-        k_part_pass1<false><<<g1, kPartThreads, bytes, b.st>>>(m, key, a, nullptr, q.sh, split, q.plan.cursor, q.sub,
+        k_part_pass1<false><<<g1, kPartThreads, bytes, b.st>>>(m, key, a, nullptr, q.sh, split, by_a, q.plan.cursor, q.sub,
                                                               q.a, nullptr);
     }
     count_launch();
@@ -1193,9 +1193,31 @@ fg_status ensure_transpose(const fg_graph *cg) {
     uint32_t *tro = b.alloc_graph<uint32_t>((int64_t)n + 1);
     int32_t *tcol = b.alloc_graph<int32_t>(m);
     int32_t *tw = b.alloc_graph<int32_t>(m);
-    uint32_t *cnt = b.alloc_tmp<uint32_t>(n);
-    uint32_t *cursor = b.alloc_tmp<uint32_t>((int64_t)n + 1);
-    if (b.status == FG_OK) {
+    const bool group = part_usable(n, m);
+    uint32_t *cnt = group ? nullptr : b.alloc_tmp<uint32_t>(n);
+    uint32_t *cursor = group ? nullptr : b.alloc_tmp<uint32_t>((int64_t)n + 1);
+    if (group) {
+        // The grouping loses the order of the sources within a list, which the
+        // atomic scatter roughly keeps and a BFS pull's early exit lives on
+        // (hubs, the first ids of a renumbered graph, first): the first
+        // sixty-fourth of the ids are flagged to come first.  R-MAT 22: a new
+        // graph's first BFS 6.5 -> 2.5 ms.
+        Grouped q;
+        group_alloc(b, q, n, 1);
+        group_hist<false>(b, n, m, v.col, nullptr, nullptr, q, nullptr, nullptr, nullptr);
+        group_pass1(b, q, m, v.col, v.src, v.w, true, n / 64, true);
+        uint32_t *deg = b.alloc_tmp<uint32_t>(n);   // then the lists' first unflagged entries
+        if (b.status == FG_OK) {
+            k_part_degrees<<<grid_for(n), kBlock, 0, b.st>>>(n, q.count, 1, nullptr, deg);
+            count_launch();
+            b.check(exclusive_scan(deg, tro, n, b.st), "scan");
+            k_part_cursors<<<grid_for(n), kBlock, 0, b.st>>>(n, q.count, 1, tro, nullptr, nullptr, deg);
+            count_launch();
+        }
+        group_pass2(b, q, m, nullptr, tcol, tw);
+        if (deg) cudaFreeAsync(deg, b.st);
+        group_free(b, q);
+    } else if (b.status == FG_OK) {
         b.check(cudaMemsetAsync(cnt, 0, (size_t)n * sizeof(uint32_t), b.st), "memset");
         if (m > 0) { k_histogram<<<grid_for(m), kBlock, 0, b.st>>>(m, v.col, cnt); count_launch(); }
         b.check(exclusive_scan(cnt, tro, n, b.st), "scan");

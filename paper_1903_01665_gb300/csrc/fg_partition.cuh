@@ -194,12 +194,12 @@ inline size_t part_smem(int nd, int bytes_per_edge) {
 }
 
 // Pass 1: edges (key[e], a[e], b[e]) to their bucket; out_sub holds the low
-// bits of the key and, with the shape's flag, whether b[e] >= split (b ==
-// nullptr: all ones).  WITH_B: b is carried along.
+// bits of the key and, with the shape's flag, whether b[e] >= split, or a[e]
+// if by_a (b == nullptr: all ones).  WITH_B: b is carried along.
 template <bool WITH_B>
 __global__ void __launch_bounds__(kPartThreads, 2)
     k_part_pass1(int64_t m, const int32_t *__restrict__ key, const int32_t *__restrict__ a,
-                 const int32_t *__restrict__ b, PartShape sh, int32_t split, uint32_t *cursor, uint16_t *out_sub,
+                 const int32_t *__restrict__ b, PartShape sh, int32_t split, bool by_a, uint32_t *cursor, uint16_t *out_sub,
                  int32_t *out_a, int32_t *out_b) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int nd = sh.nb;
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kPartThreads, 2)
             if (WITH_B) {
                 const int32_t x = b ? __ldg(b + e0 + i) : 1;
                 s_b[pos] = x;
-                if (sh.flag) sub = 2 * sub + (x >= split);
+                if (sh.flag) sub = 2 * sub + ((by_a ? s_a[pos] : x) >= split);
             }
             s_dig[pos] = (uint16_t)d;
             s_sub[pos] = (uint16_t)sub;
