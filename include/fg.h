@@ -258,7 +258,8 @@ typedef struct {
     void *stream;               /* cudaStream_t to run on; NULL = legacy default stream */
     int32_t max_rounds;         /* round / generation cap; 0 = n + 2 (FG_BUCKET on split rows: 8 n + 64) */
     int32_t wait_timeout_ms;    /* bound on any single device-side wait; 0 = 1000 ms */
-    int32_t blocks_per_sm;      /* persistent CTAs per SM; 0 = occupancy limit */
+    int32_t blocks_per_sm;      /* persistent CTAs per SM; 0 = occupancy limit (fewer CTAs on a graph too
+                                   small to give each warp 8 vertices or 64 edges) */
     int32_t inject_missing_arrival; /* testing aid for failure detection: if nonzero, CTA 0
                                    leaves the kernel without arriving at the first grid
                                    barrier, so every other CTA's bounded wait runs out and

@@ -872,7 +872,8 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
         group_alloc(b, by_dst, n, 0);
     }
     unsigned long long *wsum = b.alloc_tmp<unsigned long long>(1);
-    unsigned long long weights = 0;   // their sum, if the validation formed it
+    unsigned long long weights = 0;   // their sum, once known
+    bool mean_known = coo_group;      // the validation forms it
     if (b.status == FG_OK) {
         b.check(cudaMemsetAsync(flags, 0, sizeof(int), b.st), "memset");
         b.check(cudaMemsetAsync(wsum, 0, sizeof(unsigned long long), b.st), "memset");
@@ -915,6 +916,12 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
             if (m > 0 && !by_dst.ready) { k_histogram<<<grid_for(m), kBlock, 0, b.st>>>(m, d_dst, indeg); count_launch(); }
             k_degree_bins<false><<<grid_for(n), kBlock, 0, b.st>>>(n, indeg, bins, bins + kDegBins);
             count_launch();
+            if (!coo_group && w && m > 0) {   // with the bins' wait: the rows' light bound may need it
+                k_weight_sum<<<grid_for(m), kBlock, 0, b.st>>>(m, d_w, wsum);
+                count_launch();
+                b.check(cudaMemcpyAsync(&weights, wsum, sizeof(weights), cudaMemcpyDeviceToHost, b.st), "copy");
+                mean_known = true;
+            }
             b.check(cudaMemcpyAsync(hb, bins, sizeof(hb), cudaMemcpyDeviceToHost, b.st), "copy");
             b.check(cudaStreamSynchronize(b.st), "in-degrees");
         }
@@ -978,16 +985,7 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
     // the edges, relaxed three times each, and 1.1 relaxations an edge in all;
     // half of it needs a third more generations, twice of it 1.3 relaxations.
     // Weights too alike or too small to tell light from heavy: no split.
-    bool mean_known = coo_group;
     if (relabel && w && m > 0) {
-        if (!coo_group && b.status == FG_OK) {
-            b.check(cudaMemsetAsync(wsum, 0, sizeof(unsigned long long), b.st), "memset");
-            k_weight_sum<<<grid_for(m), kBlock, 0, b.st>>>(m, d_w, wsum);
-            count_launch();
-            b.check(cudaMemcpyAsync(&weights, wsum, sizeof(weights), cudaMemcpyDeviceToHost, b.st), "copy");
-            b.check(cudaStreamSynchronize(b.st), "weight sum");
-            mean_known = true;
-        }
         const double l = 2.0 * ((double)weights / (double)m) / std::max(1.0, (double)m / (double)n);
         if (b.status == FG_OK && l >= 2.0) g->light = l < (double)(kInf / 2) ? (int32_t)(l + 0.5) : kInf / 2;
     }
@@ -1023,6 +1021,7 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
                                                                      split);
                     count_launch();
                     group_pass2(b, by_src, m, g->new_of, col, wt);
+                    group_free(b, by_src);   // before the symmetrised view is allocated
                 }
             } else if (b.status == FG_OK && g->new_of) {   // counted and scattered by original source id
                 b.check(cudaMemsetAsync(cnt_o, 0, ((size_t)n << flag) * sizeof(uint32_t), b.st), "memset");
