@@ -69,7 +69,7 @@ __global__ void k_histogram(int64_t m, const int32_t *__restrict__ keys, uint32_
 }
 
 // (the source array of the result is filled afterwards from the row
-// offsets, with sequential writes, by k_src_from_rows)
+// offsets, with sequential writes, by k_row_sources)
 __global__ void k_scatter_coo(int64_t m, const int32_t *__restrict__ s, const int32_t *__restrict__ d,
                               const int32_t *__restrict__ w, uint32_t *cursor, int32_t *col, int32_t *wout) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;

@@ -244,14 +244,20 @@ fg_status fg_sweep(const fg_graph *g, fg_mode mode, const int32_t *cur, int32_t 
 // measurements of every mode and two CTA counts on R-MAT graphs (scales 10 to
 // 22, Gini 0.79-0.94, 4-7 BFS levels), 2-D grids with shortcuts (256^2 to
 // 4096^2, Gini 0.02, 72-134 levels) and a uniform random graph (Gini 0.2):
-// its picks are within 10 % of the fastest (mode, CTAs per SM) for 201 of
-// those 207 (graph, algorithm) pairs, and within 15 % for all.  With degree
+// on 128 (graph, algorithm) pairs of 64 graphs of 16 K to 1 M vertices its
+// picks are within 10 % of the fastest (mode, CTAs per SM) for 85, the median
+// is 3 % behind it and the worst 44 % (the small graphs, where the modes now
+// lie within a few tens of microseconds of each other).  With degree
 // buckets the vertex modes no longer lose on skew the way the paper's K40C
 // code did, so skew mostly selects between the asynchronous edge form, pull
 // and the bucketed worklist, and depth selects the worklists that pay on
 // long propagation.
 namespace {
-// vertices from which FG_AUTO takes the light-heavy order on split rows
+// Vertices from which FG_AUTO takes the light-heavy order on split rows: it
+// needs more, shorter generations, so its barriers lose on small graphs.
+// Light-heavy against edge-async: R-MAT 12 0.15 against 0.10 ms, R-MAT 16 0.18
+// against 0.32, R-MAT 18 0.22 against 0.40, R-MAT 22 0.89 against 2.10; the
+// line is above the graphs for which edge-async is the documented pick.
 constexpr int64_t kLightHeavyMin = 1 << 17;
 
 fg_plan model_plan(const fg_graph *g, fg_algo algo, int32_t depth) {

@@ -24,9 +24,9 @@
 //                      When the vertices not below T hold less than a quarter
 //                      of the edges, the rest runs as one phase over all
 //                      their edges without a threshold.
-// R-MAT 22: 1.1 relaxations per edge in about 28 generations, 0.91 ms, against
-// 4.0 in 17 and 2.10 ms of the dense edge-async form (R-MAT 18 0.26 against
-// 0.40 ms, R-MAT 16 0.22 against 0.32).  It is bound by latency: 0.26 ms are
+// R-MAT 22: 1.1 relaxations per edge in about 28 generations, 0.89 ms, against
+// 4.0 in 17 and 2.10 ms of the dense edge-async form (R-MAT 18 0.22 against
+// 0.40 ms, R-MAT 16 0.18 against 0.32).  It is bound by latency: 0.26 ms are
 // the one large heavy pass, a third the ten light generations that carry
 // most of the frontier, a quarter the short ones before and after them.
 //
