@@ -36,7 +36,7 @@ struct BatchArgs {
 };
 
 template <int ALGO, int MODE>
-__global__ void __launch_bounds__(kBlock, min_blocks<MODE>()) batch_kernel(BatchArgs b) {
+__global__ void __launch_bounds__(kBlock, min_blocks<ALGO, MODE>()) batch_kernel(BatchArgs b) {
     const int4 ct = b.cta_team[blockIdx.x];
     const Team t{ct.y, ct.z, b.team_bar + (int64_t)kBarWords * ct.x};
     const int cls = ct.w;

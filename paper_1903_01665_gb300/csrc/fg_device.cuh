@@ -2081,7 +2081,9 @@ __device__ __forceinline__ void stream_edges_async(const Team &t, const View &g,
 #endif
 // the bucketed mode runs many generations with small worklists: fewer CTAs
 // pay less per barrier (SSSP on the 1500^2 / 4096^2 grid, 5, 4 and 3 CTAs per
-// SM: 2.44 / 8.47, 2.16 / 8.03 and 1.99 / 8.03 ms)
+// SM: 2.44 / 8.47, 2.16 / 8.03 and 1.99 / 8.03 ms;
+// for BFS and CC, which take larger generations, four: CC on R-MAT 22 281 -> 229
+// us, on the 2000^2 grid 1993 -> 1701, BFS on R-MAT 22 666 -> 572)
 #ifndef FG_BUCKET_MIN_BLOCKS
 #define FG_BUCKET_MIN_BLOCKS 3
 #endif
@@ -2101,12 +2103,12 @@ __device__ __forceinline__ void stream_edges_async(const Team &t, const View &g,
 #ifndef FG_LIGHT_MIN_BLOCKS
 #define FG_LIGHT_MIN_BLOCKS 4
 #endif
-template <int MODE>
+template <int ALGO, int MODE>
 constexpr int min_blocks() {
     return MODE == kVertexSync ? FG_SYNC_MIN_BLOCKS
          : MODE == kEdgeSync   ? FG_EDGE_SYNC_MIN_BLOCKS
          : MODE == kPull       ? FG_PULL_MIN_BLOCKS
-         : MODE == kBucket     ? FG_BUCKET_MIN_BLOCKS
+         : MODE == kBucket     ? (ALGO == kSSSP ? FG_BUCKET_MIN_BLOCKS : 4)
          : MODE == kMulti      ? FG_MULTI_MIN_BLOCKS
          : MODE == kLightHeavy ? FG_LIGHT_MIN_BLOCKS
                                : FG_ASYNC_MIN_BLOCKS;

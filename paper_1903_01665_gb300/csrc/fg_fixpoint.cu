@@ -11,7 +11,7 @@ namespace fg {
 namespace {
 
 template <int ALGO, int MODE>
-__global__ void __launch_bounds__(kBlock, min_blocks<MODE>()) fixpoint_kernel(Params p) {
+__global__ void __launch_bounds__(kBlock, min_blocks<ALGO, MODE>()) fixpoint_kernel(Params p) {
     const Team t{(int)blockIdx.x, (int)gridDim.x, p.ctrl->bar};
     uint32_t ring_used;
     team_begin();
@@ -350,6 +350,10 @@ fg_status run_query(const fg_graph *G, Algo algo, Mode user_mode, int32_t source
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)fn, kBlock, 0);
     if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
     if (opt && opt->blocks_per_sm > 0) per_sm = std::min(per_sm, (int)opt->blocks_per_sm);
+    // Bucketed BFS: the fourth CTA pays where a generation holds millions of
+    // edges (R-MAT 22: 3 CTAs 666 us, 4 572); elsewhere it lengthens the barriers
+    // (2000^2 grid 1093 and 1189, 300^2 grid 544 and 661, R-MAT 18 178 and 188).
+    else if (algo == kBFS && mode == kBucket && !(G->new_of && g.n >= (1 << 20))) per_sm = std::min(per_sm, 3);
     int grid = std::min(per_sm * dp.sms, kMaxGrid);
     if (grid < 1) return fail(FG_ERR_CUDA, "kernel does not fit on an SM");
     if (!(opt && opt->blocks_per_sm > 0)) grid = useful_grid(grid, dp.sms, g);
