@@ -591,9 +591,10 @@ struct Grouped {
     uint32_t *hist() const { return words; }
 };
 
+// The same limit from every caller (kPartMaxSmem): another thread's build never lowers it.
 template <typename K>
-void part_kernel_smem(Builder &b, K k, size_t bytes) {
-    b.check(cudaFuncSetAttribute((const void *)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes),
+void part_kernel_smem(Builder &b, K k) {
+    b.check(cudaFuncSetAttribute((const void *)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPartMaxSmem),
             "shared memory of the grouping kernels");
 }
 
@@ -622,7 +623,6 @@ void group_hist(Builder &b, int32_t n, int64_t m, const int32_t *s, const int32_
                 Grouped *qt, int *flags, unsigned long long *wsum) {
     if (b.status != FG_OK) return;
     const size_t bytes = 2 * (size_t)qs.sh.nb * sizeof(uint32_t);
-    part_kernel_smem(b, k_part_hist<VALIDATE>, bytes);
     k_part_hist<VALIDATE><<<grid_for(m, 4 * kPartThreads) > 608 ? 608 : grid_for(m, 4 * kPartThreads), kPartThreads,
                             bytes, b.st>>>(m, n, s, t, w, qs.sh, qs.hist(), qt ? qt->hist() : nullptr, flags, wsum);
     count_launch();
@@ -644,10 +644,10 @@ void group_pass1(Builder &b, Grouped &q, int64_t m, const int32_t *key, const in
     const unsigned g1 = (unsigned)((m + kPartTile - 1) / kPartTile);
     const size_t bytes = part_smem(q.sh.nb, with_w ? 12 : 8);
     if (with_w) {
-        part_kernel_smem(b, k_part_pass1<true>, bytes);
+        part_kernel_smem(b, k_part_pass1<true>);
         k_part_pass1<true><<<g1, kPartThreads, bytes, b.st>>>(m, key, a, w, q.sh, split, by_a, q.plan.cursor, q.sub, q.a, q.b);
     } else {
-        part_kernel_smem(b, k_part_pass1<false>, bytes);
+        part_kernel_smem(b, k_part_pass1<false>);
         k_part_pass1<false><<<g1, kPartThreads, bytes, b.st>>>(m, key, a, nullptr, q.sh, split, by_a, q.plan.cursor, q.sub,
                                                               q.a, nullptr);
     }
@@ -665,11 +665,11 @@ void group_pass2(Builder &b, Grouped &q, int64_t m, const int32_t *map, int32_t 
     const bool with_w = q.b != nullptr;
     const size_t bytes = part_smem(q.sh.sub(), with_w ? 10 : 6);
     if (with_w) {
-        part_kernel_smem(b, k_part_pass2<true>, bytes);
+        part_kernel_smem(b, k_part_pass2<true>);
         k_part_pass2<true><<<part_grid2(m, q.sh), kPartThreads, bytes, b.st>>>(q.plan, q.sh, q.sub, q.a, q.b, map,
                                                                               q.count, out_a, out_b);
     } else {
-        part_kernel_smem(b, k_part_pass2<false>, bytes);
+        part_kernel_smem(b, k_part_pass2<false>);
         k_part_pass2<false><<<part_grid2(m, q.sh), kPartThreads, bytes, b.st>>>(q.plan, q.sh, q.sub, q.a, nullptr, map,
                                                                                q.count, out_a, nullptr);
     }

@@ -35,7 +35,8 @@ static_assert(kPartTile == 1 << kPartRankBits, "ranks take kPartRankBits");
 // buckets; 1024 ids a bucket at least keep their number low on small graphs.)
 constexpr int64_t kPartMinEdges = 1 << 20;
 constexpr int32_t kPartMaxVertices = 1 << 24;
-constexpr int kPartMinLow = 10;
+constexpr int kPartMinLow = 10, kPartMaxLow = 12;
+constexpr int kPartMaxBuckets = kPartMaxVertices >> kPartMaxLow;
 
 // How the ids 0..n-1 are cut: buckets of 2^low ids; sub-digits are the low
 // bits, and below them the flag bit, if the edges carry one (flag = 1).
@@ -48,7 +49,7 @@ inline PartShape part_shape(int32_t n, int flag) {
     int bits = 1;
     while (((int64_t)1 << bits) < n) bits++;
     PartShape s;
-    s.low = std::max(kPartMinLow, std::min(12, bits - 11));
+    s.low = std::max(kPartMinLow, std::min(kPartMaxLow, bits - 11));
     s.nb = (int)(((int64_t)n + (1 << s.low) - 1) >> s.low);
     s.flag = flag;
     return s;
@@ -189,9 +190,19 @@ __device__ __forceinline__ void part_reserve(const PartTileMem &s, int nd, uint3
     __syncthreads();
 }
 
-inline size_t part_smem(int nd, int bytes_per_edge) {
+constexpr size_t part_smem(int nd, int bytes_per_edge) {
     return (size_t)nd * 4 + (((size_t)nd * 2 + 15) & ~(size_t)15) + (size_t)kPartTile * bytes_per_edge;
 }
+// The largest tile of either pass, over every shape.  A kernel's limit on
+// dynamic shared memory belongs to the kernel in the whole process, so every
+// caller sets it to this one value: a limit by the graph at hand could be
+// lowered by another thread's build between the call that raised it and the
+// launch that needs it.  (The histogram and the counts stay within the 48 KB
+// that need no limit raised.)
+constexpr size_t kPartMaxSmem =
+    std::max(part_smem(kPartMaxBuckets, 12), part_smem(1 << (kPartMaxLow + 1), 10));
+static_assert(2 * kPartMaxBuckets * sizeof(uint32_t) <= (48 << 10), "k_part_hist");
+static_assert(sizeof(uint32_t) << (kPartMaxLow + 1) <= (48 << 10), "k_part_count");
 
 // Pass 1: edges (key[e], a[e], b[e]) to their bucket; out_sub holds the low
 // bits of the key and, with the shape's flag, whether b[e] >= split, or a[e]
