@@ -377,7 +377,7 @@ __device__ __forceinline__ int last_row_at(const uint32_t *ro, int n, uint32_t e
 }
 __global__ void __launch_bounds__(kBlock) k_row_sources(int32_t n, int64_t m, const uint32_t *__restrict__ ro,
                                                         int32_t *src) {
-    __shared__ int32_t own[kRowTile];
+    __shared__ __align__(16) int32_t own[kRowTile];   // read four marks at a time
     __shared__ int s_row[2];
     __shared__ int32_t s_max[kWarps];
     const int64_t e0 = (int64_t)blockIdx.x * kRowTile;
