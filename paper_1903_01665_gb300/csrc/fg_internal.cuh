@@ -206,6 +206,12 @@ __device__ __forceinline__ void red_min(int32_t *p, int32_t v) {
 __device__ __forceinline__ void red_or(uint32_t *p, uint32_t v) {
     asm volatile("red.relaxed.gpu.global.or.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
+// a word that others change by atomics at the same time
+__device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t *p) {
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
 // BFS visited bitmap: bit v & 31 of word v >> 5.  Bits are only ever set
 // during a query, so a stale (L1) copy can only miss bits, never show one.
 __device__ __forceinline__ bool vis_test(const uint32_t *vis, int32_t v) {

@@ -1199,8 +1199,9 @@ __device__ __forceinline__ void msb_round(const Team &t, const View &g, const Pa
 // can get.  The in-edges of v are the end of its symmetrised row, after its
 // out-edges, so no transposed view is built.  A lane tries its own vertex's
 // first four in-neighbours; rows with more to read are taken by the warp in
-// turn, hubs (1024 symmetrised edges and more) by chunks.  Only its owner
-// writes a vertex's bytes, but for the hubs, whose chunks claim by atomic OR.
+// turn, hubs (1024 symmetrised edges and more) by chunks.  A hub may lie among
+// other vertices, whose bytes share its words: both arrays are read and
+// claimed by words throughout, four lanes' bytes in one atomic OR.
 __device__ __forceinline__ void msb_reached(const Params &p, int32_t v, uint32_t newly, int32_t r, Acc &a) {
     const int32_t ov = p.orig_of ? __ldg(p.orig_of + v) : v;
 #pragma unroll
@@ -1230,20 +1231,22 @@ __device__ __forceinline__ void msb_pull_round(const Team &t, const View &g, con
         }
         return got;
     };
+    uint32_t *vis4 = reinterpret_cast<uint32_t *>(vis), *nxt4 = reinterpret_cast<uint32_t *>(nxt);
+    auto seen_by = [&](int64_t v) { return (ld_relaxed_u32(vis4 + (v >> 2)) >> ((v & 3) * 8)) & 0xffu; };
     for (int64_t i = gw; i < sv.n_high_chunks; i += nw) {
         const int2 hc = __ldg(sv.high + i);
         const int32_t v = hc.x;
-        const uint32_t need = front & ~(uint32_t)__ldcg(vis + v);
+        const uint32_t need = front & ~seen_by(v);
         const uint32_t in0 = __ldg(sv.row_off + v) + (__ldg(g.row_off + v + 1) - __ldg(g.row_off + v));
         const uint32_t b = max((uint32_t)hc.y, in0), e = min((uint32_t)hc.y + (uint32_t)kChunk, __ldg(sv.row_off + v + 1));
         if (need == 0 || b >= e) continue;
         const uint32_t bits = gather(b, e, need) & need;
         if (lane == 0 && bits) {
             const int sh = (v & 3) * 8;
-            const uint32_t old = atomicOr(reinterpret_cast<uint32_t *>(vis + (v & ~3)), bits << sh);
+            const uint32_t old = atomicOr(vis4 + (v >> 2), bits << sh);
             const uint32_t newly = bits & ~(old >> sh) & 0xffu;
             if (newly) {
-                red_or(reinterpret_cast<uint32_t *>(nxt + (v & ~3)), newly << sh);
+                red_or(nxt4 + (v >> 2), newly << sh);
                 found |= newly;
                 msb_reached(p, v, newly, r, a);
             }
@@ -1252,11 +1255,10 @@ __device__ __forceinline__ void msb_pull_round(const Team &t, const View &g, con
     const int32_t n = g.n;
     for (int64_t v0 = gw * 32; v0 < n; v0 += nw * 32) {
         const int64_t v = v0 + lane;
-        uint32_t need = 0, seen = 0, got = 0, b = 0, e = 0;
+        uint32_t need = 0, got = 0, b = 0, e = 0;
         if (lane == 0) a.scanned += min((int64_t)32, (int64_t)n - v0);
         if (v < n) {
-            seen = __ldcg(vis + v);
-            need = front & ~seen;
+            need = front & ~seen_by(v);
             if (need) {
                 const uint32_t rb = __ldg(sv.row_off + v);
                 e = __ldg(sv.row_off + v + 1);
@@ -1281,9 +1283,15 @@ __device__ __forceinline__ void msb_pull_round(const Team &t, const View &g, con
             if ((int)lane == l) got |= x;
         }
         const uint32_t newly = got & need;
+        if (!__any_sync(0xffffffffu, newly)) continue;
+        uint32_t word = newly << ((lane & 3) * 8);   // v0 is a multiple of 32
+        word |= __shfl_xor_sync(0xffffffffu, word, 1);
+        word |= __shfl_xor_sync(0xffffffffu, word, 2);
+        if ((lane & 3) == 0 && word) {
+            red_or(vis4 + (v >> 2), word);
+            red_or(nxt4 + (v >> 2), word);
+        }
         if (newly) {
-            vis[v] = (uint8_t)(seen | newly);
-            nxt[v] = (uint8_t)newly;
             found |= newly;
             msb_reached(p, (int32_t)v, newly, r, a);
         }
