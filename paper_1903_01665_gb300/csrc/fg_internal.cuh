@@ -305,7 +305,7 @@ __device__ __forceinline__ void raise_error(Ctrl *c, int bits) {
 // Barrier over the CTAs of a team (all co-resident: the launch is
 // cooperative) that also sums `add` over all its threads; the total is in
 // team_total() until the next barrier.  One word takes the arrivals, the
-// errors and the sum (12, 12 and 40 bits) in one atomic add per CTA, and the
+// errors and the sum (11, 12 and 40 bits) in one atomic add per CTA, and the
 // CTAs poll that same word, so that one poll returns the release, the sum
 // and whether any CTA recorded a fatal error: nothing else is read or
 // counted.  It is bound by L2 latency and by the adds' serialisation on one
@@ -315,13 +315,25 @@ __device__ __forceinline__ void raise_error(Ctrl *c, int bits) {
 // count 2.8 / 3.2 / 3.4 us, clusters of 2-8 CTAs with one arrival each 2.2 /
 // 2.5 / 2.7 us.  The words are used in turn; rank 0 clears the next one
 // before it arrives, when every CTA has left the barrier that used it last.
-// The wait is bounded by timeout_ns: on expiry the CTA records kStTimeout
-// and returns false.  It returns false, too, once a CTA has recorded a fatal
-// error, so every CTA of the team leaves the query at its next barrier.  A
-// one-CTA team needs only __syncthreads, and an acquire (of the status) that
-// discards the SM's L1 lines as the poll does.
+// The wait is bounded by timeout_ns: on expiry the CTA records kStTimeout,
+// marks the word as broken (bar_break) and returns false; the mark makes
+// every other CTA of the barrier return false too, those that arrive later
+// included, without a time-out of their own.  It returns false, too, once a
+// CTA has recorded a fatal error, so every CTA of the team leaves the query at
+// its next barrier.  A one-CTA team needs only __syncthreads, and an acquire
+// (of the status) that discards the SM's L1 lines as the poll does.
 constexpr int kBarErrShift = 40, kBarCntShift = 52;
-static_assert(kMaxGrid < (1 << 12), "arrivals and errors take 12 bits each");
+constexpr unsigned long long kBarBroken = 1ull << 63;
+static_assert(kMaxGrid < (1 << 11), "arrivals take 11 bits, errors 12");
+__device__ __forceinline__ int bar_arrived(unsigned long long v) { return (int)(v >> kBarCntShift) & 0x7ff; }
+// After a wait ran out: marks the word, unless the last CTA has arrived in
+// the meantime; the compare-and-swap makes it one or the other for every CTA.
+// Returns the word.
+__device__ __forceinline__ unsigned long long bar_break(unsigned long long *w, int size) {
+    unsigned long long v = ld_acquire_u64(w);
+    while (bar_arrived(v) != size && !(v & kBarBroken)) atomicCAS(w, v, v | kBarBroken), v = ld_acquire_u64(w);
+    return v;
+}
 __device__ __forceinline__ bool team_sync(const Team &t, Ctrl *c, unsigned long long timeout_ns, int add = 0) {
     BarState &s = bar_state();
     add = (int)__reduce_add_sync(0xffffffffu, (unsigned)add);
@@ -342,23 +354,22 @@ __device__ __forceinline__ bool team_sync(const Team &t, Ctrl *c, unsigned long 
             const unsigned long long one =
                 (1ull << kBarCntShift) | ((unsigned long long)(s.err != 0) << kBarErrShift) | sum;
             unsigned long long v = atom_add_acq_rel(w, one) + one;
-            int ok = 1;
-            if ((int)(v >> kBarCntShift) != t.size) {
+            if ((int)(v >> kBarCntShift) != t.size) {   // the mark counts as a difference
                 const unsigned long long t0 = global_ns();
                 unsigned spins = 0;
                 while ((int)((v = ld_acquire_u64(w)) >> kBarCntShift) != t.size) {
                     if (++spins > 32) {
+                        if (v & kBarBroken) break;
                         __nanosleep(32);
                         if (global_ns() - t0 > timeout_ns) {
-                            raise_error(c, kStTimeout);
-                            ok = 0;
+                            v = bar_break(w, t.size);
+                            if (v & kBarBroken) raise_error(c, kStTimeout);
                             break;
                         }
                     }
                 }
             }
-            if ((v >> kBarErrShift) & 0xfffu) ok = 0;
-            s.ok = ok;
+            s.ok = !(v & kBarBroken) && !((v >> kBarErrShift) & 0xfffu);
             s.sum = v & ((1ull << kBarErrShift) - 1);
         }
     }
