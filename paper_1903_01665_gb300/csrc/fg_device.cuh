@@ -2314,7 +2314,6 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
         return r;
     };
 
-    if (threadIdx.x == 0) bar_state().err = 0;   // of this query
     // the source in internal ids (a renumbered graph takes original ones)
     const int32_t source = (ALGO != kCC && p.new_of) ? __ldg(p.new_of + p.source) : p.source;
     // components by hooking and linking: labels and everything else set there

@@ -279,10 +279,15 @@ struct Team {
 
 constexpr int kStFatal = kStTimeout | kStRoundCap | kStWorklist;
 
+// BarState::err: this CTA recorded a fatal error of the query, at which the
+// whole team leaves at its next barrier; a wait ran out, so that the CTAs are
+// no longer at the same barrier and the team cannot go on with another query
+constexpr int kErrQuery = 1, kErrBroken = 2;
+
 // This CTA's side of its team's barrier.
 struct BarState {
     int slot;                          // the next barrier's word (thread 0 only)
-    int err;                           // this CTA recorded a fatal error in the current query
+    int err;                           // kErr bits of the current query
     int ok;
     int part[kWarps];                  // each warp's contribution
     unsigned long long sum;            // the last barrier's total
@@ -299,7 +304,7 @@ __device__ __forceinline__ void team_begin() {
 // CTA's state, from which its next barrier tells the team.
 __device__ __forceinline__ void raise_error(Ctrl *c, int bits) {
     atomicOr(&c->status, bits);
-    bar_state().err = 1;
+    atomicOr(&bar_state().err, bits & kStTimeout ? kErrQuery | kErrBroken : kErrQuery);
 }
 
 // Barrier over the CTAs of a team (all co-resident: the launch is
@@ -370,11 +375,21 @@ __device__ __forceinline__ bool team_sync(const Team &t, Ctrl *c, unsigned long 
                 }
             }
             s.ok = !(v & kBarBroken) && !((v >> kBarErrShift) & 0xfffu);
+            if (v & kBarBroken) s.err |= kErrBroken;
             s.sum = v & ((1ull << kBarErrShift) - 1);
         }
     }
     __syncthreads();
     return s.ok != 0;
+}
+// Between two queries of a team, by every thread: forgets the last query's
+// error (all CTAs left it at the same barrier).  False if a wait ran out in it.
+__device__ __forceinline__ bool team_next_query(const Team &t) {
+    __syncthreads();
+    const bool ok = t.size == 1 || !(bar_state().err & kErrBroken);
+    __syncthreads();
+    if (threadIdx.x == 0) bar_state().err = 0;
+    return ok;
 }
 // The sum of the team's last barrier (read it before the next one).
 __device__ __forceinline__ int64_t team_total() { return (int64_t)bar_state().sum; }

@@ -835,7 +835,6 @@ __device__ __forceinline__ void multi_body(const Params &p, const Team &t) {
     Acc a;
     int rounds = 0, n_barriers = 0;
     bool done = false;
-    if (threadIdx.x == 0) bar_state().err = 0;   // of this query
     stat_begin();
     auto sync_ = [&](int add = 0) -> bool {
         stat_flush(a);
@@ -1316,7 +1315,6 @@ __device__ __forceinline__ void multi_bfs_body(const Params &p, const Team &t) {
     Acc a;
     int rounds = 0, n_barriers = 0;
     bool done = false;
-    if (threadIdx.x == 0) bar_state().err = 0;   // of this query
     stat_begin();
     auto sync_ = [&](int add = 0) -> bool {
         stat_flush(a);
