@@ -126,6 +126,9 @@ typedef enum { FG_ALGO_SSSP = 0, FG_ALGO_BFS = 1, FG_ALGO_CC = 2 } fg_algo;
  * degree buckets of the vertex kernels (1..31, 32..1023, >= 1024 out-edges),
  * and the symmetrised CSR/COO used by connected components (every edge also
  * read backwards: the undirected nbrs iterator, Table "foreach iterators").
+ * From 2^20 edges on (and up to 2^24 vertices) the edges are sorted by
+ * partition passes, which take up to 16 bytes an edge of temporary device
+ * memory; where it is not there, by a slower sort that takes none.
  * Self-loops and duplicate edges are kept.  The handle is written to *out
  * only on success.  Errors: FG_ERR_INVALID_ARG, FG_ERR_NEGATIVE_WEIGHT,
  * FG_ERR_OUT_OF_MEMORY, FG_ERR_CUDA.

@@ -523,25 +523,64 @@ __global__ void __launch_bounds__(kBlock)
     }
 }
 
+// Edges grouped by an id (fg_partition.cuh): after pass 1, by bucket.
+struct Grouped {
+    PartShape sh;
+    PartPlan plan;
+    uint32_t *words = nullptr;    // one allocation: histogram, plan
+    uint16_t *sub = nullptr;
+    int32_t *a = nullptr, *b = nullptr;
+    uint32_t *count = nullptr;    // per sub-digit; then the cursors of pass 2
+    bool ready = false;
+    uint32_t *hist() const { return words; }
+    void release(cudaStream_t st) {
+        void *all[] = {words, sub, a, b, count};
+        for (void *p : all)
+            if (p) cudaFreeAsync(p, st);
+        *this = Grouped();
+    }
+};
+
 // RAII-free allocation helper recording into the graph for destroy
 struct Builder {
     fg_graph *g;
     cudaStream_t st;
     fg_status status = FG_OK;
     std::string msg;
+    Grouped *spare = nullptr;   // given up before an allocation fails
 
-    template <typename T>
-    T *alloc_graph(int64_t count) {
+    // The groupings are a build's largest temporaries and only make it faster:
+    // when memory runs out they are returned, to the device, and what needs
+    // them does without.
+    void give_up(Grouped &q) {
+        q.release(st);
+        int dev = 0;
+        cudaMemPool_t pool;
+        cudaStreamSynchronize(st);
+        if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetMemPool(&pool, dev) == cudaSuccess)
+            cudaMemPoolTrimTo(pool, 0);
+        cudaGetLastError();
+    }
+    void *allocate(size_t bytes) {
         if (status != FG_OK) return nullptr;
         void *p = nullptr;
-        size_t bytes = (size_t)std::max<int64_t>(count, 1) * sizeof(T);
         cudaError_t e = cudaMallocAsync(&p, bytes, st);
-        if (e != cudaSuccess) {
-            status = (e == cudaErrorMemoryAllocation) ? FG_ERR_OUT_OF_MEMORY : FG_ERR_CUDA;
-            msg = std::string("device allocation failed: ") + cudaGetErrorString(e);
+        if (e == cudaErrorMemoryAllocation && spare && spare->ready) {
             cudaGetLastError();
-            return nullptr;
+            give_up(*spare);
+            e = cudaMallocAsync(&p, bytes, st);
         }
+        if (e == cudaSuccess) return p;
+        status = (e == cudaErrorMemoryAllocation) ? FG_ERR_OUT_OF_MEMORY : FG_ERR_CUDA;
+        msg = std::string("device allocation failed: ") + cudaGetErrorString(e);
+        cudaGetLastError();
+        return nullptr;
+    }
+    template <typename T>
+    T *alloc_graph(int64_t count) {
+        const size_t bytes = (size_t)std::max<int64_t>(count, 1) * sizeof(T);
+        void *p = allocate(bytes);
+        if (!p) return nullptr;
         if (g->n_allocs >= (int)(sizeof(g->allocs) / sizeof(g->allocs[0]))) {
             cudaFreeAsync(p, st);
             status = FG_ERR_CUDA;
@@ -554,16 +593,7 @@ struct Builder {
     }
     template <typename T>
     T *alloc_tmp(int64_t count) {
-        if (status != FG_OK) return nullptr;
-        void *p = nullptr;
-        cudaError_t e = cudaMallocAsync(&p, (size_t)std::max<int64_t>(count, 1) * sizeof(T), st);
-        if (e != cudaSuccess) {
-            status = (e == cudaErrorMemoryAllocation) ? FG_ERR_OUT_OF_MEMORY : FG_ERR_CUDA;
-            msg = std::string("device allocation failed: ") + cudaGetErrorString(e);
-            cudaGetLastError();
-            return nullptr;
-        }
-        return (T *)p;
+        return (T *)allocate((size_t)std::max<int64_t>(count, 1) * sizeof(T));
     }
     bool check(cudaError_t e, const char *what) {
         if (status != FG_OK) return false;
@@ -578,18 +608,6 @@ struct Builder {
 };
 
 unsigned row_grid(int64_t m) { return (unsigned)((m + kRowTile - 1) / kRowTile); }
-
-// Edges grouped by an id (fg_partition.cuh): after pass 1, by bucket.
-struct Grouped {
-    PartShape sh;
-    PartPlan plan;
-    uint32_t *words = nullptr;    // one allocation: histogram, plan
-    uint16_t *sub = nullptr;
-    int32_t *a = nullptr, *b = nullptr;
-    uint32_t *count = nullptr;    // per sub-digit; then the cursors of pass 2
-    bool ready = false;
-    uint32_t *hist() const { return words; }
-};
 
 // The same limit from every caller (kPartMaxSmem): another thread's build never lowers it.
 template <typename K>
@@ -610,13 +628,6 @@ void group_alloc(Builder &b, Grouped &q, int32_t n, int flag) {
     b.check(cudaMemsetAsync(q.words, 0, (size_t)nb * sizeof(uint32_t), b.st), "memset");
 }
 
-void group_free(Builder &b, Grouped &q) {
-    void *all[] = {q.words, q.sub, q.a, q.b, q.count};
-    for (void *p : all)
-        if (p) cudaFreeAsync(p, b.st);
-    q = Grouped();
-}
-
 // Edges per bucket of s into qs, of t (may be null) into qt; VALIDATE as k_part_hist.
 template <bool VALIDATE>
 void group_hist(Builder &b, int32_t n, int64_t m, const int32_t *s, const int32_t *t, const int32_t *w, Grouped &qs,
@@ -629,15 +640,23 @@ void group_hist(Builder &b, int32_t n, int64_t m, const int32_t *s, const int32_
     b.check(cudaGetLastError(), "edges per bucket");
 }
 
-// Pass 1 and the counts per sub-digit, the histogram given.
-void group_pass1(Builder &b, Grouped &q, int64_t m, const int32_t *key, const int32_t *a, const int32_t *w, bool with_w,
+// Pass 1 and the counts per sub-digit, the histogram given.  False, and q
+// released, if there is no memory for it (no error: the one-pass sort needs
+// none) or an error was met before.
+bool group_pass1(Builder &b, Grouped &q, int64_t m, const int32_t *key, const int32_t *a, const int32_t *w, bool with_w,
                  int32_t split, bool by_a = false) {
-    if (b.status != FG_OK) return;
+    if (b.status != FG_OK) return false;
     q.sub = b.alloc_tmp<uint16_t>(m);
     q.a = b.alloc_tmp<int32_t>(m);
     if (with_w) q.b = b.alloc_tmp<int32_t>(m);
     q.count = b.alloc_tmp<uint32_t>(q.sh.counters());
-    if (b.status != FG_OK) return;
+    if (b.status == FG_ERR_OUT_OF_MEMORY) {
+        b.status = FG_OK;
+        b.msg.clear();
+        b.give_up(q);
+        return false;
+    }
+    if (b.status != FG_OK) return false;
     b.check(cudaMemsetAsync(q.count, 0, (size_t)q.sh.counters() * sizeof(uint32_t), b.st), "memset");
     k_part_plan<<<1, 1024, 0, b.st>>>(q.hist(), q.sh.nb, q.plan);
     count_launch();
@@ -656,7 +675,7 @@ void group_pass1(Builder &b, Grouped &q, int64_t m, const int32_t *key, const in
     k_part_count<<<part_grid2(m, q.sh), kPartThreads, cbytes, b.st>>>(q.plan, q.sh, q.sub, q.count);
     count_launch();
     b.check(cudaGetLastError(), "grouping by bucket");
-    q.ready = b.status == FG_OK;
+    return q.ready = b.status == FG_OK;
 }
 
 // Pass 2 to out_a (through map) and out_b; q.count holds the cursors.
@@ -778,7 +797,7 @@ void build_sym(Builder &b, fg_graph *g, const uint32_t *indeg = nullptr, Grouped
     int32_t *ssrc = b.alloc_graph<int32_t>(2 * m);
     if (b.status == FG_OK) {
         uint32_t *deg = b.alloc_tmp<uint32_t>(n);
-        uint32_t *cursor = b.alloc_tmp<uint32_t>((int64_t)n + 1);
+        uint32_t *cursor = nullptr;
         if (b.status == FG_OK) {
             if (indeg) {   // the in-degrees counted at creation
                 b.check(cudaMemcpyAsync(deg, indeg, (size_t)n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, b.st),
@@ -790,26 +809,27 @@ void build_sym(Builder &b, fg_graph *g, const uint32_t *indeg = nullptr, Grouped
             k_sym_degree<<<grid_for(n), kBlock, 0, b.st>>>(n, v.row_off, deg);
             count_launch();
             b.check(exclusive_scan(deg, sro, n, b.st), "scan");
+            b.spare = nullptr;   // the grouping is used now
             Grouped mine;
-            const bool grouped = (by_dst && by_dst->ready) || part_usable(n, m);
-            if (grouped) {
-                Grouped &q = by_dst && by_dst->ready ? *by_dst : mine;
-                const int32_t *map = &q == &mine ? nullptr : g->new_of;   // original ids, or internal ones
-                if (&q == &mine) {
-                    group_alloc(b, q, n, 0);
-                    group_hist<false>(b, n, m, v.col, nullptr, nullptr, q, nullptr, nullptr, nullptr);
-                    group_pass1(b, q, m, v.col, v.src, nullptr, false, 0);
-                }
-                if (b.status == FG_OK) {
-                    k_part_cursors<<<grid_for(n), kBlock, 0, b.st>>>(n, q.count, 0, sro, v.row_off, map, nullptr);
-                    count_launch();
-                    group_pass2(b, q, m, map, scol, nullptr);
-                    k_sym_out<<<grid_for(m), kBlock, 0, b.st>>>(m, v.src, v.col, v.row_off, sro, scol);
-                    count_launch();
-                    k_row_sources<<<row_grid(2 * m), kBlock, 0, b.st>>>(n, 2 * m, sro, ssrc);
-                    count_launch();
-                }
-                group_free(b, mine);
+            Grouped &q = by_dst && by_dst->ready ? *by_dst : mine;
+            const int32_t *map = &q == &mine ? nullptr : g->new_of;   // original ids, or internal ones
+            if (&q == &mine && part_usable(n, m)) {
+                group_alloc(b, q, n, 0);
+                group_hist<false>(b, n, m, v.col, nullptr, nullptr, q, nullptr, nullptr, nullptr);
+                group_pass1(b, q, m, v.col, v.src, nullptr, false, 0);
+            }
+            const bool grouped = q.ready;
+            if (!grouped) cursor = b.alloc_tmp<uint32_t>((int64_t)n + 1);
+            if (b.status != FG_OK) {
+                // reported by the caller
+            } else if (grouped) {
+                k_part_cursors<<<grid_for(n), kBlock, 0, b.st>>>(n, q.count, 0, sro, v.row_off, map, nullptr);
+                count_launch();
+                group_pass2(b, q, m, map, scol, nullptr);
+                k_sym_out<<<grid_for(m), kBlock, 0, b.st>>>(m, v.src, v.col, v.row_off, sro, scol);
+                count_launch();
+                k_row_sources<<<row_grid(2 * m), kBlock, 0, b.st>>>(n, 2 * m, sro, ssrc);
+                count_launch();
             } else if (g->new_of) {
                 k_sym_cursor_orig<<<grid_for(n), kBlock, 0, b.st>>>(n, sro, v.row_off, g->new_of, cursor);
                 count_launch();
@@ -817,7 +837,7 @@ void build_sym(Builder &b, fg_graph *g, const uint32_t *indeg = nullptr, Grouped
                 k_sym_cursor<<<grid_for(n), kBlock, 0, b.st>>>(n, sro, v.row_off, cursor);
                 count_launch();
             }
-            if (m > 0 && !grouped) {
+            if (b.status == FG_OK && m > 0 && !grouped) {
                 if (g->new_of) {
                     k_scatter_sym_renum<<<grid_for(m), kBlock, 0, b.st>>>(m, v.src, v.col, v.row_off, sro,
                                                                           g->orig_of, cursor, scol);
@@ -830,6 +850,7 @@ void build_sym(Builder &b, fg_graph *g, const uint32_t *indeg = nullptr, Grouped
                 count_launch();
             }
             b.check(cudaGetLastError(), "symmetrise");
+            mine.release(b.st);
         }
         if (deg) cudaFreeAsync(deg, b.st);
         if (cursor) cudaFreeAsync(cursor, b.st);
@@ -901,7 +922,10 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
     uint32_t *indeg = nullptr;     // in-degrees by internal id
     int32_t *t_csrc = nullptr;
     uint32_t *t_ro32 = nullptr;
-    if (coo_group && !(create_flags & FG_GRAPH_LAZY)) group_pass1(b, by_dst, m, d_dst, d_src, nullptr, false, 0);
+    if (coo_group && !(create_flags & FG_GRAPH_LAZY)) {
+        group_pass1(b, by_dst, m, d_dst, d_src, nullptr, false, 0);
+        b.spare = &by_dst;   // until the symmetrised view is written: later allocations come first
+    }
     if (b.status == FG_OK && !(create_flags & FG_GRAPH_KEEP_IDS)) {
         indeg = b.alloc_tmp<uint32_t>(n);
         unsigned long long *bins = b.alloc_tmp<unsigned long long>(2 * kDegBins);
@@ -930,9 +954,13 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
     }
     if (by_dst.ready && !indeg) {
         indeg = b.alloc_tmp<uint32_t>(n);
-        if (b.status == FG_OK)
+        if (b.status == FG_OK && by_dst.ready) {
             b.check(cudaMemcpyAsync(indeg, by_dst.count, (size_t)n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, b.st),
                     "copy");
+        } else if (indeg) {   // given up for this allocation
+            cudaFreeAsync(indeg, b.st);
+            indeg = nullptr;
+        }
     }
     const bool relabel = b.status == FG_OK && indeg &&
                          ((create_flags & FG_GRAPH_RELABEL) || g->info.in_degree_gini > kRelabelGini);
@@ -1008,21 +1036,20 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
             }
         } else {
             uint32_t *cnt = b.alloc_tmp<uint32_t>(n);
-            uint32_t *cursor = b.alloc_tmp<uint32_t>((int64_t)n + 1);
-            uint32_t *cnt_o = g->new_of && !group ? b.alloc_tmp<uint32_t>((int64_t)n << flag) : nullptr;
             if (group) {
                 by_src.sh.flag = flag;
                 group_pass1(b, by_src, m, d_src, d_dst, d_w, true, g->light);
-                if (b.status == FG_OK) {
-                    k_part_degrees<<<grid_for(n), kBlock, 0, b.st>>>(n, by_src.count, flag, g->new_of, cnt);
-                    count_launch();
-                    b.check(exclusive_scan(cnt, ro, n, b.st), "scan");
-                    k_part_cursors<<<grid_for(n), kBlock, 0, b.st>>>(n, by_src.count, flag, ro, nullptr, g->new_of,
-                                                                     split);
-                    count_launch();
-                    group_pass2(b, by_src, m, g->new_of, col, wt);
-                    group_free(b, by_src);   // before the symmetrised view is allocated
-                }
+            }
+            uint32_t *cursor = by_src.ready || g->new_of ? nullptr : b.alloc_tmp<uint32_t>((int64_t)n + 1);
+            uint32_t *cnt_o = by_src.ready || !g->new_of ? nullptr : b.alloc_tmp<uint32_t>((int64_t)n << flag);
+            if (by_src.ready) {   // as b.status is FG_OK
+                k_part_degrees<<<grid_for(n), kBlock, 0, b.st>>>(n, by_src.count, flag, g->new_of, cnt);
+                count_launch();
+                b.check(exclusive_scan(cnt, ro, n, b.st), "scan");
+                k_part_cursors<<<grid_for(n), kBlock, 0, b.st>>>(n, by_src.count, flag, ro, nullptr, g->new_of, split);
+                count_launch();
+                group_pass2(b, by_src, m, g->new_of, col, wt);
+                by_src.release(b.st);   // before the symmetrised view is allocated
             } else if (b.status == FG_OK && g->new_of) {   // counted and scattered by original source id
                 b.check(cudaMemsetAsync(cnt_o, 0, ((size_t)n << flag) * sizeof(uint32_t), b.st), "memset");
                 if (m > 0) {
@@ -1071,8 +1098,8 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
         build_sym(b, g, indeg, &by_dst);
         g->sym_built = b.status == FG_OK;
     }
-    group_free(b, by_src);
-    group_free(b, by_dst);
+    by_src.release(b.st);
+    by_dst.release(b.st);
     if (wsum) cudaFreeAsync(wsum, b.st);
 
     if (indeg) cudaFreeAsync(indeg, b.st);
@@ -1192,31 +1219,30 @@ fg_status ensure_transpose(const fg_graph *cg) {
     uint32_t *tro = b.alloc_graph<uint32_t>((int64_t)n + 1);
     int32_t *tcol = b.alloc_graph<int32_t>(m);
     int32_t *tw = b.alloc_graph<int32_t>(m);
-    const bool group = part_usable(n, m);
-    uint32_t *cnt = group ? nullptr : b.alloc_tmp<uint32_t>(n);
-    uint32_t *cursor = group ? nullptr : b.alloc_tmp<uint32_t>((int64_t)n + 1);
-    if (group) {
+    uint32_t *cnt = b.alloc_tmp<uint32_t>(n), *cursor = nullptr;
+    Grouped q;
+    if (part_usable(n, m)) {
         // The grouping loses the order of the sources within a list, which the
         // atomic scatter roughly keeps and a BFS pull's early exit lives on
         // (hubs, the first ids of a renumbered graph, first): the first
         // sixty-fourth of the ids are flagged to come first.  R-MAT 22: a new
         // graph's first BFS 6.5 -> 2.5 ms.
-        Grouped q;
         group_alloc(b, q, n, 1);
         group_hist<false>(b, n, m, v.col, nullptr, nullptr, q, nullptr, nullptr, nullptr);
         group_pass1(b, q, m, v.col, v.src, v.w, true, n / 64, true);
-        uint32_t *deg = b.alloc_tmp<uint32_t>(n);   // then the lists' first unflagged entries
-        if (b.status == FG_OK) {
-            k_part_degrees<<<grid_for(n), kBlock, 0, b.st>>>(n, q.count, 1, nullptr, deg);
-            count_launch();
-            b.check(exclusive_scan(deg, tro, n, b.st), "scan");
-            k_part_cursors<<<grid_for(n), kBlock, 0, b.st>>>(n, q.count, 1, tro, nullptr, nullptr, deg);
-            count_launch();
-        }
+    }
+    if (q.ready) {
+        k_part_degrees<<<grid_for(n), kBlock, 0, b.st>>>(n, q.count, 1, nullptr, cnt);
+        count_launch();
+        b.check(exclusive_scan(cnt, tro, n, b.st), "scan");
+        // cnt: then the lists' first unflagged entries
+        k_part_cursors<<<grid_for(n), kBlock, 0, b.st>>>(n, q.count, 1, tro, nullptr, nullptr, cnt);
+        count_launch();
         group_pass2(b, q, m, nullptr, tcol, tw);
-        if (deg) cudaFreeAsync(deg, b.st);
-        group_free(b, q);
     } else if (b.status == FG_OK) {
+        cursor = b.alloc_tmp<uint32_t>((int64_t)n + 1);
+    }
+    if (!q.ready && b.status == FG_OK) {
         b.check(cudaMemsetAsync(cnt, 0, (size_t)n * sizeof(uint32_t), b.st), "memset");
         if (m > 0) { k_histogram<<<grid_for(m), kBlock, 0, b.st>>>(m, v.col, cnt); count_launch(); }
         b.check(exclusive_scan(cnt, tro, n, b.st), "scan");
@@ -1224,6 +1250,7 @@ fg_status ensure_transpose(const fg_graph *cg) {
         if (m > 0) { k_scatter_transpose<<<grid_for(m), kBlock, 0, b.st>>>(m, v.src, v.col, v.w, cursor, tcol, tw); count_launch(); }
         b.check(cudaGetLastError(), "transpose");
     }
+    q.release(b.st);
     if (cnt) cudaFreeAsync(cnt, b.st);
     if (cursor) cudaFreeAsync(cursor, b.st);
     View t;
