@@ -259,7 +259,10 @@ fg_status fg_select_mode(const fg_graph *g, fg_algo algo, fg_mode *out);
 /* Options and statistics of fg_run.  Zero-initialised options mean defaults. */
 typedef struct {
     void *stream;               /* cudaStream_t to run on; NULL = legacy default stream */
-    int32_t max_rounds;         /* round / generation cap; 0 = n + 2 (FG_BUCKET on split rows: 8 n + 64) */
+    int32_t max_rounds;         /* round / generation cap; 0 = n + 2 (FG_BUCKET SSSP on split rows: 8 n + 64).
+                                   With a cap below 8 n + 64, FG_BUCKET SSSP on split rows runs as on
+                                   others, and FG_AUTO does not pick it there; with one below 3 it does
+                                   not pick CC by hooking and linking */
     int32_t wait_timeout_ms;    /* bound on any single device-side wait; 0 = 1000 ms */
     int32_t blocks_per_sm;      /* persistent CTAs per SM; 0 = occupancy limit (fewer CTAs on a graph too
                                    small to give each warp 8 vertices or 64 edges) */
@@ -347,7 +350,8 @@ fg_status fg_run(const fg_graph *g, fg_algo algo, int32_t src, int32_t *out, fg_
  * ones once.
  *
  * Options: stream, max_rounds (0 = n + 2 for BFS and CC, 2 k n + 2 for
- * SSSP, whose epochs add rounds, 8 k n + 64 on split rows), wait_timeout_ms,
+ * SSSP, whose epochs add rounds, 8 k n + 64 on split rows, and with a cap
+ * below that the order of other graphs), wait_timeout_ms,
  * blocks_per_sm, delta (the SSSP width; 0 = FG_BUCKET's default);
  * the other fields are ignored.  status_out[k] (may be NULL) receives each
  * query's status: they differ only when some SSSP sources overflow

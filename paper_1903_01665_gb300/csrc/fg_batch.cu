@@ -343,7 +343,7 @@ fg_status batch_launch(const fg_query *qs, int32_t nq, const fg_batch_options *o
             p.ms_k = (int32_t)un.q.size();
             p.ms_bfs = un.algo == kBFS ? 1 : 0;
             if (un.algo == kBFS && un.g->sym_built && un.g->new_of) p.tv = un.g->s;
-            p.ms_light = ms_light_width(un.g, un.algo, 0);
+            p.ms_light = ms_light_width(un.g, un.algo, p.ms_k, 0, 0);
             p.max_rounds = ms_default_rounds(view[u]->n, p.ms_k, un.algo == kSSSP, p.ms_light > 0);
             for (size_t j = 0; j < un.q.size(); j++) {
                 p.ms_src[j] = qs[un.q[j]].src;

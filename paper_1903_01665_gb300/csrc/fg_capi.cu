@@ -91,10 +91,11 @@ fg_status check_mode(fg_mode m) {
 }
 
 // FG_AUTO: the plan's mode, and its CTAs per SM unless the caller set them
-fg_status resolve_mode(const fg_graph *g, fg_algo algo, fg_mode m, Mode *out, int32_t *blocks_per_sm) {
+fg_status resolve_mode(const fg_graph *g, fg_algo algo, fg_mode m, int32_t max_rounds, Mode *out,
+                       int32_t *blocks_per_sm) {
     if (m == FG_AUTO) {
         fg_plan pl;
-        fg_status s = fg_select_plan(g, algo, &pl);
+        fg_status s = select_plan(g, algo, !rounds_for_order((Algo)algo, g->info.n, max_rounds), &pl);
         if (s != FG_OK) return s;
         m = (fg_mode)pl.mode;
         if (blocks_per_sm && *blocks_per_sm == 0) *blocks_per_sm = pl.blocks_per_sm;
@@ -119,7 +120,7 @@ fg_status query(const fg_graph *g, fg_algo algo, int32_t src, int32_t *out, fg_m
     Mode m;
     fg_options o{};
     if (opt) o = *opt;
-    s = resolve_mode(g, algo, mode, &m, &o.blocks_per_sm);
+    s = resolve_mode(g, algo, mode, o.max_rounds, &m, &o.blocks_per_sm);
     if (s != FG_OK) return s;
     return run_query(g, (Algo)algo, m, src, out, &o, stats);
 }
@@ -260,7 +261,9 @@ namespace {
 // line is above the graphs for which edge-async is the documented pick.
 constexpr int64_t kLightHeavyMin = 1 << 17;
 
-fg_plan model_plan(const fg_graph *g, fg_algo algo, int32_t depth) {
+// few_rounds: the caller's cap on rounds is below that of the orders with a count of their own
+// (rounds_for_order): the picks are those among the modes without them.
+fg_plan model_plan(const fg_graph *g, fg_algo algo, int32_t depth, bool few_rounds) {
     const int64_t n = g->info.n, m = g->info.m;
     const bool deep = depth > 32;
     const bool skew = g->degree_gini > 0.5;
@@ -268,7 +271,7 @@ fg_plan model_plan(const fg_graph *g, fg_algo algo, int32_t depth) {
     int32_t bps;
     if (algo == FG_ALGO_SSSP) {
         mode = deep ? (n >= (1 << 21) ? FG_BUCKET : FG_VERTEX_SYNC)
-             : g->g.split && n >= kLightHeavyMin ? FG_BUCKET
+             : g->g.split && n >= kLightHeavyMin && !few_rounds ? FG_BUCKET
                     : ((skew || n >= (1 << 19)) ? FG_EDGE_ASYNC : FG_EDGE_SYNC);
         bps = m <= 3000000 ? 2 : 0;
     } else if (algo == FG_ALGO_BFS) {
@@ -280,7 +283,7 @@ fg_plan model_plan(const fg_graph *g, fg_algo algo, int32_t depth) {
         // FG_EDGE_SYNC; FG_BUCKET runs fewer CTAs, which its barriers gain by
         // on small graphs: R-MAT 16 27 against 34 us, R-MAT 22 232 against 185)
         if (deep) mode = n < (1 << 23) ? FG_PULL : FG_VERTEX_SYNC;
-        else if (!skew) mode = FG_EDGE_SYNC;
+        else if (!skew || few_rounds) mode = FG_EDGE_SYNC;
         else mode = n < (1 << 19) ? FG_BUCKET : FG_VERTEX_ASYNC;
         bps = m <= 3000000 ? 2 : 0;
     }
@@ -335,21 +338,7 @@ fg_status depth_estimate(const fg_graph *g, int32_t *out) {
 fg_status fg_select_plan(const fg_graph *g, fg_algo algo, fg_plan *out) {
     if (!g || !out) return fail(FG_ERR_INVALID_ARG, "NULL argument");
     if (algo < FG_ALGO_SSSP || algo > FG_ALGO_CC) return fail(FG_ERR_INVALID_ARG, "invalid algorithm");
-    int32_t depth = 0;
-    fg_status s = depth_estimate(g, &depth);
-    if (s != FG_OK) return s;
-    fg_plan p = model_plan(g, algo, depth);
-    {
-        std::lock_guard<std::mutex> lk(g->mu);
-        if (g->tuned_mode[algo] >= 0) {
-            p.mode = g->tuned_mode[algo];
-            p.blocks_per_sm = g->tuned_bps[algo];
-            p.delta = (p.mode == FG_BUCKET && algo == FG_ALGO_SSSP) ? bucket_width(g) : 0;
-            p.tuned = 1;
-        }
-    }
-    *out = p;
-    return FG_OK;
+    return select_plan(g, algo, false, out);
 }
 
 fg_status fg_select_mode(const fg_graph *g, fg_algo algo, fg_mode *out) {
@@ -454,3 +443,21 @@ const char *fg_status_string(fg_status s) {
 }
 
 }  // extern "C"
+
+fg_status fg::select_plan(const fg_graph *g, fg_algo algo, bool few_rounds, fg_plan *out) {
+    int32_t depth = 0;
+    fg_status s = depth_estimate(g, &depth);
+    if (s != FG_OK) return s;
+    fg_plan p = model_plan(g, algo, depth, few_rounds);
+    {
+        std::lock_guard<std::mutex> lk(g->mu);
+        if (g->tuned_mode[algo] >= 0) {
+            p.mode = g->tuned_mode[algo];
+            p.blocks_per_sm = g->tuned_bps[algo];
+            p.delta = (p.mode == FG_BUCKET && algo == FG_ALGO_SSSP) ? bucket_width(g) : 0;
+            p.tuned = 1;
+        }
+    }
+    *out = p;
+    return FG_OK;
+}

@@ -2276,8 +2276,6 @@ __device__ __forceinline__ bool cc_hook_link(const Params &p, const Team &t, con
     if (!sync_()) return false;
     return cc_compress(P, g.n, tid, nth, sync_);
 }
-constexpr int kCcHookRounds = 3;   // generations it counts as: hooks, links, the last compression
-
 // The whole query -- init, rounds, convergence -- run by one team of CTAs
 // (the full grid for a single query, a slice of it in a batch).
 // Once per kernel launch, before the first fixpoint_body: the edge-sync

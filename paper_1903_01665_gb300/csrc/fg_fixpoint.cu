@@ -289,8 +289,10 @@ int32_t ms_default_rounds(int32_t n, int k, bool near_far, bool light) {
     return cap > INT32_MAX ? INT32_MAX : (int32_t)cap;
 }
 
-int32_t ms_light_width(const fg_graph *G, Algo algo, int32_t delta) {
-    return algo == kSSSP && G->g.split ? (delta > 0 ? delta : G->light) : 0;
+int32_t ms_light_width(const fg_graph *G, Algo algo, int k, int32_t delta, int32_t max_rounds) {
+    const bool light = algo == kSSSP && G->g.split &&
+                       (max_rounds <= 0 || max_rounds >= ms_default_rounds(G->g.n, k, true, true));
+    return light ? (delta > 0 ? delta : G->light) : 0;
 }
 
 // bucket mode: 5 x the mean edge weight x the mean out-degree unless the
@@ -327,7 +329,7 @@ static int useful_grid(int grid, int sms, const View &g) {
 
 fg_status run_query(const fg_graph *G, Algo algo, Mode user_mode, int32_t source, int32_t *out,
                     const fg_options *opt, fg_stats *stats) {
-    const Mode mode = kernel_mode(G, algo, user_mode);
+    const Mode mode = kernel_mode(G, algo, user_mode, opt ? opt->max_rounds : 0);
     if (kernel_for(algo, mode)) {   // the parts of a FG_GRAPH_LAZY graph this query reads
         fg_status vs = ensure_views(G, algo, (int)mode);
         if (vs != FG_OK) return vs;
@@ -536,7 +538,7 @@ fg_status run_multi(const fg_graph *G, Algo algo, int32_t k, const int32_t *srcs
     if (algo == kBFS && G->sym_built && G->new_of) p.tv = G->s;   // its rows end with the in-edges: pull rounds
     set_relabel(G, p);
     p.delta = (opt && opt->delta > 0) ? opt->delta : default_delta(G);   // the SSSP sweep's near-far width
-    p.ms_light = ms_light_width(G, algo, opt ? opt->delta : 0);
+    p.ms_light = ms_light_width(G, algo, k, opt ? opt->delta : 0, opt ? opt->max_rounds : 0);
     int32_t *dout[kMsMax] = {};
     for (int j = 0, h = 0; j < k; j++) {
         p.ms_src[j] = srcs[j];

@@ -114,9 +114,20 @@ enum Algo { kSSSP = 0, kBFS = 1, kCC = 2, kAnyAlgo = 3 };
 // kLightHeavy: FG_BUCKET SSSP on a graph whose rows are split by weight
 enum Mode { kVertexSync = 0, kVertexAsync = 1, kEdgeSync = 2, kEdgeAsync = 3, kPull = 5, kBucket = 6, kMulti = 7,
             kLightHeavy = 8 };
+// CC by hooking and linking counts as three generations: hooks, links, the last compression
+constexpr int kCcHookRounds = 3;
+// Whether a caller's cap on rounds (0: none) leaves a query the rounds that
+// an order with a count of its own may take: the light-heavy SSSP, whose
+// generations are more and shorter, and CC by hooking.  Below that FG_BUCKET
+// SSSP runs as on graphs without split rows, so that a cap that is enough for
+// the mode's own generations stays enough, and FG_AUTO picks neither.
+int32_t round_cap(Mode mode, int32_t n);   // default cap on rounds (fg_fixpoint.cu)
+inline bool rounds_for_order(Algo algo, int32_t n, int32_t max_rounds) {
+    return max_rounds <= 0 || max_rounds >= (algo == kCC ? kCcHookRounds : round_cap(kLightHeavy, n));
+}
 // the kernel that runs a public mode on a graph, and back
-inline Mode kernel_mode(const fg_graph *g, Algo algo, Mode m) {
-    return m == kBucket && algo == kSSSP && g->g.split ? kLightHeavy : m;
+inline Mode kernel_mode(const fg_graph *g, Algo algo, Mode m, int32_t max_rounds = 0) {
+    return m == kBucket && algo == kSSSP && g->g.split && rounds_for_order(kSSSP, g->g.n, max_rounds) ? kLightHeavy : m;
 }
 inline int32_t public_mode(Mode m) { return m == kLightHeavy ? (int32_t)kBucket : (int32_t)m; }
 
@@ -526,10 +537,12 @@ fg_status ensure_transpose(const fg_graph *g);
 fg_status ensure_views(const fg_graph *g, Algo algo, int mode);
 fg_status ensure_src(const fg_graph *g);
 
+// fg_select_plan (fg_capi.cu); few_rounds: among the modes without an order of a round count of its own
+fg_status select_plan(const fg_graph *g, fg_algo algo, bool few_rounds, fg_plan *out);
+
 // queries (fg_fixpoint.cu)
 int32_t default_delta(const fg_graph *G);
 int32_t bucket_width(const fg_graph *G);   // FG_BUCKET SSSP's default width
-int32_t round_cap(Mode mode, int32_t n);   // default cap on rounds
 // renumbered graphs: an internal-order result to an output in original order
 // (device or host; CC: labels to minimum original ids).  The caller has
 // checked the result; res is left unchanged.
@@ -537,8 +550,9 @@ fg_status relabel_output(const fg_graph *G, Algo algo, const int32_t *res, int32
 // fills the relabelling fields of a query's Params from its graph
 void set_relabel(const fg_graph *G, Params &p);
 int32_t ms_default_rounds(int32_t n, int k, bool near_far, bool light);
-// the width of the light-heavy order for a multi-source SSSP sweep, 0 if the graph's rows are not split
-int32_t ms_light_width(const fg_graph *G, Algo algo, int32_t delta);
+// the width of the light-heavy order for a multi-source SSSP sweep of k sources, 0 if the graph's rows are not
+// split or the caller's cap on rounds (0: none) is below the order's own
+int32_t ms_light_width(const fg_graph *G, Algo algo, int k, int32_t delta, int32_t max_rounds);
 fg_status run_multi(const fg_graph *g, Algo algo, int32_t k, const int32_t *srcs, int32_t *const *outs,
                     const fg_options *opt, fg_status *status_out, fg_stats *stats);
 fg_status run_query(const fg_graph *g, Algo algo, Mode mode, int32_t source, int32_t *out,
