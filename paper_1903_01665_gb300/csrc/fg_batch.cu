@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "fg_batch_kernel.cuh"
+#include "fg_team_plan.cuh"
 
 namespace fg {
 
@@ -58,10 +59,6 @@ BatchFn batch_kernel_for(int kind) {
 // 1484^2, R-MAT of 2^11 to 2^20 vertices; a 1484^2 grid's SSSP: 7.6, 4.6 and
 // 3.2 ms on 152, 304 and 608 CTAs), b half as much again for the teams that
 // run beside it (a batch of 24 units: measured 1.0 to 1.6 times the fit).
-struct UnitCost {
-    double a = 0, b = 0;
-    double ms(int p) const { return a + b / p; }
-};
 UnitCost unit_cost(const BatchUnit &u, const View &v) {
     int depth;
     {
@@ -94,61 +91,6 @@ UnitCost unit_cost(const BatchUnit &u, const View &v) {
     c.a = 1e-3 * rounds * round_us;
     c.b = 1.5 * (1e-6 * visits * visit_ns + 6e-7 * rounds * scan);
     return c;
-}
-
-struct KindPlan {
-    int kind = 0;
-    std::vector<int> queries;                 // units of the batch of this kind
-    std::vector<int> class_size;              // team size per class
-    std::vector<std::vector<int>> class_q;    // units per class, largest work first
-    std::vector<int> class_teams;             // teams per class
-    int capacity = 1;                         // co-resident CTAs
-    int ctas = 0;
-};
-
-// Team sizes: 1, 2, 3, 4, 6, 8, 12, 16, ...
-int next_team(int p) { return p < 2 ? 2 : (p & (p - 1)) == 0 ? p + p / 2 : p / 3 * 4; }
-
-// Plans the teams of every kind for a common makespan T ms: each unit gets the
-// smallest team that finishes it in T, the units of one size
-// share as many teams as their times fill, and T is the smallest at which all
-// teams are resident together.  (Team sizes by edge count and CTAs by a guess
-// of the work, as before, left the longest unit of a mixed batch on a fifth
-// of the device while a third of it idled: 12 graphs, 15.6 ms.)
-void plan_teams(std::map<int, KindPlan> &kinds, const std::vector<UnitCost> &cost) {
-    double t0 = 1e30, tmax = 0;
-    for (auto &kv : kinds)
-        for (int u : kv.second.queries) tmax = std::max(tmax, cost[u].ms(kv.second.capacity));
-    t0 = std::max(tmax, 1e-3);
-    for (double T = t0;; T *= 1.06) {
-        double used = 0;
-        for (auto &kv : kinds) {
-            KindPlan &kp = kv.second;
-            std::map<int, std::vector<int>> by_size;
-            std::map<int, double> load;
-            for (int u : kp.queries) {
-                int p = 1;
-                while (p < kp.capacity && cost[u].ms(p) > T) p = std::min(kp.capacity, next_team(p));
-                by_size[p].push_back(u);
-                load[p] += cost[u].ms(p);
-            }
-            kp.class_size.clear();
-            kp.class_q.clear();
-            kp.class_teams.clear();
-            kp.ctas = 0;
-            for (auto &c : by_size) {
-                std::vector<int> v = c.second;
-                std::sort(v.begin(), v.end(), [&](int x, int y) { return cost[x].ms(c.first) > cost[y].ms(c.first); });
-                const int teams = std::min((int)v.size(), std::max(1, (int)(1.1 * load[c.first] / T + 0.999)));
-                kp.class_size.push_back(c.first);
-                kp.class_q.push_back(v);
-                kp.class_teams.push_back(teams);
-                kp.ctas += teams * c.first;
-            }
-            used += (double)kp.ctas / kp.capacity;
-        }
-        if (used <= 1.0 || T > 1e4 * t0) break;
-    }
 }
 
 }  // namespace
