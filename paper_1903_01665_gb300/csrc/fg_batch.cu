@@ -443,6 +443,10 @@ fg_status batch_finish(BatchJob &job, fg_status *status_out, fg_stats *stats_out
         else if (hc.status & kStWorklist) us = FG_ERR_CUDA;
         else if (!hc.done) us = FG_ERR_TIMEOUT;
         for (int i : un.q) qst[i] = us;
+        if (us == FG_OK && (hc.status & kStOverflow) && un.algo == kSSSP && un.mode != kMulti) {
+            us = ensure_src(un.g);   // the check reads the edge sources, which a FG_GRAPH_LAZY graph may not have yet
+            for (int i : un.q) qst[i] = us;
+        }
         if (us == FG_OK && (hc.status & kStOverflow) && un.algo == kSSSP) {
             int *flag = reinterpret_cast<int *>(p.ctrl);
             int hf = 0;
