@@ -48,6 +48,7 @@ BatchFn batch_kernel_for(int kind) {
         case kBFS * 16 + kBucket: return batch_kernel<kBFS, kBucket>;
         case kCC * 16 + kBucket: return batch_kernel<kCC, kBucket>;
         case kAnyAlgo * 16 + kMulti: return batch_kernel<kAnyAlgo, kMulti>;
+        case kSSSP * 16 + kMultiLight: return batch_kernel<kSSSP, kMultiLight>;
     }
     return nullptr;
 }
@@ -85,7 +86,10 @@ UnitCost unit_cost(const BatchUnit &u, const View &v) {
                                                              : deep                      ? 9.0
                                                                                          : 5.0);
         visit_ns = 3.5;
-        scan = u.mode == kVertexAsync || u.mode == kEdgeAsync || u.mode == kBucket ? 0 : n;
+        scan = u.mode == kVertexAsync || u.mode == kEdgeAsync || u.mode == kBucket ||
+                       u.mode == kHook || u.mode == kHookBucket
+                   ? 0
+                   : n;
     }
     UnitCost c;
     c.a = 1e-3 * rounds * round_us;
@@ -202,8 +206,12 @@ fg_status batch_launch(const fg_query *qs, int32_t nq, const fg_batch_options *o
             job.qmode[i] = un.mode;
             job.qunit[i] = u;
         }
-        // every multi-source sweep, SSSP or BFS, in one kernel (one launch)
-        const int kind = un.mode == kMulti ? kAnyAlgo * 16 + kMulti : un.algo * 16 + (int)un.mode;
+        // every multi-source sweep, SSSP or BFS, in one kernel (one launch), but for the light-heavy ones; CC by
+        // hooking goes with them
+        const bool light = un.mode == kMulti && ms_light_width(un.g, un.algo, (int)un.q.size(), 0, 0) > 0;
+        const int kind = light                                                         ? kSSSP * 16 + kMultiLight
+                         : un.mode == kMulti || un.mode == kHook || un.mode == kHookBucket ? kAnyAlgo * 16 + kMulti
+                                                                                       : un.algo * 16 + (int)un.mode;
         KindPlan &kp = kinds[kind];
         kp.kind = kind;
         kp.queries.push_back(u);
@@ -293,6 +301,7 @@ fg_status batch_launch(const fg_query *qs, int32_t nq, const fg_batch_options *o
             }
         } else {
             p.out = job.dout[un.q[0]];
+            p.cc_hook = un.mode == kHook || un.mode == kHookBucket;
         }
     }
     job.params.assign(h_params, h_params + nu);

@@ -2109,7 +2109,8 @@ constexpr int min_blocks() {
          : MODE == kEdgeSync   ? FG_EDGE_SYNC_MIN_BLOCKS
          : MODE == kPull       ? FG_PULL_MIN_BLOCKS
          : MODE == kBucket     ? (ALGO == kSSSP ? FG_BUCKET_MIN_BLOCKS : 4)
-         : MODE == kMulti      ? FG_MULTI_MIN_BLOCKS
+         : MODE == kMulti || MODE == kMultiLight ? FG_MULTI_MIN_BLOCKS
+         : MODE == kHookBucket ? 4
          : MODE == kLightHeavy ? FG_LIGHT_MIN_BLOCKS
                                : FG_ASYNC_MIN_BLOCKS;
 }
@@ -2276,6 +2277,49 @@ __device__ __forceinline__ bool cc_hook_link(const Params &p, const Team &t, con
     if (!sync_()) return false;
     return cc_compress(P, g.n, tid, nth, sync_);
 }
+
+// A CC result in internal ids to a batch's output: in original order, each
+// label the smallest original id of its component (cc_min starts at INF).
+template <class RESULT, class SYNC>
+__device__ __forceinline__ void cc_output(const Params &p, int64_t tid, int64_t nth, const RESULT &result,
+                                          const SYNC &sync_) {
+    const int32_t n = p.g.n;
+    cc_min_orig_warp(tid >> 5, nth >> 5, n, result, p.orig_of, p.cc_min);
+    if (sync_())
+        for (int64_t v = tid; v < n; v += nth) p.out[v] = ldcg(p.cc_min + result(__ldg(p.new_of + v)));
+}
+
+// The whole query in this order.
+__device__ __forceinline__ void cc_hook_body(const Params &p, const Team &t) {
+    Ctrl *c = p.ctrl;
+    const int32_t n = p.g.n;
+    const int64_t tid = t.rank * (int64_t)kBlock + threadIdx.x;
+    const int64_t nth = (int64_t)t.size * kBlock;
+    Acc a;
+    int n_barriers = 0;
+    stat_begin();
+    auto sync_ = [&](int add = 0) -> bool {
+        stat_flush(a);
+        const bool r = team_sync(t, c, p.timeout_ns, add);
+        if (tid == 0) {
+            if (p.trace && n_barriers < p.trace_cap) p.trace[n_barriers] = global_ns();
+            n_barriers++;
+        }
+        return r;
+    };
+    if (p.cc_min)
+        for (int64_t v = tid; v < n; v += nth) p.cc_min[v] = kInf;
+    if (p.inject_missing_arrival && t.rank == 0) return;   // failure-detection test
+    const bool done = cc_hook_link(p, t, p.g, a, sync_);
+    stat_report(a, c);
+    if (tid == 0) {
+        c->rounds = kCcHookRounds;
+        c->barriers = n_barriers;
+        c->done = done;
+    }
+    if (done && p.out) cc_output(p, tid, nth, [&](int64_t u) { return ldcg(p.A + u); }, sync_);
+}
+
 // The whole query -- init, rounds, convergence -- run by one team of CTAs
 // (the full grid for a single query, a slice of it in a batch).
 // Once per kernel launch, before the first fixpoint_body: the edge-sync
@@ -2314,12 +2358,8 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
 
     // the source in internal ids (a renumbered graph takes original ones)
     const int32_t source = (ALGO != kCC && p.new_of) ? __ldg(p.new_of + p.source) : p.source;
-    // components by hooking and linking: labels and everything else set there
-    const bool cc_hook = ALGO == kCC && (MODE == kVertexAsync || MODE == kBucket) && p.new_of;
     // ---- init: values, stamps, initial worklist (a2)
-    if (cc_hook && p.cc_min)
-        for (int64_t v = tid; v < n; v += nth) p.cc_min[v] = kInf;
-    for (int64_t v = cc_hook ? n : tid; v < n; v += nth) {
+    for (int64_t v = tid; v < n; v += nth) {
         int32_t x = (ALGO == kCC) ? (int32_t)v : (v == source ? 0 : kInf);
         p.A[v] = x;
         if (SYNC && ALGO != kBFS) {
@@ -2363,18 +2403,9 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
     }
     // failure-detection test: CTA 0 never arrives, the others' waits run out
     if (p.inject_missing_arrival && t.rank == 0) return;
-    bool ok = cc_hook || sync_();
+    bool ok = sync_();
 
-    if (cc_hook) {
-        if constexpr (ALGO == kCC && (MODE == kVertexAsync || MODE == kBucket)) {
-            if (p.max_rounds < kCcHookRounds) {
-                if (tid == 0) atomicOr(&c->status, kStRoundCap);
-            } else {
-                rounds = kCcHookRounds;
-                done = cc_hook_link(p, t, g, a, sync_);
-            }
-        }
-    } else if (SYNC && ok) {
+    if (SYNC && ok) {
         int64_t ch_prev = 0;     // changes of the previous round, from its barrier (the same in every thread)
         int64_t ch_before = 0;   // changes of the round before it
         constexpr bool kW = (ALGO == kSSSP);   // the edge rings carry weights for SSSP only
@@ -2717,9 +2748,7 @@ __device__ __forceinline__ void fixpoint_body(const Params &p, const Team &t, ui
             return x;
         };
         if (ALGO == kCC && p.orig_of) {
-            cc_min_orig_warp(tid >> 5, nth >> 5, n, result, p.orig_of, p.cc_min);
-            if (sync_())
-                for (int64_t v = tid; v < n; v += nth) p.out[v] = ldcg(p.cc_min + result(__ldg(p.new_of + v)));
+            cc_output(p, tid, nth, result, sync_);
         } else {
             for (int64_t v = tid; v < n; v += nth) p.out[v] = result(p.new_of ? __ldg(p.new_of + v) : v);
         }

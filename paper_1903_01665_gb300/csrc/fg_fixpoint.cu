@@ -70,7 +70,8 @@ KernelFn kernel_for(Algo algo, Mode mode) {
     FG_K(kCC, kVertexSync) FG_K(kCC, kVertexAsync) FG_K(kCC, kEdgeSync) FG_K(kCC, kEdgeAsync)
     FG_K(kSSSP, kPull) FG_K(kBFS, kPull) FG_K(kCC, kPull)
     FG_K(kSSSP, kBucket) FG_K(kBFS, kBucket) FG_K(kCC, kBucket)
-    FG_K(kSSSP, kMulti) FG_K(kBFS, kMulti) FG_K(kSSSP, kLightHeavy)
+    FG_K(kSSSP, kMulti) FG_K(kBFS, kMulti) FG_K(kSSSP, kLightHeavy) FG_K(kSSSP, kMultiLight)
+    FG_K(kCC, kHook) FG_K(kCC, kHookBucket)
 #undef FG_K
     return nullptr;
 }
@@ -206,6 +207,8 @@ size_t query_workspace_bytes(const View &g, Algo algo, Mode mode) {
     const int32_t n = g.n;
     if (mode == kLightHeavy)   // control block, distances, marks
         return Workspace::need(1, sizeof(Ctrl)) + Workspace::need(n, 4) + Workspace::need(lh_mark_bytes(n), 1);
+    if (mode == kHook || mode == kHookBucket)   // control block, labels
+        return Workspace::need(1, sizeof(Ctrl)) + Workspace::need(n, 4);
     if (mode == kMulti) {
         if (algo == kBFS)   // control block, reached-by masks, three frontier mask arrays
             return Workspace::need(1, sizeof(Ctrl)) + Workspace::need(msb_pad(n), 1) +
@@ -240,6 +243,10 @@ void carve_query_workspace(char *base, const View &g, Algo algo, Mode mode, Para
     if (mode == kLightHeavy) {
         p.A = ws.take<int32_t>(n);
         p.marks = ws.take<uint8_t>(lh_mark_bytes(n));
+        return;
+    }
+    if (mode == kHook || mode == kHookBucket) {
+        p.A = ws.take<int32_t>(n);
         return;
     }
     if (mode == kMulti) {
@@ -510,7 +517,8 @@ fg_status run_multi(const fg_graph *G, Algo algo, int32_t k, const int32_t *srcs
     if (dev != G->device) return all(fail(FG_ERR_INVALID_ARG, "the current device is not the graph's device"));
     DeviceProps dp = device_props(dev);
     if (!dp.coop) return all(fail(FG_ERR_CUDA, "device does not support cooperative launches"));
-    KernelFn fn = kernel_for(algo, kMulti);
+    const int32_t ms_light = ms_light_width(G, algo, k, opt ? opt->delta : 0, opt ? opt->max_rounds : 0);
+    KernelFn fn = kernel_for(algo, ms_light > 0 ? kMultiLight : kMulti);
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)fn, kBlock, 0);
     if (e != cudaSuccess) return all(cuda_fail(e, "occupancy query"));
@@ -538,7 +546,7 @@ fg_status run_multi(const fg_graph *G, Algo algo, int32_t k, const int32_t *srcs
     if (algo == kBFS && G->sym_built && G->new_of) p.tv = G->s;   // its rows end with the in-edges: pull rounds
     set_relabel(G, p);
     p.delta = (opt && opt->delta > 0) ? opt->delta : default_delta(G);   // the SSSP sweep's near-far width
-    p.ms_light = ms_light_width(G, algo, k, opt ? opt->delta : 0, opt ? opt->max_rounds : 0);
+    p.ms_light = ms_light;
     int32_t *dout[kMsMax] = {};
     for (int j = 0, h = 0; j < k; j++) {
         p.ms_src[j] = srcs[j];

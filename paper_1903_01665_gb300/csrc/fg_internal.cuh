@@ -112,24 +112,31 @@ enum Algo { kSSSP = 0, kBFS = 1, kCC = 2, kAnyAlgo = 3 };
 // one fixpoint); not a public fg_mode, it is reached through fg_run_multi
 // and the fusion of same-graph queries in batches and the server
 // kLightHeavy: FG_BUCKET SSSP on a graph whose rows are split by weight
+// kMultiLight: the multi-source SSSP sweep on such a graph (only chooses the kernel)
+// kHook, kHookBucket: FG_VERTEX_ASYNC and FG_BUCKET CC on a renumbered graph
 enum Mode { kVertexSync = 0, kVertexAsync = 1, kEdgeSync = 2, kEdgeAsync = 3, kPull = 5, kBucket = 6, kMulti = 7,
-            kLightHeavy = 8 };
+            kLightHeavy = 8, kMultiLight = 9, kHook = 10, kHookBucket = 11 };
 // CC by hooking and linking counts as three generations: hooks, links, the last compression
 constexpr int kCcHookRounds = 3;
 // Whether a caller's cap on rounds (0: none) leaves a query the rounds that
 // an order with a count of its own may take: the light-heavy SSSP, whose
 // generations are more and shorter, and CC by hooking.  Below that FG_BUCKET
-// SSSP runs as on graphs without split rows, so that a cap that is enough for
-// the mode's own generations stays enough, and FG_AUTO picks neither.
+// SSSP runs as on graphs without split rows and CC as on graphs in their own
+// order, so that a cap that is enough for the mode's own generations stays
+// enough, and FG_AUTO picks neither.
 int32_t round_cap(Mode mode, int32_t n);   // default cap on rounds (fg_fixpoint.cu)
 inline bool rounds_for_order(Algo algo, int32_t n, int32_t max_rounds) {
     return max_rounds <= 0 || max_rounds >= (algo == kCC ? kCcHookRounds : round_cap(kLightHeavy, n));
 }
 // the kernel that runs a public mode on a graph, and back
 inline Mode kernel_mode(const fg_graph *g, Algo algo, Mode m, int32_t max_rounds = 0) {
-    return m == kBucket && algo == kSSSP && g->g.split && rounds_for_order(kSSSP, g->g.n, max_rounds) ? kLightHeavy : m;
+    if (algo == kBFS || !rounds_for_order(algo, g->g.n, max_rounds)) return m;
+    if (algo == kSSSP) return m == kBucket && g->g.split ? kLightHeavy : m;
+    return !g->new_of ? m : m == kVertexAsync ? kHook : m == kBucket ? kHookBucket : m;
 }
-inline int32_t public_mode(Mode m) { return m == kLightHeavy ? (int32_t)kBucket : (int32_t)m; }
+inline int32_t public_mode(Mode m) {
+    return m == kLightHeavy || m == kHookBucket ? (int32_t)kBucket : m == kHook ? (int32_t)kVertexAsync : (int32_t)m;
+}
 
 // worklist classes (vertex-async): low, mid, high chunks; edge-async uses class 0 only
 enum { kWlLow = 0, kWlMid = 1, kWlHigh = 2 };
@@ -158,6 +165,7 @@ struct Params {
     int32_t *out = nullptr;                // batch: device output the team copies the result to
     int32_t ms_k = 0;                      // multi-source: sources in the sweep (A = rows of 8 values, S0 = stamps)
     int32_t ms_light = 0;                  // multi-source SSSP: the light-heavy order's first width (0: plain near-far)
+    int32_t cc_hook = 0;                   // batch: CC by hooking, in the kernel of the multi-source sweeps
     int32_t ms_bfs = 0;                    // multi-source: unit weights (BFS levels)
     int32_t ms_src[8] = {};                // multi-source: source of each slot
     int32_t *ms_out[8] = {};               // multi-source: device output of each slot (null: not written)

@@ -818,6 +818,62 @@ __device__ __forceinline__ bool ml_sweep(const Params &p, const Team &t, const i
     }
 }
 
+// Rows at INF but the sources' own slots.
+__device__ __forceinline__ bool ms_init_row(int32_t *D, int64_t v, const int32_t (&msrc)[kMsMax]) {
+    int32_t x[kMsMax];
+    bool src = false;
+#pragma unroll
+    for (int s = 0; s < kMsMax; s++) {
+        const bool mine = msrc[s] == (int32_t)v;
+        x[s] = mine ? 0 : kInf;
+        src |= mine;
+    }
+    int4 *row = reinterpret_cast<int4 *>(D + (size_t)v * kMsMax);
+    row[0] = make_int4(x[0], x[1], x[2], x[3]);
+    row[1] = make_int4(x[4], x[5], x[6], x[7]);
+    return src;
+}
+// Slot s of every row to source s's output, in original order.
+__device__ __forceinline__ void ms_write(const Params &p, int64_t tid, int64_t nth) {
+    for (int64_t v = tid; v < p.g.n; v += nth) {
+        int32_t x[kMsMax];
+        ms_load_row(p.A + (size_t)(p.new_of ? __ldg(p.new_of + v) : v) * kMsMax, x, true);
+#pragma unroll
+        for (int s = 0; s < kMsMax; s++)
+            if (s < p.ms_k && p.ms_out[s]) p.ms_out[s][v] = x[s];
+    }
+}
+
+// The whole multi-source SSSP in the light-heavy order.
+__device__ __forceinline__ void ml_body(const Params &p, const Team &t) {
+    Ctrl *c = p.ctrl;
+    const int32_t n = p.g.n;
+    const int64_t tid = t.rank * (int64_t)kBlock + threadIdx.x;
+    const int64_t nth = (int64_t)t.size * kBlock;
+    Acc a;
+    int rounds = 0, n_barriers = 0, splits = 0;
+    stat_begin();
+    auto sync_ = [&](int add = 0) -> bool {
+        stat_flush(a);
+        const bool ok = team_sync(t, c, p.timeout_ns, add);
+        n_barriers++;
+        return ok;
+    };
+    int32_t msrc[kMsMax];
+    ms_internal_sources(p, p.ms_k, msrc);
+    for (int64_t v = tid; v < n; v += nth) ms_init_row(p.A, v, msrc);
+    const bool done = ml_sweep(p, t, msrc, a, rounds, splits, sync_);
+    stat_report(a, c);
+    if (tid == 0) {
+        c->rounds = rounds;
+        c->barriers = n_barriers;
+        c->done = done;
+        c->splits = splits;
+    }
+    // (the last barrier made the overflow bit visible to every CTA)
+    if (done && !(__ldcg(&c->status) & kStOverflow)) ms_write(p, tid, nth);
+}
+
 // The whole multi-source query run by one team: init, rounds until one
 // lowers nothing and no vertex is far-pending, then the rows are written out
 // per source (unless a candidate overflowed: the host then checks which
@@ -846,21 +902,8 @@ __device__ __forceinline__ void multi_body(const Params &p, const Team &t) {
     int32_t msrc[kMsMax];
     ms_internal_sources(p, k, msrc);
     for (int64_t v = tid; v < n; v += nth) {
-        int32_t x[kMsMax];
-        bool src = false;
-#pragma unroll
-        for (int s = 0; s < kMsMax; s++) {
-            const bool mine = msrc[s] == (int32_t)v;
-            x[s] = mine ? 0 : kInf;
-            src |= mine;
-        }
-        int4 *row = reinterpret_cast<int4 *>(D + (size_t)v * kMsMax);
-        row[0] = make_int4(x[0], x[1], x[2], x[3]);
-        row[1] = make_int4(x[4], x[5], x[6], x[7]);
-        if (!p.ms_light) {
-            stamp[v] = src ? 1 : 0;
-            p.far_mark[v] = 0;   // rounds start at 1
-        }
+        stamp[v] = ms_init_row(D, v, msrc) ? 1 : 0;
+        p.far_mark[v] = 0;   // rounds start at 1
     }
     if (tid == 0)
         for (int e = 0; e < 3; e++) c->far_min[e] = kInf;
@@ -872,12 +915,7 @@ __device__ __forceinline__ void multi_body(const Params &p, const Team &t) {
         s_epoch0 = 1;
         s_splits = 0;
     }
-    if (p.ms_light) {
-        int splits = 0;
-        done = ml_sweep(p, t, msrc, a, rounds, splits, sync_);
-        if (threadIdx.x == 0) s_splits = splits;
-    }
-    bool ok = !p.ms_light && sync_();
+    bool ok = sync_();
     for (int r = 1; ok; r++) {
         if (r > p.max_rounds) {
             if (tid == 0) atomicOr(&c->status, kStRoundCap);
@@ -948,15 +986,7 @@ __device__ __forceinline__ void multi_body(const Params &p, const Team &t) {
     }
     // ---- results: slot s of every row to source s's output, in original
     // order (the barrier above made the overflow bit visible to every CTA)
-    if (done && !(__ldcg(&c->status) & kStOverflow)) {
-        for (int64_t v = tid; v < n; v += nth) {
-            int32_t x[kMsMax];
-            ms_load_row(D + (size_t)(p.new_of ? __ldg(p.new_of + v) : v) * kMsMax, x, true);
-#pragma unroll
-            for (int s = 0; s < kMsMax; s++)
-                if (s < k && p.ms_out[s]) p.ms_out[s][v] = x[s];
-        }
-    }
+    if (done && !(__ldcg(&c->status) & kStOverflow)) ms_write(p, tid, nth);
 }
 
 // Overflow test of a multi-source sweep: source s overflowed iff some edge
@@ -1386,20 +1416,29 @@ __device__ __forceinline__ void multi_bfs_body(const Params &p, const Team &t) {
     }
 }
 
-// A query of either kind, as the kernels run it.
+// A query of any kind, as the kernels run it.  Orders that share nothing but
+// the call have kernels of their own: the light-heavy sweep inlined beside the
+// near-far one made that one spill 752 bytes (48 without it), hooking beside
+// propagation the vertex-async CC 124 instead of 28.  In a batch, hooking
+// shares the sweeps' kernel, which has the registers for it.
 template <int ALGO, int MODE>
 __device__ __forceinline__ void query_body(const Params &p, const Team &t, uint32_t &ring_used) {
     if constexpr (MODE == kLightHeavy) {
         light_heavy_body(p, t);
     } else if constexpr (MODE == kMulti) {
         if constexpr (ALGO == kAnyAlgo) {
-            if (p.ms_bfs) multi_bfs_body(p, t);
+            if (p.cc_hook) cc_hook_body(p, t);
+            else if (p.ms_bfs) multi_bfs_body(p, t);
             else multi_body<kSSSP>(p, t);
         } else if constexpr (ALGO == kBFS) {
             multi_bfs_body(p, t);
         } else if constexpr (ALGO == kSSSP) {
             multi_body<kSSSP>(p, t);
         }
+    } else if constexpr (MODE == kMultiLight) {
+        ml_body(p, t);
+    } else if constexpr (MODE == kHook || MODE == kHookBucket) {
+        cc_hook_body(p, t);
     } else {
         fixpoint_body<ALGO, MODE>(p, t, ring_used);
     }
