@@ -261,8 +261,8 @@ typedef struct {
     void *stream;               /* cudaStream_t to run on; NULL = legacy default stream */
     int32_t max_rounds;         /* round / generation cap; 0 = n + 2 (FG_BUCKET SSSP on split rows: 8 n + 64).
                                    With a cap below 8 n + 64, FG_BUCKET SSSP on split rows runs as on
-                                   others, and FG_AUTO does not pick it there; with one below 3 CC
-                                   does without hooking and linking */
+                                   others, and FG_AUTO does not pick it there; with one below 3 it does
+                                   not pick CC by hooking and linking */
     int32_t wait_timeout_ms;    /* bound on any single device-side wait; 0 = 1000 ms */
     int32_t blocks_per_sm;      /* persistent CTAs per SM; 0 = occupancy limit (fewer CTAs on a graph too
                                    small to give each warp 8 vertices or 64 edges) */
@@ -347,7 +347,8 @@ fg_status fg_run(const fg_graph *g, fg_algo algo, int32_t src, int32_t *out, fg_
  *
  * On a renumbered graph with split rows (FG_BUCKET above) the light edges of
  * all sources go first, each source below its own threshold, then the heavy
- * ones once.
+ * ones once: from 2^20 vertices on where at most two fifths of the edges are
+ * light, from 2^24 in any case, and with a width (delta) of the caller's.
  *
  * Options: stream, max_rounds (0 = n + 2 for BFS and CC, 2 k n + 2 for
  * SSSP, whose epochs add rounds, 8 k n + 64 on split rows, and with a cap

@@ -90,6 +90,16 @@ __global__ void k_weight_sum(int64_t m, const int32_t *__restrict__ w, unsigned 
     if ((threadIdx.x & 31) == 0 && x) atomicAdd(sum, x);
 }
 
+// Edges in the light parts of the rows.
+__global__ void k_light_edges(int32_t n, const uint32_t *__restrict__ ro, const uint32_t *__restrict__ split,
+                              unsigned long long *sum) {
+    unsigned long long x = 0;
+    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
+        x += split[v] - ro[v];
+    x = warp_sum(x);
+    if (x && lane_id() == 0) atomicAdd(sum, x);
+}
+
 // Out-degree histogram in power-of-two bins (bin 0: no out-edge; bin k:
 // degrees in [2^(k-1), 2^k)) with each bin's degree sum: the Lorenz curve of
 // the degree distribution, from which the host forms a Gini coefficient.
@@ -1120,7 +1130,7 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
     }
     {   // mean weight (the bucket mode's default width) and the degree bins
         // (the selection model's skew measure), in one small allocation
-        unsigned long long *d_sum = nullptr, h[1 + 2 * kDegBins] = {};
+        unsigned long long *d_sum = nullptr, h[2 + 2 * kDegBins] = {};   // the last: light edges
         cudaError_t e = cudaMalloc(&d_sum, sizeof(h));
         if (e == cudaSuccess) e = cudaMemset(d_sum, 0, sizeof(h));
         if (e == cudaSuccess && m > 0 && !mean_known) {
@@ -1130,6 +1140,10 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
         if (e == cudaSuccess) {
             k_degree_bins<true><<<grid_for(n), kBlock>>>(n, v.row_off, d_sum + 1, d_sum + 1 + kDegBins);
             count_launch();
+            if (split) {
+                k_light_edges<<<grid_for(n), kBlock>>>(n, v.row_off, split, d_sum + 1 + 2 * kDegBins);
+                count_launch();
+            }
             e = cudaMemcpy(h, d_sum, sizeof(h), cudaMemcpyDeviceToHost);
         }
         if (d_sum) cudaFree(d_sum);
@@ -1141,6 +1155,7 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
         if (mean_known) h[0] = w ? weights : (unsigned long long)m;
         if (m > 0) g->w_mean = (double)h[0] / (double)m;
         g->degree_gini = gini_of_bins(h + 1, h + 1 + kDegBins);
+        if (m > 0) g->light_share = (double)h[1 + 2 * kDegBins] / (double)m;
     }
     fg_graph_info_t &I = g->info;
     I.n = n;

@@ -2310,10 +2310,12 @@ __device__ __forceinline__ void cc_hook_body(const Params &p, const Team &t) {
     if (p.cc_min)
         for (int64_t v = tid; v < n; v += nth) p.cc_min[v] = kInf;
     if (p.inject_missing_arrival && t.rank == 0) return;   // failure-detection test
-    const bool done = cc_hook_link(p, t, p.g, a, sync_);
+    const bool cap = p.max_rounds < kCcHookRounds;
+    if (cap && tid == 0) atomicOr(&c->status, kStRoundCap);
+    const bool done = !cap && cc_hook_link(p, t, p.g, a, sync_);
     stat_report(a, c);
     if (tid == 0) {
-        c->rounds = kCcHookRounds;
+        c->rounds = cap ? 0 : kCcHookRounds;
         c->barriers = n_barriers;
         c->done = done;
     }

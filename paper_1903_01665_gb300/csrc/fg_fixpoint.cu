@@ -296,8 +296,22 @@ int32_t ms_default_rounds(int32_t n, int k, bool near_far, bool light) {
     return cap > INT32_MAX ? INT32_MAX : (int32_t)cap;
 }
 
+// A sweep of several sources takes the light-heavy order from 2^20 vertices on
+// where at most two fifths of the edges are light, else from 2^24: its barriers
+// lose on small graphs, and edges that are half light are relaxed as often as
+// in the near-far order.  Light-heavy against near-far, 2 and 8 sources on
+// R-MAT with weights U[1,1000] (6 % light): scale 18 0.76 / 0.68 and 1.11 / 0.89
+// ms, scale 20 0.70 / 1.39 and 1.63 / 1.86, scale 24 8.2 / 13.8 and 11.4 / 18.4.
+// Exponential and Pareto weights (12 and 37 %): 0.64 to 1.07 of the near-far
+// time from scale 20 on.  Log-normal ones and ones of two values (48 and 50 %):
+// 0.77 to 1.64 of it at scales 20 to 23, more than it at 19 of 24 points, 0.75 to 1.04
+// at 24.  A width of the caller's is the light-heavy order's.
+constexpr int32_t kMultiLightMin = 1 << 20, kMultiLightAny = 1 << 24;
+constexpr double kMultiLightShare = 0.4;
 int32_t ms_light_width(const fg_graph *G, Algo algo, int k, int32_t delta, int32_t max_rounds) {
-    const bool light = algo == kSSSP && G->g.split &&
+    const bool pays = delta > 0 || G->g.n >= kMultiLightAny ||
+                      (G->g.n >= kMultiLightMin && G->light_share <= kMultiLightShare);
+    const bool light = algo == kSSSP && pays && G->g.split &&
                        (max_rounds <= 0 || max_rounds >= ms_default_rounds(G->g.n, k, true, true));
     return light ? (delta > 0 ? delta : G->light) : 0;
 }

@@ -65,6 +65,7 @@ struct fg_graph {
     mutable std::mutex mu;
     mutable int32_t diam_est = -1;
     int32_t light = 0;          // edges below this weight come first in their row (0: rows are not split)
+    double light_share = 0.0;   // edges below it, of all
     double w_mean = 1.0;        // mean edge weight (bucket mode's default width)
     double degree_gini = 0.0;   // Gini coefficient of the out-degrees (the selection model's skew)
     // renumbered vertices (by in-degree class), else null: every view holds
@@ -121,18 +122,17 @@ constexpr int kCcHookRounds = 3;
 // Whether a caller's cap on rounds (0: none) leaves a query the rounds that
 // an order with a count of its own may take: the light-heavy SSSP, whose
 // generations are more and shorter, and CC by hooking.  Below that FG_BUCKET
-// SSSP runs as on graphs without split rows and CC as on graphs in their own
-// order, so that a cap that is enough for the mode's own generations stays
-// enough, and FG_AUTO picks neither.
+// SSSP runs as on graphs without split rows, so that a cap that is enough for
+// the mode's own generations stays enough, and FG_AUTO picks neither.
 int32_t round_cap(Mode mode, int32_t n);   // default cap on rounds (fg_fixpoint.cu)
 inline bool rounds_for_order(Algo algo, int32_t n, int32_t max_rounds) {
     return max_rounds <= 0 || max_rounds >= (algo == kCC ? kCcHookRounds : round_cap(kLightHeavy, n));
 }
 // the kernel that runs a public mode on a graph, and back
 inline Mode kernel_mode(const fg_graph *g, Algo algo, Mode m, int32_t max_rounds = 0) {
-    if (algo == kBFS || !rounds_for_order(algo, g->g.n, max_rounds)) return m;
-    if (algo == kSSSP) return m == kBucket && g->g.split ? kLightHeavy : m;
-    return !g->new_of ? m : m == kVertexAsync ? kHook : m == kBucket ? kHookBucket : m;
+    if (algo == kSSSP) return m == kBucket && g->g.split && rounds_for_order(kSSSP, g->g.n, max_rounds) ? kLightHeavy : m;
+    if (algo == kCC && g->new_of) return m == kVertexAsync ? kHook : m == kBucket ? kHookBucket : m;
+    return m;
 }
 inline int32_t public_mode(Mode m) {
     return m == kLightHeavy || m == kHookBucket ? (int32_t)kBucket : m == kHook ? (int32_t)kVertexAsync : (int32_t)m;
