@@ -927,7 +927,7 @@ __device__ __forceinline__ int block_compact(bool offer, int32_t idx, int32_t *s
 // low vertices by threads with the warp's edges redistributed over its lanes.
 // Activity is tested for many items at once (256 chunks per CTA, 32 mid
 // vertices per warp) so that inactive items cost one parallel load.
-template <class OP, class PUSH>
+template <bool SHORT_LIST = true, class OP, class PUSH>
 __device__ __forceinline__ void expand_vertices(const Team &t, const uint32_t *__restrict__ row_off, const int32_t *__restrict__ col,
                                                 const int32_t *low, int n_low, const int32_t *mid, int n_mid,
                                                 const int2 *high, int n_high, const OP &op, const PUSH &push,
@@ -1015,8 +1015,9 @@ __device__ __forceinline__ void expand_vertices(const Team &t, const uint32_t *_
         }
     }
     // low-degree vertices: a thread each, edges redistributed over the warp
-    // (8 or 16 vertices a warp when the list is short, as in scan_step)
-    const int step = n_low > nw * 16 ? 32 : n_low > nw * 8 ? 16 : 8;
+    // (8 or 16 vertices a warp when the list is short, as in scan_step, unless the
+    // caller knows that it is not)
+    const int step = !SHORT_LIST || n_low > nw * 16 ? 32 : n_low > nw * 8 ? 16 : 8;
     for (int base = gw * step; base < n_low; base += nw * step) {
         int i = base + (int)lane;
         int32_t vv = 0, u = 0;

@@ -24,17 +24,20 @@ __global__ void __launch_bounds__(kBlock, min_blocks<ALGO, MODE>()) fixpoint_ker
 // vertex variant is held to 32 registers, 8 CTAs per SM: all 64 warps of an
 // SM in flight for its latency-bound gathers (at 40 registers, 6 CTAs, its
 // all-active round ran 3 % slower under ncu); the edge variant keeps 6 CTAs
-// at 40 registers.
+// at 40 registers.  SHORT: the low class's list is short enough for fewer than
+// 32 vertices a warp step; that choice inside one kernel costs it a spill
+// (2 M uniform vertices 103 -> 111 us), and its lack a small graph a fifth
+// (R-MAT 14 20 -> 24 us).
 constexpr unsigned long long kSweepTimeoutNs = 2000000000ull;
-template <int MODE>
+template <int MODE, bool SHORT>
 __global__ void __launch_bounds__(kBlock, MODE == kVertexSync ? 8 : 6)
     sweep_kernel(View g, const int32_t *cur, int32_t *next, Ctrl *c) {
     const Team t{(int)blockIdx.x, (int)gridDim.x, nullptr};
     Acc a;
     SweepOp op{g.w, cur, next};
     if constexpr (MODE == kVertexSync) {
-        expand_vertices(t, g.row_off, g.col, g.low, g.n_low, g.mid, g.n_mid, g.high, g.n_high_chunks, op, NoPush{},
-                        a);
+        expand_vertices<SHORT>(t, g.row_off, g.col, g.low, g.n_low, g.mid, g.n_mid, g.high, g.n_high_chunks, op,
+                               NoPush{}, a);
     } else {
         uint32_t used = 0;
         rings_init(edge_rings<true>());
@@ -691,13 +694,15 @@ fg_status run_sweep(const fg_graph *G, Mode mode, const int32_t *cur, int32_t *n
         cur = icur;
         next = inext;
     }
-    auto fn = (mode == kVertexSync) ? sweep_kernel<kVertexSync> : sweep_kernel<kEdgeSync>;
+    auto fn = (mode == kVertexSync) ? sweep_kernel<kVertexSync, false> : sweep_kernel<kEdgeSync, false>;
     int per_sm = 0;
 #ifdef FG_L1_CARVEOUT
     cudaFuncSetAttribute((const void *)fn, cudaFuncAttributePreferredSharedMemoryCarveout, FG_L1_CARVEOUT);
 #endif
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)fn, kBlock, 0);
     int grid = std::max(1, per_sm * dp.sms);
+    // (held to the same registers: as many CTAs)
+    if (mode == kVertexSync && g.n_low <= (int64_t)grid * kWarps * 16) fn = sweep_kernel<kVertexSync, true>;
     Ctrl *c = nullptr;
     cudaError_t e = cudaMallocAsync((void **)&c, sizeof(Ctrl), st);
     if (e != cudaSuccess) {
