@@ -1,5 +1,6 @@
 """Which order a multi-source SSSP sweep takes on a renumbered graph: light edges first on large graphs whose edges are
-mostly heavy, near-far (what a cap below the other order's rounds selects) on small ones and where half are light."""
+mostly heavy, near-far on small ones and where half are light.  In a batch the near-far sweeps share a launch with the
+BFS ones, the others have their own."""
 import numpy as np
 import pytest
 
@@ -17,14 +18,12 @@ def test_order(scale, weights, light):
     if weights == "two values":
         rng = np.random.Generator(np.random.PCG64(1))
         g = gg.Graph(g.n, g.src, g.dst, np.where(rng.random(g.src.size) < 0.5, 1, 10000), "two")
-    srcs = [int(s) for s in gg.sources(g, 4, seed=2)]
+    srcs = [int(s) for s in gg.sources(g, 2, seed=2)]
     with graph_handle(g, where="device") as h:
-        def sweep(**kw):
-            outs = [make_out(g.n, "device") for _ in srcs]
-            st, _, stats = fg.fg_run_multi(h, fg.FG_ALGO_SSSP, srcs, outs, **kw)
-            fg.check(st)
-            for o, s in zip(outs, srcs):
-                np.testing.assert_array_equal(as_numpy(o), run(h, g.n, fg.FG_ALGO_SSSP, s, fg.FG_VERTEX_SYNC)[0])
-            return stats.rounds
-        own, near_far = sweep(), sweep(max_rounds=8 * 4 * g.n + 63)
-        assert (own > 1.5 * near_far) == light
+        qs = [(h, algo, s, make_out(g.n, "device"), fg.FG_VERTEX_SYNC)
+              for algo in (fg.FG_ALGO_SSSP, fg.FG_ALGO_BFS) for s in srcs]
+        st, _, _, bst = fg.fg_run_batch(qs, fuse_same_graph=True)
+        fg.check(st)
+        for _, algo, s, out, mode in qs:
+            np.testing.assert_array_equal(as_numpy(out), run(h, g.n, algo, s, mode)[0])
+        assert bst.launches == (2 if light else 1)
