@@ -51,7 +51,10 @@
  *                   vertex below T changes, then the heavy ones of the
  *                   vertices that did, each once; T moves on when that
  *                   lowers nothing below it, and the last quarter of the edges
- *                   runs without a threshold.
+ *                   runs without a threshold.  Not on a graph known to be deep
+ *                   (fg_select_plan's estimate, or the last query's rounds): a
+ *                   query that reaches 128 such generations without a width of
+ *                   the caller's is run again in the near-far order.
  *
  * All reach the same unique fixpoint, so their outputs are identical.
  *
@@ -229,8 +232,8 @@ fg_status fg_cc(const fg_graph *g, int32_t *label_out, fg_mode mode);
  * R-MAT, grid and uniform random graphs of 2^10 to 2^24 vertices (deep = more
  * than 32 levels, skewed = Gini above 0.5):
  *   SSSP  deep: FG_BUCKET from 2^21 vertices, else FG_VERTEX_SYNC;
- *         shallow: FG_BUCKET from 2^17 vertices if the rows are split into
- *         light and heavy edges, else FG_EDGE_ASYNC if skewed or from 2^19
+ *         shallow: FG_BUCKET from 2^17 vertices if it takes light edges first,
+ *         else FG_EDGE_ASYNC if skewed or from 2^19
  *         vertices, else FG_EDGE_SYNC;
  *   BFS   deep: FG_BUCKET from 2^21 vertices, else FG_VERTEX_SYNC;
  *         shallow: FG_PULL if skewed, else FG_VERTEX_SYNC;

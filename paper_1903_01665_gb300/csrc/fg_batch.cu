@@ -68,7 +68,7 @@ UnitCost unit_cost(const BatchUnit &u, const View &v) {
     }
     const bool skew = u.g->degree_gini > 0.5;
     if (depth < 0) depth = skew ? 10 : 100;
-    const bool deep = depth > 32;
+    const bool deep = depth > kDeepLevels;
     const double k = (double)u.q.size(), m = (double)v.m, n = (double)v.n;
     double rounds, round_us, visits, visit_ns, scan;   // scan: vertices' words read per round, in int32
     if (u.mode == kMulti) {
@@ -199,6 +199,7 @@ fg_status batch_launch(const fg_query *qs, int32_t nq, const fg_batch_options *o
     job.qunit.assign(nq, 0);
     std::map<int, KindPlan> kinds;
     std::vector<UnitCost> cost(nu);
+    std::vector<int32_t> light(nu, 0);   // a fused SSSP sweep's first width in the light-heavy order
     for (int u = 0; u < nu; u++) {
         const BatchUnit &un = units[u];
         view[u] = (un.algo == kCC) ? &un.g->s : &un.g->g;
@@ -208,8 +209,8 @@ fg_status batch_launch(const fg_query *qs, int32_t nq, const fg_batch_options *o
         }
         // every multi-source sweep, SSSP or BFS, in one kernel (one launch), but for the light-heavy ones; CC by
         // hooking goes with them
-        const bool light = un.mode == kMulti && ms_light_width(un.g, un.algo, (int)un.q.size(), 0, 0) > 0;
-        const int kind = light                                                         ? kSSSP * 16 + kMultiLight
+        if (un.mode == kMulti) light[u] = ms_light_width(un.g, un.algo, (int)un.q.size(), 0, 0);
+        const int kind = light[u]                                                       ? kSSSP * 16 + kMultiLight
                          : un.mode == kMulti || un.mode == kHook || un.mode == kHookBucket ? kAnyAlgo * 16 + kMulti
                                                                                        : un.algo * 16 + (int)un.mode;
         KindPlan &kp = kinds[kind];
@@ -284,7 +285,8 @@ fg_status batch_launch(const fg_query *qs, int32_t nq, const fg_batch_options *o
         const BatchUnit &un = units[u];
         Params &p = h_params[u];
         if (un.mode == kPull) p.tv = (un.algo == kCC) ? un.g->s : un.g->t;
-        p.delta = un.mode == kLightHeavy ? bucket_width(un.g) : default_delta(un.g);
+        p.delta = un.mode == kLightHeavy ? un.g->light : default_delta(un.g);
+        p.light_rounds = kLightRounds;
         p.ctrl = job.d_ctrls + u;
         p.source = un.algo == kCC ? 0 : qs[un.q[0]].src;
         p.max_rounds = round_cap(un.mode, view[u]->n);
@@ -293,7 +295,7 @@ fg_status batch_launch(const fg_query *qs, int32_t nq, const fg_batch_options *o
             p.ms_k = (int32_t)un.q.size();
             p.ms_bfs = un.algo == kBFS ? 1 : 0;
             if (un.algo == kBFS && un.g->sym_built && un.g->new_of) p.tv = un.g->s;
-            p.ms_light = ms_light_width(un.g, un.algo, p.ms_k, 0, 0);
+            p.ms_light = light[u];
             p.max_rounds = ms_default_rounds(view[u]->n, p.ms_k, un.algo == kSSSP, p.ms_light > 0);
             for (size_t j = 0; j < un.q.size(); j++) {
                 p.ms_src[j] = qs[un.q[j]].src;
@@ -440,6 +442,7 @@ fg_status batch_finish(BatchJob &job, fg_status *status_out, fg_stats *stats_out
     float ms = 0.f;
     if (job.status == FG_OK && job.ev0 && job.ev1) cudaEventElapsedTime(&ms, job.ev0, job.ev1);
     std::vector<fg_status> qst(nq, FG_OK);
+    std::vector<int> again;   // units whose light-heavy order reached its limit of generations
     for (int u = 0; u < nu && job.status == FG_OK; u++) {
         const Ctrl &hc = job.h_ctrls[u];
         const BatchUnit &un = job.units[u];
@@ -450,7 +453,10 @@ fg_status batch_finish(BatchJob &job, fg_status *status_out, fg_stats *stats_out
         if (hc.status & kStTimeout) us = FG_ERR_TIMEOUT;
         else if (hc.status & kStRoundCap) us = FG_ERR_TIMEOUT;
         else if (hc.status & kStWorklist) us = FG_ERR_CUDA;
-        else if (!hc.done) us = FG_ERR_TIMEOUT;
+        else if (hc.status & kStLong) {
+            again.push_back(u);
+            continue;
+        } else if (!hc.done) us = FG_ERR_TIMEOUT;
         for (int i : un.q) qst[i] = us;
         if (us == FG_OK && (hc.status & kStOverflow) && un.algo == kSSSP && un.mode != kMulti) {
             us = ensure_src(un.g);   // the check reads the edge sources, which a FG_GRAPH_LAZY graph may not have yet
@@ -515,17 +521,6 @@ fg_status batch_finish(BatchJob &job, fg_status *status_out, fg_stats *stats_out
             }
     }
     ck(cudaStreamSynchronize(st), "result copies");
-    if (job.status != FG_OK)
-        for (int i = 0; i < nq; i++) qst[i] = job.status;
-    fg_status first_err = FG_OK;
-    std::string first_msg;
-    for (int i = 0; i < nq; i++) {
-        if (status_out) status_out[i] = qst[i];
-        if (qst[i] != FG_OK && first_err == FG_OK) {
-            first_err = qst[i];
-            first_msg = "batch query " + std::to_string(i) + " failed: " + fg_status_string(qst[i]);
-        }
-    }
     if (job.exec) cudaGraphExecDestroy(job.exec);
     if (job.graph) cudaGraphDestroy(job.graph);
     for (size_t k = 0; k < job.ks.size(); k++) {
@@ -543,6 +538,39 @@ fg_status batch_finish(BatchJob &job, fg_status *status_out, fg_stats *stats_out
     job.kev.clear();
     job.fork = job.ev0 = job.ev1 = job.done = nullptr;
     job.base = nullptr;
+    for (int u : again) {   // in the order of other graphs, with the batch's memory given back
+        if (job.status != FG_OK) break;
+        const BatchUnit &un = job.units[u];
+        note_order(un.g, true);
+        const int k = (int)un.q.size();
+        int32_t srcs[kMsMax], *outs[kMsMax];
+        fg_status each[kMsMax];
+        for (int j = 0; j < k; j++) {
+            srcs[j] = job.qs[un.q[j]].src;
+            outs[j] = job.qs[un.q[j]].out;
+        }
+        fg_options o{};
+        o.stream = st;
+        o.wait_timeout_ms = (int32_t)(job.params[u].timeout_ns / 1000000ull);
+        fg_stats s{};
+        if (un.mode == kMulti) run_multi(un.g, un.algo, k, srcs, outs, &o, each, &s);
+        else each[0] = run_query(un.g, un.algo, (Mode)public_mode(un.mode), srcs[0], outs[0], &o, &s);
+        for (int j = 0; j < k; j++) {
+            qst[un.q[j]] = each[un.mode == kMulti ? j : 0];
+            if (stats_out) stats_out[un.q[j]] = s;
+        }
+    }
+    if (job.status != FG_OK)
+        for (int i = 0; i < nq; i++) qst[i] = job.status;
+    fg_status first_err = FG_OK;
+    std::string first_msg;
+    for (int i = 0; i < nq; i++) {
+        if (status_out) status_out[i] = qst[i];
+        if (qst[i] != FG_OK && first_err == FG_OK) {
+            first_err = qst[i];
+            first_msg = "batch query " + std::to_string(i) + " failed: " + fg_status_string(qst[i]);
+        }
+    }
     if (bstats) {
         bstats->kernel_ms = ms;
         bstats->launches = job.launches;

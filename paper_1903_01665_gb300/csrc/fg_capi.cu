@@ -265,13 +265,13 @@ constexpr int64_t kLightHeavyMin = 1 << 17;
 // (rounds_for_order): the picks are those among the modes without them.
 fg_plan model_plan(const fg_graph *g, fg_algo algo, int32_t depth, bool few_rounds) {
     const int64_t n = g->info.n, m = g->info.m;
-    const bool deep = depth > 32;
+    const bool deep = depth > kDeepLevels;
     const bool skew = g->degree_gini > 0.5;
     fg_mode mode;
     int32_t bps;
     if (algo == FG_ALGO_SSSP) {
         mode = deep ? (n >= (1 << 21) ? FG_BUCKET : FG_VERTEX_SYNC)
-             : g->g.split && n >= kLightHeavyMin && !few_rounds ? FG_BUCKET
+             : n >= kLightHeavyMin && !few_rounds && light_order(g) ? FG_BUCKET
                     : ((skew || n >= (1 << 19)) ? FG_EDGE_ASYNC : FG_EDGE_SYNC);
         bps = m <= 3000000 ? 2 : 0;
     } else if (algo == FG_ALGO_BFS) {
@@ -449,12 +449,13 @@ fg_status fg::select_plan(const fg_graph *g, fg_algo algo, bool few_rounds, fg_p
     fg_status s = depth_estimate(g, &depth);
     if (s != FG_OK) return s;
     fg_plan p = model_plan(g, algo, depth, few_rounds);
+    const int32_t width = bucket_width(g);
     {
         std::lock_guard<std::mutex> lk(g->mu);
         if (g->tuned_mode[algo] >= 0) {
             p.mode = g->tuned_mode[algo];
             p.blocks_per_sm = g->tuned_bps[algo];
-            p.delta = (p.mode == FG_BUCKET && algo == FG_ALGO_SSSP) ? bucket_width(g) : 0;
+            p.delta = (p.mode == FG_BUCKET && algo == FG_ALGO_SSSP) ? width : 0;
             p.tuned = 1;
         }
     }

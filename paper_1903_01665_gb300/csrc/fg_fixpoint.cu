@@ -314,7 +314,7 @@ constexpr double kMultiLightShare = 0.4;
 int32_t ms_light_width(const fg_graph *G, Algo algo, int k, int32_t delta, int32_t max_rounds) {
     const bool pays = delta > 0 || G->g.n >= kMultiLightAny ||
                       (G->g.n >= kMultiLightMin && G->light_share <= kMultiLightShare);
-    const bool light = algo == kSSSP && pays && G->g.split &&
+    const bool light = algo == kSSSP && pays && light_order(G) &&
                        (max_rounds <= 0 || max_rounds >= ms_default_rounds(G->g.n, k, true, true));
     return light ? (delta > 0 ? delta : G->light) : 0;
 }
@@ -331,7 +331,7 @@ int32_t default_delta(const fg_graph *G) {
     return d >= (double)(kInf / 2) ? kInf / 2 : std::max(1, (int32_t)(d + 0.5));
 }
 
-int32_t bucket_width(const fg_graph *G) { return G->g.split ? G->light : default_delta(G); }
+int32_t bucket_width(const fg_graph *G) { return light_order(G) ? G->light : default_delta(G); }
 
 // Default round cap: a round of the synchronous modes, or a worklist
 // generation, settles at least one more hop, so n + 1 suffice.  The
@@ -392,7 +392,8 @@ fg_status run_query(const fg_graph *G, Algo algo, Mode user_mode, int32_t source
     Params p;
     carve_query_workspace(wsbase, g, algo, mode, p);
     if (mode == kPull) p.tv = (algo == kCC) ? G->s : G->t;
-    p.delta = (opt && opt->delta > 0) ? opt->delta : mode == kLightHeavy ? bucket_width(G) : default_delta(G);
+    p.delta = (opt && opt->delta > 0) ? opt->delta : mode == kLightHeavy ? G->light : default_delta(G);
+    p.light_rounds = opt && opt->delta > 0 ? 0 : kLightRounds;
     struct {
         char *base;
     } ws{wsbase};
@@ -433,7 +434,8 @@ fg_status run_query(const fg_graph *G, Algo algo, Mode user_mode, int32_t source
         cudaGetLastError();
     }
     const int32_t *result = (hc.result_in_b && p.B) ? p.B : p.A;
-    if (status == FG_OK) {
+    const bool again = status == FG_OK && (hc.status & kStLong) && !(hc.status & kStFatal);
+    if (status == FG_OK && !again) {
         if (hc.status & kStTimeout) {
             status = FG_ERR_TIMEOUT;
             msg = "a device-side wait exceeded the timeout";
@@ -468,7 +470,9 @@ fg_status run_query(const fg_graph *G, Algo algo, Mode user_mode, int32_t source
             }
         }
     }
-    if (status == FG_OK && G->new_of) {   // internal order to original order
+    if (again) {
+        // run once more below, in the order of other graphs
+    } else if (status == FG_OK && G->new_of) {   // internal order to original order
         status = relabel_output(G, algo, result, out, st);
         if (status != FG_OK) msg = fg_last_error();
     } else if (status == FG_OK) {
@@ -484,6 +488,13 @@ fg_status run_query(const fg_graph *G, Algo algo, Mode user_mode, int32_t source
     cudaEventDestroy(ev0);
     cudaEventDestroy(ev1);
     cudaFreeAsync(ws.base, st);
+    if (again) {
+        note_order(G, true);
+        status = run_query(G, algo, user_mode, source, out, opt, stats);
+        if (stats) stats->kernel_ms += ms;
+        return status;
+    }
+    if (algo == kSSSP && mode != kLightHeavy && status == FG_OK && hc.rounds <= kDeepLevels) note_order(G, false);
     if (stats) {
         stats->mode = public_mode(mode);
         stats->rounds = hc.rounds;
@@ -564,6 +575,7 @@ fg_status run_multi(const fg_graph *G, Algo algo, int32_t k, const int32_t *srcs
     set_relabel(G, p);
     p.delta = (opt && opt->delta > 0) ? opt->delta : default_delta(G);   // the SSSP sweep's near-far width
     p.ms_light = ms_light;
+    p.light_rounds = opt && opt->delta > 0 ? 0 : kLightRounds;
     int32_t *dout[kMsMax] = {};
     for (int j = 0, h = 0; j < k; j++) {
         p.ms_src[j] = srcs[j];
@@ -579,6 +591,7 @@ fg_status run_multi(const fg_graph *G, Algo algo, int32_t k, const int32_t *srcs
     cudaEventCreate(&ev1);
     fg_status status = FG_OK;
     std::string msg;
+    bool again = false;   // the light-heavy order reached its limit of generations
     Ctrl hc{};
     e = cudaMemsetAsync(p.ctrl, 0, sizeof(Ctrl), st);
     if (e == cudaSuccess) e = cudaEventRecord(ev0, st);
@@ -600,13 +613,15 @@ fg_status run_multi(const fg_graph *G, Algo algo, int32_t k, const int32_t *srcs
     } else if (hc.status & kStRoundCap) {
         status = FG_ERR_TIMEOUT;
         msg = "round cap reached before the fixpoint";
+    } else if (hc.status & kStLong) {
+        again = true;
     } else if (!hc.done) {
         status = FG_ERR_CUDA;
         msg = "internal error: the multi-source sweep ended without a fixpoint";
     }
     fg_status slot[kMsMax];
     for (int j = 0; j < kMsMax; j++) slot[j] = status;
-    if (status == FG_OK && (hc.status & kStOverflow)) {
+    if (status == FG_OK && !again && (hc.status & kStOverflow)) {
         // which sources overflowed; the kernel wrote no output, so write the others'
         int *flag = reinterpret_cast<int *>(p.ctrl);
         int hf = 0;
@@ -633,7 +648,7 @@ fg_status run_multi(const fg_graph *G, Algo algo, int32_t k, const int32_t *srcs
             msg = "a finite shortest distance is >= INT32_MAX";
         }
     }
-    for (int j = 0; j < k && e == cudaSuccess; j++)
+    for (int j = 0; j < k && e == cudaSuccess && !again; j++)
         if (slot[j] == FG_OK && !on_dev[j])
             e = cudaMemcpyAsync(outs[j], dout[j], (size_t)n * sizeof(int32_t), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -646,6 +661,13 @@ fg_status run_multi(const fg_graph *G, Algo algo, int32_t k, const int32_t *srcs
     cudaEventDestroy(ev0);
     cudaEventDestroy(ev1);
     cudaFreeAsync(base, st);
+    if (again) {   // in the order of other graphs
+        note_order(G, true);
+        status = run_multi(G, algo, k, srcs, outs, opt, status_out, stats);
+        if (stats) stats->kernel_ms += ms;
+        return status;
+    }
+    if (algo == kSSSP && ms_light == 0 && hc.done && hc.rounds <= kDeepLevels) note_order(G, false);
     if (stats) {
         *stats = fg_stats{};
         stats->mode = -1;

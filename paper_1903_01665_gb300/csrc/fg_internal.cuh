@@ -28,6 +28,7 @@ constexpr int kStTimeout = 1;          // a grid barrier wait ran out
 constexpr int kStRoundCap = 2;         // max_rounds reached
 constexpr int kStOverflow = 4;         // a candidate >= INT32_MAX was formed (checked on host)
 constexpr int kStWorklist = 8;         // a worklist append exceeded its capacity
+constexpr int kStLong = 16;            // the light-heavy order reached its limit of generations (no error: light_order)
 
 // ---------------------------------------------------------------- graph
 // One adjacency: the directed graph, or its symmetrised copy for CC.
@@ -64,6 +65,7 @@ struct fg_graph {
     // lazily computed diameter estimate and autotuned modes for fg_select_mode
     mutable std::mutex mu;
     mutable int32_t diam_est = -1;
+    mutable bool long_order = false;   // the last SSSP that told took many generations (light_order)
     int32_t light = 0;          // edges below this weight come first in their row (0: rows are not split)
     double light_share = 0.0;   // edges below it, of all
     double w_mean = 1.0;        // mean edge weight (bucket mode's default width)
@@ -109,6 +111,7 @@ struct Ctrl {
 // kAnyAlgo: a batch kernel of multi-source sweeps of either algorithm (the
 // unit's Params.ms_bfs decides)
 enum Algo { kSSSP = 0, kBFS = 1, kCC = 2, kAnyAlgo = 3 };
+constexpr int kDeepLevels = 32;   // a graph with more BFS levels is deep, to the selection model too
 // kMulti: the multi-source sweep (up to 8 SSSP or BFS sources on one graph in
 // one fixpoint); not a public fg_mode, it is reached through fg_run_multi
 // and the fusion of same-graph queries in batches and the server
@@ -128,9 +131,32 @@ int32_t round_cap(Mode mode, int32_t n);   // default cap on rounds (fg_fixpoint
 inline bool rounds_for_order(Algo algo, int32_t n, int32_t max_rounds) {
     return max_rounds <= 0 || max_rounds >= (algo == kCC ? kCcHookRounds : round_cap(kLightHeavy, n));
 }
+// Whether SSSP on a graph with split rows takes the light-heavy order.  It is
+// made for graphs whose hubs are a few hops from everything: 20 to 80 short
+// generations, each testing every vertex's mark.  A graph may have skewed
+// degrees and a long diameter all the same (an R-MAT joined to a grid, a web
+// graph's tails): then it needs hundreds of them and takes twice the time of
+// the near-far order (one source) or four times (eight): R-MAT 18 and a 500^2
+// grid 5.5 against 2.6 ms and 21.1 against 5.0.  So not on a graph that is
+// known to be deep by the depth estimate, nor after a query that reached
+// kLightRounds generations, which is then run in the near-far order, until one
+// in another order ends within the rounds of a shallow graph (a far source alone
+// does not make a graph deep).  A caller's width sets no limit.
+constexpr int kLightRounds = 128;
+inline bool light_order(const fg_graph *g) {
+    if (!g->g.split) return false;
+    std::lock_guard<std::mutex> lk(g->mu);
+    return !g->long_order && g->diam_est <= kDeepLevels;
+}
+inline void note_order(const fg_graph *g, bool is_long) {
+    if (!g->g.split) return;
+    std::lock_guard<std::mutex> lk(g->mu);
+    g->long_order = is_long;
+}
 // the kernel that runs a public mode on a graph, and back
 inline Mode kernel_mode(const fg_graph *g, Algo algo, Mode m, int32_t max_rounds = 0) {
-    if (algo == kSSSP) return m == kBucket && g->g.split && rounds_for_order(kSSSP, g->g.n, max_rounds) ? kLightHeavy : m;
+    if (algo == kSSSP)
+        return m == kBucket && rounds_for_order(kSSSP, g->g.n, max_rounds) && light_order(g) ? kLightHeavy : m;
     if (algo == kCC && g->new_of) return m == kVertexAsync ? kHook : m == kBucket ? kHookBucket : m;
     return m;
 }
@@ -164,6 +190,7 @@ struct Params {
     int32_t inject_missing_arrival = 0;
     int32_t *out = nullptr;                // batch: device output the team copies the result to
     int32_t ms_k = 0;                      // multi-source: sources in the sweep (A = rows of 8 values, S0 = stamps)
+    int32_t light_rounds = 0;              // light-heavy: generations after which the query ends with kStLong (0: none)
     int32_t ms_light = 0;                  // multi-source SSSP: the light-heavy order's first width (0: plain near-far)
     int32_t cc_hook = 0;                   // batch: CC by hooking, in the kernel of the multi-source sweeps
     int32_t ms_bfs = 0;                    // multi-source: unit weights (BFS levels)

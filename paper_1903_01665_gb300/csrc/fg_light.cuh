@@ -378,6 +378,10 @@ __device__ __forceinline__ void light_heavy_body(const Params &p, const Team &t)
             if (tid == 0) atomicOr(&c->status, kStRoundCap);
             break;
         }
+        if (p.light_rounds && work_gens >= p.light_rounds) {
+            if (tid == 0) atomicOr(&c->status, kStLong);
+            break;
+        }
         work_gens++;
         rounds++;
         const uint8_t *cur = F + (gen % 3) * np;

@@ -699,6 +699,10 @@ __device__ __forceinline__ bool ml_sweep(const Params &p, const Team &t, const i
             if (tid == 0) atomicOr(&c->status, kStRoundCap);
             return false;
         }
+        if (p.light_rounds && work >= p.light_rounds) {
+            if (tid == 0) atomicOr(&c->status, kStLong);
+            return false;
+        }
         work++;
         rounds++;
         const uint8_t *cur = F + (gen % 3) * np;
