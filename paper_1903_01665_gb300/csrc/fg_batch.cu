@@ -60,7 +60,7 @@ BatchFn batch_kernel_for(int kind) {
 // 1484^2, R-MAT of 2^11 to 2^20 vertices; a 1484^2 grid's SSSP: 7.6, 4.6 and
 // 3.2 ms on 152, 304 and 608 CTAs), b half as much again for the teams that
 // run beside it (a batch of 24 units: measured 1.0 to 1.6 times the fit).
-UnitCost unit_cost(const BatchUnit &u, const View &v) {
+UnitCost unit_cost(const BatchUnit &u, const View &v, bool light) {
     int depth;
     {
         std::lock_guard<std::mutex> lk(u.g->mu);
@@ -73,9 +73,9 @@ UnitCost unit_cost(const BatchUnit &u, const View &v) {
     double rounds, round_us, visits, visit_ns, scan;   // scan: vertices' words read per round, in int32
     if (u.mode == kMulti) {
         const bool sssp = u.algo == kSSSP;
-        rounds = sssp ? (deep ? 1.5 * depth : 40) : depth + 1;
+        rounds = sssp ? (deep ? 1.5 * depth : light ? 40 : 17) : depth + 1;
         round_us = deep ? 7 : sssp ? 20 : 12;
-        visits = m * (sssp ? (deep ? 1.2 + 2.2 * k : 2.3) : (deep ? 0.97 * k : 2.2));
+        visits = m * (sssp ? (deep ? 1.2 + 2.2 * k : light ? 2.3 : 6.0) : (deep ? 0.97 * k : 2.2));
         visit_ns = deep ? (sssp ? 7.4 : 8.7) : (sssp ? 4.9 : 2.7);
         scan = sssp ? n : n / 2;
     } else {
@@ -209,14 +209,14 @@ fg_status batch_launch(const fg_query *qs, int32_t nq, const fg_batch_options *o
         }
         // every multi-source sweep, SSSP or BFS, in one kernel (one launch), but for the light-heavy ones; CC by
         // hooking goes with them
-        if (un.mode == kMulti) light[u] = ms_light_width(un.g, un.algo, (int)un.q.size(), 0, 0);
+        if (un.mode == kMulti) light[u] = ms_light_width(un.g, un.algo, (int)un.q.size(), 0, 0, true);
         const int kind = light[u]                                                       ? kSSSP * 16 + kMultiLight
                          : un.mode == kMulti || un.mode == kHook || un.mode == kHookBucket ? kAnyAlgo * 16 + kMulti
                                                                                        : un.algo * 16 + (int)un.mode;
         KindPlan &kp = kinds[kind];
         kp.kind = kind;
         kp.queries.push_back(u);
-        cost[u] = unit_cost(un, *view[u]);
+        cost[u] = unit_cost(un, *view[u], light[u] > 0);
     }
     for (auto &kv : kinds) {
         KindPlan &kp = kv.second;

@@ -308,12 +308,15 @@ int32_t ms_default_rounds(int32_t n, int k, bool near_far, bool light) {
 // Exponential and Pareto weights (12 and 37 %): 0.64 to 1.07 of the near-far
 // time from scale 20 on.  Log-normal ones and ones of two values (48 and 50 %):
 // 0.77 to 1.64 of it at scales 20 to 23, more than it at 19 of 24 points, 0.75 to 1.04
-// at 24.  A width of the caller's is the light-heavy order's.
-constexpr int32_t kMultiLightMin = 1 << 20, kMultiLightAny = 1 << 24;
+// at 24.  A width of the caller's is the light-heavy order's.  In a batch a
+// team is a part of the device: its barriers cost less and the edges more, and
+// the order pays from 2^14 vertices on (12 graphs of 2^10 to 2^20 vertices, 96
+// queries: 7.9 ms, from 2^20 on 10.4; 12 of 2^13 to 2^18 4.2 and 5.8).
+constexpr int32_t kMultiLightMin = 1 << 20, kMultiLightBatch = 1 << 14, kMultiLightAny = 1 << 24;
 constexpr double kMultiLightShare = 0.4;
-int32_t ms_light_width(const fg_graph *G, Algo algo, int k, int32_t delta, int32_t max_rounds) {
+int32_t ms_light_width(const fg_graph *G, Algo algo, int k, int32_t delta, int32_t max_rounds, bool batch) {
     const bool pays = delta > 0 || G->g.n >= kMultiLightAny ||
-                      (G->g.n >= kMultiLightMin && G->light_share <= kMultiLightShare);
+                      (G->g.n >= (batch ? kMultiLightBatch : kMultiLightMin) && G->light_share <= kMultiLightShare);
     const bool light = algo == kSSSP && pays && light_order(G) &&
                        (max_rounds <= 0 || max_rounds >= ms_default_rounds(G->g.n, k, true, true));
     return light ? (delta > 0 ? delta : G->light) : 0;
@@ -545,7 +548,7 @@ fg_status run_multi(const fg_graph *G, Algo algo, int32_t k, const int32_t *srcs
     if (dev != G->device) return all(fail(FG_ERR_INVALID_ARG, "the current device is not the graph's device"));
     DeviceProps dp = device_props(dev);
     if (!dp.coop) return all(fail(FG_ERR_CUDA, "device does not support cooperative launches"));
-    const int32_t ms_light = ms_light_width(G, algo, k, opt ? opt->delta : 0, opt ? opt->max_rounds : 0);
+    const int32_t ms_light = ms_light_width(G, algo, k, opt ? opt->delta : 0, opt ? opt->max_rounds : 0, false);
     KernelFn fn = kernel_for(algo, ms_light > 0 ? kMultiLight : kMulti);
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)fn, kBlock, 0);

@@ -587,7 +587,7 @@ void set_relabel(const fg_graph *G, Params &p);
 int32_t ms_default_rounds(int32_t n, int k, bool near_far, bool light);
 // the width of the light-heavy order for a multi-source SSSP sweep of k sources, 0 if the graph's rows are not
 // split or the caller's cap on rounds (0: none) is below the order's own
-int32_t ms_light_width(const fg_graph *G, Algo algo, int k, int32_t delta, int32_t max_rounds);
+int32_t ms_light_width(const fg_graph *G, Algo algo, int k, int32_t delta, int32_t max_rounds, bool batch);
 fg_status run_multi(const fg_graph *g, Algo algo, int32_t k, const int32_t *srcs, int32_t *const *outs,
                     const fg_options *opt, fg_status *status_out, fg_stats *stats);
 fg_status run_query(const fg_graph *g, Algo algo, Mode mode, int32_t source, int32_t *out,
