@@ -1460,44 +1460,44 @@ __device__ __forceinline__ void pull_vertices(const Team &t, const View &tv, con
         }
 #pragma unroll
         for (int q = 0; q < kPer; q++) {
-        const int32_t v = vs[q];
-        const uint32_t rb = rbs[q], d = ds[q];
-        if (OP::kEarly && !__any_sync(0xffffffffu, d > 0)) continue;
-        s_min[wid][lane] = kInf;
-        __syncwarp();
-        const uint32_t incl = warp_inclusive_scan(d);
-        const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-        const uint32_t excl = incl - d;
-        if (lane == 0) a.pulled += total;
-        for (uint32_t k0 = 0; k0 < total; k0 += 32 * kU) {
-            int32_t u[kU], wv[kU], own[kU];
-            uint32_t e[kU];
+            const int32_t v = vs[q];
+            const uint32_t rb = rbs[q], d = ds[q];
+            if (OP::kEarly && !__any_sync(0xffffffffu, d > 0)) continue;
+            s_min[wid][lane] = kInf;
+            __syncwarp();
+            const uint32_t incl = warp_inclusive_scan(d);
+            const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+            const uint32_t excl = incl - d;
+            if (lane == 0) a.pulled += total;
+            for (uint32_t k0 = 0; k0 < total; k0 += 32 * kU) {
+                int32_t u[kU], wv[kU], own[kU];
+                uint32_t e[kU];
 #pragma unroll
-            for (int j = 0; j < kU; j++) {
-                const uint32_t k = k0 + 32 * j + lane;
-                int owner = 0;
+                for (int j = 0; j < kU; j++) {
+                    const uint32_t k = k0 + 32 * j + lane;
+                    int owner = 0;
 #pragma unroll
-                for (int step = 16; step > 0; step >>= 1) {
-                    const uint32_t pv = __shfl_sync(0xffffffffu, incl, owner + step - 1);
-                    if (pv <= k) owner += step;
+                    for (int step = 16; step > 0; step >>= 1) {
+                        const uint32_t pv = __shfl_sync(0xffffffffu, incl, owner + step - 1);
+                        if (pv <= k) owner += step;
+                    }
+                    const uint32_t ob = __shfl_sync(0xffffffffu, rb, owner);
+                    const uint32_t oe = __shfl_sync(0xffffffffu, excl, owner);
+                    own[j] = owner;
+                    e[j] = ob + (k - oe);
+                    u[j] = k < total ? ld_edge(tv.col + e[j]) : -1;
+                    wv[j] = k < total ? op.weight(e[j]) : 0;
                 }
-                const uint32_t ob = __shfl_sync(0xffffffffu, rb, owner);
-                const uint32_t oe = __shfl_sync(0xffffffffu, excl, owner);
-                own[j] = owner;
-                e[j] = ob + (k - oe);
-                u[j] = k < total ? ld_edge(tv.col + e[j]) : -1;
-                wv[j] = k < total ? op.weight(e[j]) : 0;
+#pragma unroll
+                for (int j = 0; j < kU; j++)
+                    if (u[j] >= 0) {
+                        const int32_t cnd = op.cand(u[j], wv[j], a);
+                        if (cnd != kInf) atomicMin(&s_min[wid][own[j]], cnd);
+                    }
             }
-#pragma unroll
-            for (int j = 0; j < kU; j++)
-                if (u[j] >= 0) {
-                    const int32_t cnd = op.cand(u[j], wv[j], a);
-                    if (cnd != kInf) atomicMin(&s_min[wid][own[j]], cnd);
-                }
-        }
-        __syncwarp();
-        if (d > 0) op.finish(v, s_min[wid][lane], a);
-        __syncwarp();
+            __syncwarp();
+            if (d > 0) op.finish(v, s_min[wid][lane], a);
+            __syncwarp();
         }
     }
 }
@@ -2088,6 +2088,9 @@ __device__ __forceinline__ void stream_edges_async(const Team &t, const View &g,
 #ifndef FG_BUCKET_MIN_BLOCKS
 #define FG_BUCKET_MIN_BLOCKS 3
 #endif
+#ifndef FG_BUCKET_WIDE_MIN_BLOCKS
+#define FG_BUCKET_WIDE_MIN_BLOCKS 4
+#endif
 #ifndef FG_PULL_MIN_BLOCKS
 #define FG_PULL_MIN_BLOCKS 6
 #endif
@@ -2109,9 +2112,9 @@ constexpr int min_blocks() {
     return MODE == kVertexSync ? FG_SYNC_MIN_BLOCKS
          : MODE == kEdgeSync   ? FG_EDGE_SYNC_MIN_BLOCKS
          : MODE == kPull       ? FG_PULL_MIN_BLOCKS
-         : MODE == kBucket     ? (ALGO == kSSSP ? FG_BUCKET_MIN_BLOCKS : 4)
+         : MODE == kBucket     ? (ALGO == kSSSP ? FG_BUCKET_MIN_BLOCKS : FG_BUCKET_WIDE_MIN_BLOCKS)
          : MODE == kMulti || MODE == kMultiLight ? FG_MULTI_MIN_BLOCKS
-         : MODE == kHookBucket ? 4
+         : MODE == kHookBucket ? FG_BUCKET_WIDE_MIN_BLOCKS
          : MODE == kLightHeavy ? FG_LIGHT_MIN_BLOCKS
                                : FG_ASYNC_MIN_BLOCKS;
 }
@@ -2140,7 +2143,7 @@ constexpr int min_blocks() {
 // 3, and the chains are a handful of steps.  A graph in its own order (a
 // grid) has chains as long as its side, and keeps the propagation.  The
 // walks read through L1: the big tree's root is one word that every vertex
-// asks for, and at one L2 slice those reads alone took 60 ms.  Measured on
+// asks for, and at one L2 slice those reads alone took tens of milliseconds.  Measured on
 // R-MAT 22: 1.28 -> 0.18 ms, R-MAT 16 0.11 -> 0.03 ms; it is bound by the row
 // heads' sectors (85 us) and the barriers of five short passes.
 constexpr int kCcSampleLow = 4, kCcSampleMid = 32, kCcSampleHigh = 256;   // neighbours hooked by, per degree class
