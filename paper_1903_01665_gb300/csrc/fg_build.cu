@@ -1142,7 +1142,7 @@ fg_status build_graph_from_coo(int32_t n, int64_t m, const int32_t *src, const i
             count_launch();
             if (split) {
                 // few CTAs: a warp's sum is one atomic on one word (R-MAT 22, a warp per 32 vertices: 49 us)
-                k_light_edges<<<std::min(grid_for(n), 608u), kBlock>>>(n, v.row_off, split, d_sum + 1 + 2 * kDegBins);
+                k_light_edges<<<std::min(grid_for(n), 608), kBlock>>>(n, v.row_off, split, d_sum + 1 + 2 * kDegBins);
                 count_launch();
             }
             e = cudaMemcpy(h, d_sum, sizeof(h), cudaMemcpyDeviceToHost);
