@@ -354,9 +354,11 @@ static int useful_grid(int grid, int sms, const View &g) {
     return (int)std::min<int64_t>(grid, std::max<int64_t>(std::min(sms, grid), useful));
 }
 
-fg_status run_query(const fg_graph *G, Algo algo, Mode user_mode, int32_t source, int32_t *out,
-                    const fg_options *opt, fg_stats *stats) {
-    const Mode mode = kernel_mode(G, algo, user_mode, opt ? opt->max_rounds : 0);
+// One query by one kernel.  light_rounds: the light-heavy order's limit of
+// generations, after which nothing is written and *again set (0: none).
+static fg_status run_kernel(const fg_graph *G, Algo algo, Mode mode, int32_t light_rounds, int32_t source, int32_t *out,
+                            const fg_options *opt, fg_stats *stats, bool *again) {
+    *again = false;
     if (kernel_for(algo, mode)) {   // the parts of a FG_GRAPH_LAZY graph this query reads
         fg_status vs = ensure_views(G, algo, (int)mode);
         if (vs != FG_OK) return vs;
@@ -396,7 +398,7 @@ fg_status run_query(const fg_graph *G, Algo algo, Mode user_mode, int32_t source
     carve_query_workspace(wsbase, g, algo, mode, p);
     if (mode == kPull) p.tv = (algo == kCC) ? G->s : G->t;
     p.delta = (opt && opt->delta > 0) ? opt->delta : mode == kLightHeavy ? G->light : default_delta(G);
-    p.light_rounds = opt && opt->delta > 0 ? 0 : kLightRounds;
+    p.light_rounds = light_rounds;
     struct {
         char *base;
     } ws{wsbase};
@@ -437,8 +439,8 @@ fg_status run_query(const fg_graph *G, Algo algo, Mode user_mode, int32_t source
         cudaGetLastError();
     }
     const int32_t *result = (hc.result_in_b && p.B) ? p.B : p.A;
-    const bool again = status == FG_OK && (hc.status & kStLong) && !(hc.status & kStFatal);
-    if (status == FG_OK && !again) {
+    *again = status == FG_OK && (hc.status & kStLong) && !(hc.status & kStFatal);
+    if (status == FG_OK && !*again) {
         if (hc.status & kStTimeout) {
             status = FG_ERR_TIMEOUT;
             msg = "a device-side wait exceeded the timeout";
@@ -473,8 +475,8 @@ fg_status run_query(const fg_graph *G, Algo algo, Mode user_mode, int32_t source
             }
         }
     }
-    if (again) {
-        // run once more below, in the order of other graphs
+    if (*again) {
+        // run once more, in the order of other graphs
     } else if (status == FG_OK && G->new_of) {   // internal order to original order
         status = relabel_output(G, algo, result, out, st);
         if (status != FG_OK) msg = fg_last_error();
@@ -491,12 +493,6 @@ fg_status run_query(const fg_graph *G, Algo algo, Mode user_mode, int32_t source
     cudaEventDestroy(ev0);
     cudaEventDestroy(ev1);
     cudaFreeAsync(ws.base, st);
-    if (again) {
-        note_order(G, true);
-        status = run_query(G, algo, user_mode, source, out, opt, stats);
-        if (stats) stats->kernel_ms += ms;
-        return status;
-    }
     if (algo == kSSSP && mode != kLightHeavy && status == FG_OK && hc.rounds <= kDeepLevels) note_order(G, false);
     if (stats) {
         stats->mode = public_mode(mode);
@@ -515,6 +511,27 @@ fg_status run_query(const fg_graph *G, Algo algo, Mode user_mode, int32_t source
     }
     if (status != FG_OK) return fail(status, msg);
     return FG_OK;
+}
+
+fg_status run_query(const fg_graph *G, Algo algo, Mode user_mode, int32_t source, int32_t *out,
+                    const fg_options *opt, fg_stats *stats) {
+    const int32_t max_rounds = opt ? opt->max_rounds : 0;
+    Mode mode = kernel_mode(G, algo, user_mode, max_rounds);
+    bool again = false;
+    const int32_t limit = opt && opt->delta > 0 ? 0 : kLightRounds;
+    fg_status s = run_kernel(G, algo, mode, limit, source, out, opt, stats, &again);
+    if (again) {
+        note_order(G, true);
+        const float first = stats ? stats->kernel_ms : 0.f;
+        mode = user_mode;
+        s = run_kernel(G, algo, mode, 0, source, out, opt, stats, &again);
+        if (stats) stats->kernel_ms += first;
+    }
+    // the near-far order takes three times the light-heavy one's memory: without it, the slower order
+    if (s == FG_ERR_OUT_OF_MEMORY && mode == kBucket && algo == kSSSP && G->g.split &&
+        rounds_for_order(algo, G->g.n, max_rounds))
+        s = run_kernel(G, algo, kLightHeavy, 0, source, out, opt, stats, &again);
+    return s;
 }
 
 // Up to kMsMax queries of one algorithm on one graph.  SSSP and BFS run as

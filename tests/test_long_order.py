@@ -8,6 +8,7 @@ import graphgen as gg
 import oracle
 import paper_1903_01665_gb300 as fg
 from tests.gpu_util import as_numpy, graph_handle, make_out, run
+from tests.test_build_memory import _memory_bound
 
 pytestmark = pytest.mark.gpu
 LIMIT = 128   # generations of the light-heavy order
@@ -134,3 +135,25 @@ def test_batch(deep, graph):
                 np.testing.assert_array_equal(as_numpy(o), w)
             np.testing.assert_array_equal(last, exp)
             assert all(s.mode == fg.FG_BUCKET for s in stats) and stats[-1].rounds <= LIMIT
+
+
+def test_near_far_without_the_memory_for_it(deep):
+    """The near-far order takes 28 bytes a vertex, the other 9: where only that is there, it runs after all."""
+    import torch
+    g, srcs, _ = deep
+    g = gg.Graph(6 << 20, g.src, g.dst, g.w, "deep, isolated vertices")
+    want = oracle.sssp(g.n, g.src, g.dst, g.w, srcs[0])[1]
+    with graph_handle(g, flags=fg.FG_GRAPH_RELABEL, where="device") as h:
+        st, plan = fg.fg_select_plan(h, fg.FG_ALGO_SSSP)
+        fg.check(st)
+        assert plan.depth_est > 32
+        out = make_out(g.n, "device")
+        torch.cuda.synchronize()
+        rounds = []
+        for limit in (96 << 20, 512 << 20):
+            with _memory_bound(limit):
+                st, stats = fg.fg_run(h, fg.FG_ALGO_SSSP, srcs[0], out, fg.FG_BUCKET)
+                fg.check(st)
+            rounds.append(stats.rounds)
+            np.testing.assert_array_equal(as_numpy(out), want)
+        assert rounds[0] > LIMIT > 0 and rounds[0] > rounds[1]
