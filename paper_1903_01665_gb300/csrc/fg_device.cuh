@@ -2144,8 +2144,9 @@ constexpr int min_blocks() {
 // grid) has chains as long as its side, and keeps the propagation.  The
 // walks read through L1: the big tree's root is one word that every vertex
 // asks for, and at one L2 slice those reads alone took tens of milliseconds.  Measured on
-// R-MAT 22: 1.28 -> 0.18 ms, R-MAT 16 0.11 -> 0.03 ms; it is bound by the row
-// heads' sectors (85 us) and the barriers of five short passes.
+// R-MAT 22: 1.28 -> 0.18 ms, R-MAT 16 0.11 -> 0.03 ms.  It is bound by latency:
+// 190 MB of DRAM and 17.8 M L2 sectors in 0.17 ms, a sixth of either's rate, in
+// five short passes with a barrier after each.
 constexpr int kCcSampleLow = 4, kCcSampleMid = 32, kCcSampleHigh = 256;   // neighbours hooked by, per degree class
 constexpr int kCcHubs = 4096, kCcHubSample = 64;
 

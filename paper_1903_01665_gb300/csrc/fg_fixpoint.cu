@@ -26,8 +26,8 @@ __global__ void __launch_bounds__(kBlock, min_blocks<ALGO, MODE>()) fixpoint_ker
 // all-active round ran 3 % slower under ncu); the edge variant keeps 6 CTAs
 // at 40 registers.  SHORT: the low class's list is short enough for fewer than
 // 32 vertices a warp step; that choice inside one kernel costs it a spill
-// (2 M uniform vertices 103 -> 111 us), and its lack a small graph a fifth
-// (R-MAT 14 20 -> 24 us).
+// (R-MAT 22 268 -> 266 us without it, R-MAT 20 90 -> 86, 2 M uniform vertices
+// 111 -> 108), and its lack a small graph a fifth (R-MAT 14 20 -> 24 us).
 constexpr unsigned long long kSweepTimeoutNs = 2000000000ull;
 template <int MODE, bool SHORT>
 __global__ void __launch_bounds__(kBlock, MODE == kVertexSync ? 8 : 6)

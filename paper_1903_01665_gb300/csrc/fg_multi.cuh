@@ -391,11 +391,13 @@ __device__ __forceinline__ int32_t ms_far_min(const int32_t (&x)[kMsMax], int32_
 // are masked on load, so the relaxation itself does not ask.  R-MAT 24, 8
 // sources: 1.69 G edge visits in 17 rounds and 17.3 ms in the plain near-far
 // order, 0.60 to 0.88 G in 50 to 80 and 10.6 to 14.6 ms in this one (R-MAT 22
-// 4.5 -> 3.1 to 4.2 ms).  It is bound by the rows' probes: 32 bytes of 537 MB each.  Measured and left out:
-// a bit per vertex whose slots are all settled, tested before a heavy edge's
-// row (11.0 ms: the slots settle at different times), 3 or 2 CTAs per SM
-// instead of 4 (11.7, 14.4 ms), one edge a lane (11.3 ms), the passes as
-// functions of their own (10.9 ms).
+// 4.5 -> 3.0 to 4.2 ms).  It is bound by the latency of the rows' probes, 32
+// bytes of 537 MB each (R-MAT 22, 134 MB: 4.3 GB of DRAM and 645 M L2 sectors in
+// 3.0 ms, a fifth of either's rate; warps wait at barriers and for loads).
+// Measured and left out: a bit per vertex whose slots are all settled, tested
+// before a heavy edge's row (11.0 ms: the slots settle at different times), 3
+// or 2 CTAs per SM instead of 4 (11.7, 14.4 ms), one edge a lane (11.3 ms), the
+// passes as functions of their own (10.9 ms).
 // A source row as it is relaxed: slots at or above their threshold have no candidate.
 __device__ __forceinline__ void ml_load_source(const int32_t *row, int32_t (&x)[kMsMax], bool fresh) {
     ms_load_row(row, x, fresh);

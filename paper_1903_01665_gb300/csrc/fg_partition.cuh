@@ -16,6 +16,10 @@
 // that the few vertices that hold most edges of a skewed graph neither
 // unbalance the work nor contend for a global counter.  The order of edges
 // within a vertex is that of the atomics.
+// R-MAT 22, with the weights: histogram 0.14 ms, pass 1 0.61 (1.47 GB of DRAM,
+// 2.4 TB/s; a third of the stalls are shared memory's), counts 0.16, pass 2 1.09
+// (1.29 GB; the warps wait for the random read of the renumbering, an edge
+// each: 0.60 without one); pass 1 and 2 without the weights 0.45 and 0.57.
 #pragma once
 
 #include <algorithm>
