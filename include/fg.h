@@ -352,7 +352,7 @@ fg_status fg_run(const fg_graph *g, fg_algo algo, int32_t src, int32_t *out, fg_
  * all sources go first, each source below its own threshold, then the heavy
  * ones once: from 2^20 vertices on where at most two fifths of the edges are
  * light, from 2^24 in any case, and with a width (delta) of the caller's (in a
- * batch, whose teams are smaller, from 2^14 instead of 2^20).
+ * batch, whose teams are smaller, from 2^16 instead of 2^20).
  *
  * Options: stream, max_rounds (0 = n + 2 for BFS and CC, 2 k n + 2 for
  * SSSP, whose epochs add rounds, 8 k n + 64 on split rows, and with a cap

@@ -310,9 +310,10 @@ int32_t ms_default_rounds(int32_t n, int k, bool near_far, bool light) {
 // 0.77 to 1.64 of it at scales 20 to 23, more than it at 19 of 24 points, 0.75 to 1.04
 // at 24.  A width of the caller's is the light-heavy order's.  In a batch a
 // team is a part of the device: its barriers cost less and the edges more, and
-// the order pays from 2^14 vertices on (12 graphs of 2^10 to 2^20 vertices, 96
-// queries: 7.9 ms, from 2^20 on 10.4; 12 of 2^13 to 2^18 4.2 and 5.8).
-constexpr int32_t kMultiLightMin = 1 << 20, kMultiLightBatch = 1 << 14, kMultiLightAny = 1 << 24;
+// the order pays from 2^16 vertices on (12 graphs of 2^10 to 2^20 vertices, 96
+// queries: 7.9 ms, from 2^20 on 10.4; 12 of 2^13 to 2^18 4.2 and 5.8).  From 2^14
+// on, batches of small graphs lose 1 to 2 % to the launch of its own.
+constexpr int32_t kMultiLightMin = 1 << 20, kMultiLightBatch = 1 << 16, kMultiLightAny = 1 << 24;
 constexpr double kMultiLightShare = 0.4;
 int32_t ms_light_width(const fg_graph *G, Algo algo, int k, int32_t delta, int32_t max_rounds, bool batch) {
     const bool pays = delta > 0 || G->g.n >= kMultiLightAny ||

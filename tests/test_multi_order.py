@@ -11,8 +11,8 @@ from tests.gpu_util import as_numpy, graph_handle, make_out, run
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("scale, weights, light", [(10, "uniform", False), (13, "uniform", False),
-                                                   (14, "uniform", True), (14, "two values", False),
+@pytest.mark.parametrize("scale, weights, light", [(10, "uniform", False), (15, "uniform", False),
+                                                   (16, "uniform", True), (16, "two values", False),
                                                    (20, "uniform", True), (20, "two values", False)])
 def test_order(scale, weights, light):
     g = gg.rmat(scale, seed=3)
