@@ -58,10 +58,10 @@ ALGO_NAMES = ["sssp", "bfs", "cc"]
 # at capture time).
 NCU_TRAFFIC: dict = {
     # profiles/sssp_rmat22_traffic.md: one launch each, first seeded source, R-MAT 22 (renumbered)
-    "fixpoint_kernel<sssp,vertex_sync>": {"bytes_per_launch": 3287055360 + 114013440, "src_sha": "8838b6b616d8089c"},
-    "fixpoint_kernel<sssp,edge_sync>": {"bytes_per_launch": 4751374592 + 76789760, "src_sha": "8838b6b616d8089c"},
-    "fixpoint_kernel<sssp,vertex_async>": {"bytes_per_launch": 2479128064 + 43311616, "src_sha": "8838b6b616d8089c"},
-    "fixpoint_kernel<sssp,edge_async>": {"bytes_per_launch": 4150399488 + 93541888, "src_sha": "8838b6b616d8089c"},
+    "fixpoint_kernel<sssp,vertex_sync>": {"bytes_per_launch": 3285663488 + 113620992, "src_sha": "4185640a9447bc30"},
+    "fixpoint_kernel<sssp,edge_sync>": {"bytes_per_launch": 4751988736 + 76744704, "src_sha": "4185640a9447bc30"},
+    "fixpoint_kernel<sssp,vertex_async>": {"bytes_per_launch": 2417305856 + 42260480, "src_sha": "4185640a9447bc30"},
+    "fixpoint_kernel<sssp,edge_async>": {"bytes_per_launch": 3598629120 + 89779968, "src_sha": "4185640a9447bc30"},
 }
 
 
@@ -69,8 +69,8 @@ NCU_TRAFFIC: dict = {
 # state), same validity rule
 NCU_SWEEP_DRAM: dict = {
     # profiles/sweep_rmat22.md: the sweep roofline state on R-MAT 22 (renumbered), one launch each
-    "vertex_sync": {"bytes": 586489088 + 3308800, "src_sha": "8838b6b616d8089c"},
-    "edge_sync": {"bytes": 829719040 + 4009728, "src_sha": "8838b6b616d8089c"},
+    "vertex_sync": {"bytes": 586781952 + 3275008, "src_sha": "4185640a9447bc30"},
+    "edge_sync": {"bytes": 829747968 + 3731456, "src_sha": "4185640a9447bc30"},
 }
 
 KERNEL_SOURCES = ("fg_internal.cuh", "fg_device.cuh", "fg_light.cuh", "fg_fixpoint.cu")
